@@ -50,6 +50,7 @@ struct fft_plan_s {
   int* status = nullptr;   // set by kernels whose bounded waits give up
   void* work = nullptr;    // cf[spec.work_elems]
   PassLaunch launches[kMaxPasses];  // whole-batch launches, device pointers filled
+  JoinedLaunch joined;              // both passes of a two-pass plan as one launch
   // lazily created resources of fft_execute_host
   cudaStream_t s_h2d = nullptr, s_k = nullptr, s_d2h = nullptr;
   cudaEvent_t ev_start = nullptr, ev_h2d = nullptr, ev_k = nullptr, ev_end = nullptr;
@@ -117,14 +118,16 @@ fft_status_t build_plan(fft_plan_t* out, const int64_t* n, int dims, int64_t bat
   p->caps = caps;
   p->spec = spec;
   cudaError_t e;
-  e = cudaMalloc(&p->tables, (size_t)spec.table_elems * 8 + 16);
+  // after the tables: the status word, then the joined launch's counters
+  const size_t words = 16 + (spec.joined ? 4 * (size_t)(2 + 2 * spec.join_ring) : 0);
+  e = cudaMalloc(&p->tables, (size_t)spec.table_elems * 8 + words);
   if (e != cudaSuccess) {
     delete p;
     cudaGetLastError();
     return fail(FFT_ERR_OUT_OF_MEMORY, "twiddle tables: %s", cudaGetErrorString(e));
   }
   p->status = reinterpret_cast<int*>(static_cast<char*>(p->tables) + (size_t)spec.table_elems * 8);
-  e = cudaMemset(p->status, 0, 16);
+  e = cudaMemset(p->status, 0, words);
   if (e != cudaSuccess) {
     cudaFree(p->tables);
     delete p;
@@ -146,6 +149,9 @@ fft_status_t build_plan(fft_plan_t* out, const int64_t* n, int dims, int64_t bat
   if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   if (e == cudaSuccess)
     e = bind_launches(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status, p->launches);
+  if (e == cudaSuccess && spec.joined)
+    e = bind_joined(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status,
+                    reinterpret_cast<unsigned*>(p->status + 4), &p->joined);
   if (e != cudaSuccess) {
     fft_plan_destroy(p);
     return cuda_fail(e, "twiddle generation");
@@ -196,7 +202,7 @@ fft_status_t fft_execute(fft_plan_t plan, const void* in, void* out, void* strea
     return fail(FFT_ERR_BAD_PLAN, "plan was created on device %d, current device is %d",
                 plan->device, dev);
   e = enqueue_passes(plan->spec, plan->launches, in, out, plan->work, 0, plan->spec.batch,
-                     static_cast<cudaStream_t>(stream));
+                     static_cast<cudaStream_t>(stream), -1, &plan->joined);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return FFT_OK;
 }
@@ -253,7 +259,8 @@ fft_status_t fft_execute_host(fft_plan_t plan, const void* host_in, void* host_o
     cudaStreamWaitEvent(plan->s_k, plan->ev_h2d, 0);
     // the chunks run one after the other on s_k, so each reuses the workspace
     // from its start
-    e = enqueue_passes(s, plan->launches, di + off, dout + off, wk, b0, nb, plan->s_k);
+    e = enqueue_passes(s, plan->launches, di + off, dout + off, wk, b0, nb, plan->s_k, -1,
+                       &plan->joined);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     cudaEventRecord(plan->ev_k, plan->s_k);
     cudaStreamWaitEvent(plan->s_d2h, plan->ev_k, 0);
@@ -295,7 +302,7 @@ fft_status_t fft_execute_graph(fft_plan_t plan, const void* in, void* out, void*
     e = cudaStreamBeginCapture(plan->s_capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "begin capture");
     cudaError_t le = enqueue_passes(plan->spec, plan->launches, in, out, plan->work, 0,
-                                    plan->spec.batch, plan->s_capture);
+                                    plan->spec.batch, plan->s_capture, -1, &plan->joined);
     e = cudaStreamEndCapture(plan->s_capture, &graph);
     if (le != cudaSuccess || e != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
@@ -359,7 +366,7 @@ fft_status_t fft_plan_workspace_bytes(fft_plan_t plan, size_t* bytes) {
 fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches) {
   if (!plan_ok(plan)) return fail(FFT_ERR_BAD_PLAN, "null or destroyed plan");
   if (!launches) return fail(FFT_ERR_INVALID_ARG, "launches is null");
-  *launches = plan->spec.batch == 0 ? 0 : (int)plan->spec.passes.size();
+  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined ? 1 : (int)plan->spec.passes.size();
   return FFT_OK;
 }
 

@@ -84,6 +84,20 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
   return cudaSuccess;
 }
 
+cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
+                        unsigned* counters, JoinedLaunch* j) {
+  const int logn = (int)(s.passes[0].logL + s.passes[1].logL);
+  cudaError_t e = prepare_joined(logn, s.direction == FFT_INVERSE, caps.sm_count, j);
+  if (e != cudaSuccess) return e;
+  j->d.tw1 = tables + s.join_tw1;
+  j->d.tw2 = tables + s.join_tw2;
+  j->d.o.lag = s.join_lag;
+  j->d.o.ring = s.join_ring;
+  j->d.ctr = counters;
+  j->d.status = status;
+  return cudaSuccess;
+}
+
 cudaError_t enqueue_tables(const PlanSpec& s, cf* tables, cudaStream_t st) {
   for (const TwSegment& t : s.tables) {
     cudaError_t e = launch_twiddle_gen(tables + t.off, t.count, t.den, t.mode, t.r, t.mult, st);
@@ -94,15 +108,15 @@ cudaError_t enqueue_tables(const PlanSpec& s, cf* tables, cudaStream_t st) {
 
 static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, const void* in,
                                  void* out, void* work, int64_t b0, int64_t nb, cudaStream_t st,
-                                 int64_t work2_off);
+                                 int64_t work2_off, const JoinedLaunch* joined);
 
 cudaError_t enqueue_passes(const PlanSpec& s, const PassLaunch* launches, const void* in,
                            void* out, void* work, int64_t b0, int64_t nb, cudaStream_t st,
-                           int64_t work2_off) {
+                           int64_t work2_off, const JoinedLaunch* joined) {
   if (work2_off < 0) work2_off = s.work2_off;
   if (nb <= 0) return cudaSuccess;
   if (s.chunk_batch <= 0 || nb <= s.chunk_batch)
-    return enqueue_range(s, launches, in, out, work, b0, nb, st, work2_off);
+    return enqueue_range(s, launches, in, out, work, b0, nb, st, work2_off, joined);
   // sub-batches in stream order, each reusing the workspace from its start
   const int64_t E = s.dims == 1 ? s.n[0] : s.n[0] * s.n[1];
   const int64_t eb = elem_bytes(s.precision);
@@ -110,7 +124,7 @@ cudaError_t enqueue_passes(const PlanSpec& s, const PassLaunch* launches, const 
     const int64_t n = std::min(s.chunk_batch, nb - c);
     cudaError_t e = enqueue_range(s, launches, static_cast<const char*>(in) + c * E * eb,
                                   static_cast<char*>(out) + c * E * eb, work, b0 + c, n, st,
-                                  work2_off);
+                                  work2_off, joined);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -118,9 +132,16 @@ cudaError_t enqueue_passes(const PlanSpec& s, const PassLaunch* launches, const 
 
 static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, const void* in,
                                  void* out, void* work, int64_t b0, int64_t nb, cudaStream_t st,
-                                 int64_t work2_off) {
+                                 int64_t work2_off, const JoinedLaunch* joined) {
   if (nb <= 0) return cudaSuccess;
   const int64_t E = s.dims == 1 ? s.n[0] : s.n[0] * s.n[1];
+  if (joined && joined->fn && work) {
+    // the output of one transform is written while the input of a later one is
+    // still read: in place or apart, not partly overlapping
+    const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out, bytes = (uintptr_t)(nb * E) * 8;
+    if (a == b || a + bytes <= b || b + bytes <= a)
+      return launch_joined(*joined, nb, in, out, work, st);
+  }
   // the second workspace buffer of six-step plans
   void* work2 = work ? static_cast<char*>(work) + work2_off * elem_bytes(s.precision) : nullptr;
   auto buf = [&](int b) -> void* {

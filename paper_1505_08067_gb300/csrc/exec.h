@@ -25,8 +25,16 @@ cudaError_t enqueue_tables(const PlanSpec& s, cf* tables, cudaStream_t st);
 // work2_off: offset (elements) of a six-step plan's second workspace buffer
 // when the workspace was sized for fewer transforms than the plan's (a
 // server job's own workspace); -1 = the plan's.
+// joined: the launch that runs both passes of a two-pass plan at once, for a
+// caller that owns its counters as it owns `work` (no other execution uses
+// either meanwhile); null = one launch per pass.
 cudaError_t enqueue_passes(const PlanSpec& s, const PassLaunch* launches, const void* in,
                            void* out, void* work, int64_t b0, int64_t nb, cudaStream_t st,
-                           int64_t work2_off = -1);
+                           int64_t work2_off = -1, const JoinedLaunch* joined = nullptr);
+
+// Fills `j` for a plan whose passes run as one launch (PlanSpec::joined):
+// `counters` = device words, 2 + 2 * join_ring of them, all zero.
+cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
+                        unsigned* counters, JoinedLaunch* j);
 
 }  // namespace gbfft

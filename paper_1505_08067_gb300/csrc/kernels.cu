@@ -124,22 +124,17 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// Tensor map for the column tiles of pass `d` over buffer `p` with strides
-// `st` (d.in or d.out): rows of st.e complex64 elements, boxes of G columns x
-// `box_rows` rows.  False when the layout does not allow it (cols_map_rows),
-// `p` is not 16-byte aligned, or the encoder refuses.
-static bool encode_cols_map(const PassDesc& d, const Strides& st, const void* p, int box_rows,
-                            unsigned char (&map)[128]) {
-  int64_t rows = 0;
-  if (!cols_map_rows(d, st, rows) || ((uintptr_t)p & 15)) return false;
+bool encode_rows_map(const void* p, int64_t cols, int64_t rows, int box_cols, int box_rows,
+                     unsigned char (&map)[128]) {
+  if ((uintptr_t)p & 15) return false;
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
-  static_assert(sizeof(CUtensorMap) == sizeof(map), "tensor map size");
-  const cuuint64_t dims[2] = {(cuuint64_t)st.e, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)st.e * 8};
-  const cuuint32_t box[2] = {(cuuint32_t)d.G, (cuuint32_t)box_rows};
-  const cuuint32_t elem_strides[2] = {1, 1};
   CUtensorMap m;
+  static_assert(sizeof(CUtensorMap) == sizeof(map), "tensor map size");
+  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)cols * 8};
+  const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+  const cuuint32_t elem_strides[2] = {1, 1};
   if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void*>(p), dims, strides, box,
           elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -148,24 +143,21 @@ static bool encode_cols_map(const PassDesc& d, const Strides& st, const void* p,
   return true;
 }
 
+// Tensor map for the column tiles of pass `d` over buffer `p` with strides
+// `st` (d.in or d.out): rows of st.e complex64 elements, boxes of G columns x
+// `box_rows` rows.  False when the layout does not allow it (cols_map_rows),
+// `p` is not 16-byte aligned, or the encoder refuses.
+static bool encode_cols_map(const PassDesc& d, const Strides& st, const void* p, int box_rows,
+                            unsigned char (&map)[128]) {
+  int64_t rows = 0;
+  return cols_map_rows(d, st, rows) && encode_rows_map(p, st.e, rows, d.G, box_rows, map);
+}
+
 // Tensor map of the filter frame of a convolution over column tiles
 // (cols_filter_staged): dims {in.e, L}, boxes of G columns x min(L, 256) rows.
 static bool encode_filter_map(PassDesc& d) {
   const int L = 1 << d.logL;
-  if (!cols_filter_staged(d) || ((uintptr_t)d.h & 15)) return false;
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)d.in.e, (cuuint64_t)L};
-  const cuuint64_t strides[1] = {(cuuint64_t)d.in.e * 8};
-  const cuuint32_t box[2] = {(cuuint32_t)d.G, (cuuint32_t)(L < 256 ? L : 256)};
-  const cuuint32_t elem_strides[2] = {1, 1};
-  CUtensorMap m;
-  if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<cf*>(d.h), dims, strides, box,
-          elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return false;
-  memcpy(d.tmap_h, &m, sizeof(m));
-  return true;
+  return cols_filter_staged(d) && encode_rows_map(d.h, d.in.e, L, d.G, L < 256 ? L : 256, d.tmap_h);
 }
 
 bool encode_cols_maps(PassDesc& d, bool map_in, bool map_out, const void* in, void* out) {

@@ -4,8 +4,38 @@
 #include <stddef.h>
 
 #include "fft_core.h"
+#include "fft_join.h"
 
 namespace gbfft {
+
+// The joined two-pass kernel (joined.cuh).
+struct JoinDesc {
+  const cf* tw1;  // w_{N1}^j, w_{N2}^j
+  const cf* tw2;
+  JoinOrder o;
+  unsigned* ctr;  // 2 + 2 ring counters, zero between launches
+  int* status;
+  // when `mapped`, a tensor map of the input viewed as rows of N2 complex64
+  // elements in boxes of G1 columns: first-pass tiles are prefetched into L2
+  int mapped;
+  alignas(64) unsigned char tmap_in[128];
+};
+struct JoinedLaunch {
+  const void* fn = nullptr;  // null: the plan's passes run as launches of their own
+  int max_grid = 0;          // resident blocks
+  int block = 0;
+  size_t smem = 0;
+  int n1 = 0, n2 = 0, g1 = 0, box_rows = 0;
+  JoinDesc d{};
+};
+// Kernel for N = 2^logn, its opt-in shared memory and resident blocks.
+cudaError_t prepare_joined(int logn, bool inverse, int sm_count, JoinedLaunch* j);
+cudaError_t launch_joined(const JoinedLaunch& j, int64_t nb, const void* in, void* out, void* work,
+                          cudaStream_t st);
+// Tensor map (128 bytes) over `rows` rows of `cols` complex64 elements at `p`,
+// boxes of box_cols x box_rows; false if `p` or the driver does not allow it.
+bool encode_rows_map(const void* p, int64_t cols, int64_t rows, int box_cols, int box_rows,
+                     unsigned char (&map)[128]);
 
 // Job table of a coalesced launch (see stockham_grouped): up to kMaxGroup jobs
 // of one contiguous single-pass shape, each with its own buffers.

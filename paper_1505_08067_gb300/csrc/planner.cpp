@@ -207,6 +207,21 @@ static PassSpec contiguous_pass(int logL, int64_t batch, int64_t units_per_batch
   return p;
 }
 
+// Does a two-pass plan of `batch` transforms per sub-batch run its passes as
+// one launch, and in what order (fft_join.h)?
+static void plan_joined(PlanSpec& s, int logN, int64_t batch, const Caps& caps) {
+  if (logN < kJoinMinLog || logN > kJoinMaxLog) return;
+  if (batch << logN < kJoinMinElems) return;
+  // ticks of the lag: 2.5 times the tiles in work at once (join_blocks_log)
+  const int tl = join_tile_log(logN);
+  const int64_t tiles = int64_t(1) << (logN - tl);  // per transform and pass
+  const int64_t resident = (int64_t)caps.sm_count << join_blocks_log(tl);
+  const int64_t lag = std::max<int64_t>(1, (5 * resident + 4 * tiles - 1) / (4 * tiles));
+  s.joined = true;
+  s.join_lag = (int)std::min(lag, batch);
+  s.join_ring = (int)std::min(2 * lag, batch);
+}
+
 void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direction,
                int precision, const fft_plan_options_t* opt, const Caps& caps,
                const ConvSpec* conv) {
@@ -470,6 +485,9 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       const int64_t chunk = two_pass_chunk(N);
       s.chunk_batch = batch > chunk ? chunk : 0;
       s.work_elems = std::min(batch, chunk) * N;
+      const bool defaults = !o.radix && !o.schedule && o.max_block_log2 <= 0 && !o.tile &&
+                            !o.generic && !o.variant && !o.epilogue && !o.split_log2;
+      if (defaults) plan_joined(s, logN, std::min(batch, chunk), caps);
     }
   } else {
     const int64_t rows = n[0], cols = n[1];
@@ -549,6 +567,16 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       off = (off + 1) & ~int64_t(1);
     }
   }
+  if (s.joined) {
+    const int logN = ilog2(s.n[0]);
+    const int64_t N1 = int64_t(1) << (logN / 2), N2 = s.n[0] / N1;
+    s.join_tw1 = off;
+    s.tables.push_back(TwSegment{off, N1, N1, 1, 1, 1});
+    off += N1;
+    s.join_tw2 = off;
+    s.tables.push_back(TwSegment{off, N2, N2, 1, 1, 1});
+    off += N2;
+  }
   s.table_elems = off;
   for (auto& p : s.passes) {
     if (p.kind == PASS_FFT) {
@@ -605,7 +633,7 @@ std::string describe(const PlanSpec& s) {
     << ",\"precision\":" << s.precision << ",\"max_block_log2\":" << s.max_block_log2
     << ",\"generic\":" << (s.generic_only ? 1 : 0) << ",\"conv\":" << (s.conv ? 1 : 0)
     << ",\"workspace_bytes\":" << s.work_elems * 8 << ",\"table_elems\":" << s.table_elems
-    << ",\"chunk_batch\":" << s.chunk_batch
+    << ",\"chunk_batch\":" << s.chunk_batch << ",\"joined\":" << (s.joined ? 1 : 0)
     << ",\"passes\":[";
   for (size_t i = 0; i < s.passes.size(); ++i) {
     const PassSpec& p = s.passes[i];

@@ -1,0 +1,192 @@
+// Test infrastructure: replays the joined two-pass kernel (fft_join.h) on the
+// CPU, tile by tile in ticket order and thread by thread, with every access
+// checked: global and workspace offsets inside their buffers, shared slots
+// inside the tile and written in the phase before they are read, no slot
+// written twice in a phase, every output written once, workspace elements read
+// only after the transform's own first pass wrote them.  Also checks the tile
+// order: what a ticket waits for is complete once the tickets before it are.
+// It never stands in for the GPU.
+#include <math.h>
+#include <stdint.h>
+#include <stdio.h>
+#include <string.h>
+
+#include <string>
+#include <vector>
+
+#include "fft_join.h"
+
+using namespace gbfft;
+
+namespace {
+
+struct Ctx {
+  const cf *in, *tw1, *tw2;
+  cf *out, *work;
+  int64_t in_len, out_len, work_len;
+  std::vector<uint8_t> out_hits;
+  std::vector<int64_t> work_owner;  // transform whose first pass wrote the element
+  int64_t b;                        // transform being replayed
+  int tw1_len, tw2_len;
+  const cf* sm;
+  int smem_len, conflicts;
+  std::vector<int64_t> phase_of;
+  int64_t phase, errors;
+  std::string first;
+};
+Ctx g;
+
+void err(const char* what, int64_t i) {
+  if (g.errors++ == 0) {
+    char b[160];
+    snprintf(b, sizeof b, "%s (index %lld)", what, (long long)i);
+    g.first = b;
+  }
+}
+
+struct CheckMem {
+  static cf ldin(const cf* p, int off) {
+    const int64_t i = p - g.in + off;
+    if (i < 0 || i >= g.in_len) { err("input load out of bounds", i); return mk(0, 0); }
+    return g.in[i];
+  }
+  static cf ldw(const cf* p, int off) {
+    const int64_t i = p - g.work + off;
+    if (i < 0 || i >= g.work_len) { err("workspace load out of bounds", i); return mk(0, 0); }
+    if (g.work_owner[i] != g.b) err("workspace element of another transform", i);
+    return g.work[i];
+  }
+  static void stw(cf* p, int off, cf v) {
+    const int64_t i = p - g.work + off;
+    if (i < 0 || i >= g.work_len) { err("workspace store out of bounds", i); return; }
+    if (g.work_owner[i] == g.b) err("workspace element written twice", i);
+    g.work_owner[i] = g.b;
+    g.work[i] = v;
+  }
+  static void stout(cf* p, int off, cf v) {
+    const int64_t i = p - g.out + off;
+    if (i < 0 || i >= g.out_len) { err("output store out of bounds", i); return; }
+    if (g.out_hits[i]++) err("output element written twice", i);
+    g.out[i] = v;
+  }
+  static int at(const cf* s, int i) {
+    i += (int)(s - g.sm);
+    if (i < 0 || i >= g.smem_len) { err("shared slot out of bounds", i); return 0; }
+    return i;
+  }
+  static cf lds(const cf* s, int i) {
+    i = at(s, i);
+    if (g.phase_of[i] != g.phase) err("shared slot read that the last phase did not write", i);
+    return g.sm[i];
+  }
+  static void sts(cf* s, int i, cf v) {
+    i = at(s, i);
+    if (g.phase_of[i] == g.phase) err("shared slot written twice in a phase", i);
+    g.phase_of[i] = g.phase;
+    const_cast<cf*>(g.sm)[i] = v;
+  }
+  static cf ldtw(const cf* p) {
+    const bool one = p >= g.tw1 && p < g.tw1 + g.tw1_len, two = p >= g.tw2 && p < g.tw2 + g.tw2_len;
+    if (!one && !two) { err("twiddle load out of bounds", 0); return mk(1, 0); }
+    return *p;
+  }
+  static cf rotor(int64_t m, int logN) {
+    if (m < 0 || m >= int64_t(1) << logN) err("rotor exponent out of range", m);
+    const double a = -2.0 * M_PI * (double)m / (double)(int64_t(1) << logN);
+    return mk((float)cos(a), (float)sin(a));
+  }
+};
+
+std::vector<cf> roots(int n) {
+  std::vector<cf> t(n);
+  for (int j = 0; j < n; ++j) t[j] = mk((float)cos(2 * M_PI * j / n), (float)-sin(2 * M_PI * j / n));
+  return t;
+}
+
+template <class SH, bool ROWL, class First, class Store>
+void tile(cf* sm, cf* st, const cf* tw, int col0, int logN, First first, Store store) {
+  using B = JoinBody<SH, ROWL, CheckMem>;
+  std::vector<cf> regs((size_t)SH::kThreads * kJoinR);
+  auto v = [&](int t) -> cf (&)[kJoinR] { return *reinterpret_cast<cf(*)[kJoinR]>(&regs[(size_t)t * kJoinR]); };
+  auto each = [&](auto f) { for (int t = 0; t < SH::kThreads; ++t) f(v(t), t); };
+  ++g.phase;
+  if (ROWL)
+    for (int lane = 0; lane < 32; ++lane) B::steps(st, col0, logN, lane);
+  each([&](cf (&r)[kJoinR], int t) { first(r, t); B::dft0(r); B::template put<0>(r, sm, t); });
+  each([&](cf (&r)[kJoinR], int t) {
+    B::template get<SH::kLast>(r, sm, t);
+    B::template turn<SH::kLast, ROWL>(r, tw, col0, logN, t);  // pass 1 carries the four-step twiddle
+    store(r, t);
+  });
+}
+
+template <int LOGN, bool INV>
+int64_t run(int64_t nb, int lag, int ring, const cf* in, cf* out) {
+  using PR = JoinPair<LOGN>;
+  using B1 = JoinBody<typename PR::P1, true, CheckMem>;
+  using B2 = JoinBody<typename PR::P2, false, CheckMem>;
+  g = Ctx{};
+  std::vector<cf> t1 = roots(PR::kN1), t2 = roots(PR::kN2), work((size_t)ring * PR::kN),
+                  sm(PR::kTileSlots + PR::kSteps);
+  g.in = in;
+  g.out = out;
+  g.in_len = g.out_len = nb * PR::kN;
+  g.work = work.data();
+  g.work_len = (int64_t)work.size();
+  g.out_hits.assign(g.out_len, 0);
+  g.work_owner.assign(g.work_len, -1);
+  g.tw1 = t1.data();
+  g.tw2 = t2.data();
+  g.tw1_len = PR::kN1;
+  g.tw2_len = PR::kN2;
+  g.sm = sm.data();
+  g.smem_len = (int)sm.size();
+  g.phase_of.assign(sm.size(), -1);
+  cf* st = sm.data() + PR::kTileSlots;
+  static_assert(join_tile_log(LOGN) == PR::kTileLog, "the planner's tile");
+  JoinOrder o{nb, LOGN - PR::kTileLog, lag < nb ? lag : (int)nb, ring};
+  std::vector<uint32_t> done(2 * ring, 0);
+  for (int64_t t = 0; t < join_tickets(o); ++t) {
+    const JoinTicket k = join_ticket(o, t);
+    const JoinDep dep = join_dep(o, k);
+    if (k.b < 0 || k.b >= nb || k.tile < 0 || k.tile >= PR::kTiles) { err("ticket out of range", t); break; }
+    if (done[dep.pass * ring + dep.slot] < dep.count) err("a ticket waits for a later one", t);
+    const int slot = (int)(k.b % ring);
+    cf* w = work.data() + (int64_t)slot * PR::kN;
+    g.b = k.b;
+    if (k.pass == 0) {
+      const int col0 = k.tile * PR::kG1;
+      tile<typename PR::P1, true>(
+          sm.data(), st, g.tw1, col0, LOGN,
+          [&](cf (&v)[kJoinR], int i) { B1::template first<INV, false>(v, in + k.b * PR::kN + col0, PR::kN2, i); },
+          [&](cf (&v)[kJoinR], int i) { B1::template store_block<PR::kG2>(v, w + col0 * PR::kG2, st, PR::kN2, i); });
+    } else {
+      tile<typename PR::P2, false>(
+          sm.data(), st, g.tw2, 0, 0,
+          [&](cf (&v)[kJoinR], int i) { B2::template first<false, true>(v, w + k.tile * PR::kTile, PR::kG2, i); },
+          [&](cf (&v)[kJoinR], int i) { B2::template store_cols<INV>(v, out + k.b * PR::kN + k.tile * PR::kG2, PR::kN1, i); });
+    }
+    ++done[k.pass * ring + slot];
+  }
+  for (int64_t i = 0; i < g.out_len; ++i)
+    if (g.out_hits[i] != 1) { err("output element not written exactly once", i); break; }
+  return g.errors;
+}
+
+}  // namespace
+
+extern "C" int64_t join_run(int logn, int64_t nb, int inverse, int lag, int ring, const float* in,
+                            float* out, char* msg, size_t len) {
+  const cf* x = reinterpret_cast<const cf*>(in);
+  cf* y = reinterpret_cast<cf*>(out);
+  int64_t e = -1;
+  switch (logn) {
+#define GB_RUN(L) \
+  case L: e = inverse ? run<L, true>(nb, lag, ring, x, y) : run<L, false>(nb, lag, ring, x, y); break;
+    GB_RUN(15) GB_RUN(16) GB_RUN(17) GB_RUN(18) GB_RUN(19) GB_RUN(20)
+#undef GB_RUN
+    default: break;
+  }
+  snprintf(msg, len, "%s", g.first.c_str());
+  return e;
+}

@@ -1,0 +1,79 @@
+"""The joined two-pass kernel (both passes of 2^15 .. 2^20 in one launch) at the
+edges of its range: the smallest batches that take it, ragged batches whose ring
+of workspace slots wraps, in place, buffers that are only 8-byte aligned,
+repeated and overlapping-buffer calls, against the FP64 oracle."""
+import numpy as np
+import pytest
+
+from paper_1505_08067_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _check(oracle, y, x_np, idx, direction, logn):
+    ref = oracle.fft_select(x_np, idx, direction)
+    assert np.max(oracle.rel_l2(y[torch.from_numpy(idx).cuda()].cpu().numpy(), ref)) <= 1e-6 * logn
+
+
+@pytest.mark.parametrize("logn,batch", [(15, 64), (15, 391), (16, 193), (17, 16), (17, 75), (18, 8),
+                                        (18, 39), (19, 4), (19, 17), (20, 2), (20, 9)])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_joined(gb, oracle, logn, batch, direction):
+    n = 2 ** logn
+    x_np = synth.uniform(700 + logn, batch, n)
+    idx = np.unique([0, batch // 2, batch - 1])
+    buf = torch.empty(batch * n + 1, dtype=torch.complex64, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    with gb.Plan(n, batch, direction) as p:
+        assert p.describe()["joined"] == 1 and p.launch_count == 1
+        first = None
+        for shift in (0, 1):  # 16-byte and 8-byte aligned input
+            x = buf[shift:shift + batch * n].view(batch, n)
+            x.copy_(torch.from_numpy(x_np))
+            y = torch.empty(batch, n, dtype=torch.complex64, device="cuda")
+            p.execute(x, y)
+            first = y if first is None else first
+            assert torch.equal(first, y)  # the counters are clean after each launch
+        _check(oracle, first, x_np, idx, direction, logn)
+        p.execute(x, x)
+        gb.fft_plan_sync_status(p.handle, s)
+        assert torch.equal(first, x)
+
+
+@pytest.mark.parametrize("logn,batch", [(15, 63), (20, 1), (21, 2)])
+def test_not_joined(gb, logn, batch):
+    with gb.Plan(2 ** logn, batch) as p:
+        assert p.describe()["joined"] == 0 and p.launch_count == 2
+
+
+def test_partly_overlapping_buffers(gb, oracle):
+    """Output one transform after the input: the passes run apart, so that all
+    of the input is read before any output is written."""
+    logn, batch = 16, 40
+    n = 2 ** logn
+    x_np = synth.uniform(771, batch, n)
+    buf = torch.empty((batch + 1) * n, dtype=torch.complex64, device="cuda")
+    buf[:batch * n].copy_(torch.from_numpy(x_np).view(-1))
+    with gb.Plan(n, batch) as p:
+        assert p.describe()["joined"] == 1
+        p.execute(buf[:batch * n], buf[n:])
+        torch.cuda.synchronize()
+    _check(oracle, buf[n:].view(batch, n), x_np, np.array([0, 1, batch - 1]), -1, logn)
+
+
+def test_two_plans_on_two_streams(gb, oracle):
+    logn, batch = 17, 40
+    n = 2 ** logn
+    xs = [torch.from_numpy(synth.uniform(780 + i, batch, n)).cuda() for i in range(2)]
+    streams = [torch.cuda.Stream() for _ in xs]
+    torch.cuda.synchronize()
+    with gb.Plan(n, batch) as p, gb.Plan(n, batch) as q:
+        want = [p.execute(x) for x in xs]
+        torch.cuda.synchronize()
+        got = [torch.empty_like(x) for x in xs]
+        for _ in range(8):
+            for plan, x, y, s in zip((p, q), xs, got, streams):
+                plan.execute(x, y, stream=s)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
