@@ -220,8 +220,8 @@ GBFFT_API fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches);
  * TMA / cp.async staged kernel, used when the source is 16-byte aligned, else
  * the compile-time kernel of the shape), "compile_time", "generic",
  * "tensor_core" or "copy" -- with its persistent-grid size and L2-prefetch
- * flag; "joined": 1 when both passes of a two-pass plan run as one launch of
- * the joined kernel, 0 when each runs the kernel named for it) written to buf (NUL-terminated, truncated to len).  Returns
+ * flag; "joined": 1 when both passes of a two-pass or 2D plan run as one launch
+ * of a joined kernel, 0 when each runs the kernel named for it) written to buf (NUL-terminated, truncated to len).  Returns
  * FFT_ERR_INVALID_ARG if buf is too small for the whole text.
  */
 GBFFT_API fft_status_t fft_plan_describe(fft_plan_t plan, char* buf, size_t len);

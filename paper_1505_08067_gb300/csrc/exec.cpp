@@ -86,8 +86,10 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
 
 cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
                         unsigned* counters, JoinedLaunch* j) {
-  const int logn = (int)(s.passes[0].logL + s.passes[1].logL);
-  cudaError_t e = prepare_joined(logn, s.direction == FFT_INVERSE, caps.sm_count, j);
+  const int l0 = s.passes[0].logL, l1 = s.passes[1].logL;
+  const bool inv = s.direction == FFT_INVERSE;
+  const cudaError_t e = s.dims == 2 ? prepare_joined_frames(l1, l0, inv, caps.sm_count, j)
+                                    : prepare_joined(l0 + l1, inv, caps.sm_count, j);
   if (e != cudaSuccess) return e;
   j->d.tw1 = tables + s.join_tw1;
   j->d.tw2 = tables + s.join_tw2;
@@ -135,7 +137,7 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
                                  int64_t work2_off, const JoinedLaunch* joined) {
   if (nb <= 0) return cudaSuccess;
   const int64_t E = s.dims == 1 ? s.n[0] : s.n[0] * s.n[1];
-  if (joined && joined->fn && work) {
+  if (joined && joined->fn && (work || joined->frames)) {
     // the output of one transform is written while the input of a later one is
     // still read: in place or apart, not partly overlapping
     const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out, bytes = (uintptr_t)(nb * E) * 8;

@@ -1,15 +1,15 @@
-// Per-thread phases of the joined two-pass kernel (joined.cu): both passes of
-// a four-step transform (Sec. 3.3) as column passes over tiles of 8192
-// elements, 32 per thread.
+// Per-thread phases of the joined kernels (joined.cuh): the two passes of a
+// four-step transform (Sec. 3.3), or the row and column passes of 2D frames
+// (Sec. 3.1), over tiles of 4096 .. 16384 elements, 32 per thread.
 //
-// One exchange instead of two: a pass of 256 / 512 / 1024 points is two stages
+// One exchange instead of two: a pass of up to 1024 points is two stages
 // (16 x 16, 32 x 16, 32 x 32), so its tile crosses shared memory once, and one
-// stage fewer is twiddled.  (2048 points: 16 x 16 x 8.)  A stage's twiddles
+// stage fewer is twiddled (2048 .. 8192 points: three).  A stage's twiddles
 // w^{ik}, i < r, are products of at most log2 r table values w^{k 2^m}, each
 // FP64-generated and rounded once, which is closer to the exact value than the
 // powers of a single root, and costs as many multiplies.
 //
-// N = N1 N2, x[n1 N2 + n2], X[k2 N1 + k1]:
+// Four-step transforms.  N = N1 N2, x[n1 N2 + n2], X[k2 N1 + k1]:
 //   pass 1  a tile holds G1 = 8192 / N1 adjacent columns n2; the output is
 //           multiplied by w_N^{n2 k1} and written to the workspace in blocks of
 //           G2 = 8192 / N2 values k1: element (n2, k1) at
@@ -105,33 +105,48 @@ struct JoinShape {
   GB_HDC static constexpr int radix(int s) { return 1 << rlog(s); }
   GB_HDC static constexpr int ns(int s) { return s == 0 ? 1 : s == 1 ? 1 << RA : 1 << (RA + RB); }
   static constexpr int kLast = kNst - 1;
-  // Shared-memory layouts.  By column (ROWL = false): adjacent columns
-  // adjacent, G slots of padding after every 2^RA rows where G < 16.  By
-  // transform (ROWL = true): a padding slot after every 2^RA elements and a
-  // pitch of max(1, 16 / G) mod 16.  With the thread maps below the 16 lanes
-  // of a half warp (64-bit accesses) then always touch 16 distinct slots mod 16.
-  static constexpr int kColPad = kG < 16 ? kG : 0;
-  static constexpr int kPitch0 = kL + (kL >> RA);
-  static constexpr int kPitch = kPitch0 + (((kG < 16 ? 16 / kG : 1) - kPitch0) & 15);
-  static constexpr int kSlotsCol = kL * kG + (kL >> RA) * kColPad;
-  static constexpr int kSlotsRow = kG * kPitch;
 };
 
-// Which butterfly (transform c of the tile, butterfly jb) the index
-// u = q * 256 + thread id is: adjacent lanes along the columns, or 16 lanes along
-// jb and the columns next.
-enum { JMAP_COLS = 0, JMAP_BLOCK = 1 };
+// What a tile's pass is: the first of a four-step transform (columns in, blocks
+// of the workspace out), columns in and out, or contiguous rows in and out.
+enum { JOIN_FIRST = 0, JOIN_COLS = 1, JOIN_ROWS = 2 };
 
-// ROWL: the shared layout.  Mem: the memory policy (the device's, or the CPU
-// replay's): ldin / ldw (input, workspace), stw / stout, lds / sts, ldtw, rotor.
-template <class SH, bool ROWL, class Mem>
+// Mem: the memory policy (the device's, or the CPU replay's): ldin / ldw
+// (input, intermediate), stw / stout, lds / sts, ldtw, rotor.
+template <class SH, int KIND, class Mem>
 struct JoinBody {
-  static constexpr int G = SH::kG, L = SH::kL, R = kJoinR, T = SH::kThreads;
-  static constexpr int kSlots = ROWL ? SH::kSlotsRow : SH::kSlotsCol;
+  static constexpr int G = SH::kG, L = SH::kL, R = kJoinR, T = SH::kThreads, TILE = SH::kTile;
+  GB_HDC static constexpr int jbs(int s) { return L >> SH::rlog(s); }  // butterflies of stage s
 
-  template <int MAP>
+  // Shared-memory layouts.  Column passes: adjacent columns adjacent, G slots
+  // of padding after every 2^RA rows where G < 16.  The others: transform by
+  // transform, a padding slot after every 2^RA elements and a pitch mod 16 of
+  // 16 / G (first passes, whose loads put G lanes across the transforms) or of
+  // the lanes along a transform (rows).  The 16 lanes of a half warp (64-bit
+  // accesses) then touch 16 distinct slots mod 16 (rows of 32: two share one).
+  static constexpr int kColPad = G < 16 ? G : 0;
+  static constexpr int kMinJb = jbs(0) < jbs(SH::kLast) ? jbs(0) : jbs(SH::kLast);
+  static constexpr int kPitch0 = L + (L >> SH::kRA);
+  static constexpr int kPitchMod =
+      KIND == JOIN_ROWS ? (kMinJb < 16 ? kMinJb : 0) : (G < 16 ? 16 / G : 1);
+  static constexpr int kPitch = kPitch0 + ((kPitchMod - kPitch0) & 15);
+  static constexpr int kSlots =
+      KIND == JOIN_COLS ? L * G + (L >> SH::kRA) * kColPad : G * kPitch;
+  GB_HD static int slot(int pos, int c) {
+    if (KIND != JOIN_COLS) return c * kPitch + pos + (pos >> SH::kRA);
+    return pos * G + c + (pos >> SH::kRA) * kColPad;
+  }
+
+  // Which butterfly (transform c of the tile, butterfly jb) of stage S the index
+  // u = q T + thread id is: adjacent lanes across the columns where memory is
+  // read or written by columns, along jb for rows; the last stage of a first
+  // pass has 16 lanes along jb and the columns next.
+  template <int S>
   GB_HD static void coords(int u, int& c, int& jb) {
-    if (MAP == JMAP_COLS) {
+    if (KIND == JOIN_ROWS) {
+      jb = u % jbs(S);
+      c = u / jbs(S);
+    } else if (KIND == JOIN_COLS || S == 0) {
       c = u % G;
       jb = u / G;
     } else {
@@ -139,30 +154,60 @@ struct JoinBody {
       jb = (u & 15) | (u / (16 * G)) << 4;
     }
   }
-  GB_HD static int slot(int pos, int c) {
-    if (ROWL) return c * SH::kPitch + pos + (pos >> SH::kRA);
-    return pos * G + c + (pos >> SH::kRA) * SH::kColPad;
-  }
-  // Thread map of stage s: the loads' (columns) at first, the stores' at
-  // last; a middle stage's lanes follow the shared layout.
-  GB_HDC static constexpr int map_of(int s) {
-    return s == 0 || !ROWL ? JMAP_COLS : JMAP_BLOCK;
-  }
 
-  // Stage 0: element a of column c at base + a*e + c; WORK: from the workspace.
+  // Stage 0 of a column pass: element a of column c at base + a*e + c; WORK:
+  // from the workspace.
   template <bool INV, bool WORK>
   GB_HD static void first(cf (&v)[R], const cf* base, int e, int tid) {
     constexpr int RR = SH::radix(0), NB = R / RR;
 GB_UNROLL
     for (int q = 0; q < NB; ++q) {
       int c, jb;
-      coords<JMAP_COLS>(q * T + tid, c, jb);
+      coords<0>(q * T + tid, c, jb);
       const cf* p = base + (int64_t)jb * e + c;
 GB_UNROLL
       for (int i = 0; i < RR; ++i) {
         const cf x = WORK ? Mem::ldw(p, i * (L / RR) * e) : Mem::ldin(p, i * (L / RR) * e);
         v[q * RR + i] = INV ? mk(x.y, x.x) : x;
       }
+    }
+  }
+  // Stage 0 of a row pass: the tile's first `valid` rows, consecutive at base;
+  // zeros for the rest.
+  template <bool INV>
+  GB_HD static void first_rows(cf (&v)[R], const cf* base, int64_t valid, int tid) {
+    constexpr int RR = SH::radix(0), NB = R / RR;
+GB_UNROLL
+    for (int q = 0; q < NB; ++q) {
+      int c, jb;
+      coords<0>(q * T + tid, c, jb);
+      const cf* p = base + c * L + jb;
+      const bool ok = c < valid;
+GB_UNROLL
+      for (int i = 0; i < RR; ++i) {
+        const cf x = ok ? Mem::ldin(p, i * (L / RR)) : mk(0.f, 0.f);
+        v[q * RR + i] = INV ? mk(x.y, x.x) : x;
+      }
+    }
+  }
+  // Column `col` of all frames of L rows of 2^lc elements: its first element.
+  GB_HD static int64_t frame_col(int64_t col, int lc) {
+    return ((col >> lc) << (SH::kLogL + lc)) + (col & ((int64_t(1) << lc) - 1));
+  }
+  // Stage 0 of a frame's column pass: columns col0 .. col0 + G - 1 of all the
+  // frames in buf, of which there are `cols`; zeros beyond.
+  GB_HD static void first_frame(cf (&v)[R], const cf* buf, int64_t col0, int64_t cols, int lc,
+                                int tid) {
+    constexpr int RR = SH::radix(0), NB = R / RR;
+GB_UNROLL
+    for (int q = 0; q < NB; ++q) {
+      int c, jb;
+      coords<0>(q * T + tid, c, jb);
+      const cf* p = buf + frame_col(col0 + c, lc) + (jb << lc);
+      const bool ok = col0 + c < cols;
+GB_UNROLL
+      for (int i = 0; i < RR; ++i)
+        v[q * RR + i] = ok ? Mem::ldw(p, (i * (L / RR)) << lc) : mk(0.f, 0.f);
     }
   }
   GB_HD static void dft0(cf (&v)[R]) {
@@ -178,7 +223,7 @@ GB_UNROLL
 GB_UNROLL
     for (int q = 0; q < NB; ++q) {
       int c, jb;
-      coords<map_of(S)>(q * T + tid, c, jb);
+      coords<S>(q * T + tid, c, jb);
       const int k = jb & (Ns - 1);
       const int base = (jb - k) * RR + k;
 GB_UNROLL
@@ -193,7 +238,7 @@ GB_UNROLL
 GB_UNROLL
     for (int q = 0; q < NB; ++q) {
       int c, jb;
-      coords<map_of(S)>(q * T + tid, c, jb);
+      coords<S>(q * T + tid, c, jb);
 GB_UNROLL
       for (int i = 0; i < RR; ++i) v[q * RR + i] = Mem::lds(sm, slot(jb + i * (L / RR), c));
     }
@@ -208,7 +253,7 @@ GB_UNROLL
 GB_UNROLL
     for (int q = 0; q < NB; ++q) {
       int c, jb;
-      coords<map_of(S)>(q * T + tid, c, jb);
+      coords<S>(q * T + tid, c, jb);
       const int k = (jb & (Ns - 1)) * (L / (Ns * RR));
       cf w[RR];
       if (TW4) {
@@ -229,8 +274,7 @@ GB_UNROLL
   }
 
   // The second factor of the four-step twiddle, w_N^{col Ns i} of the last
-  // stage, for every column of the tile: st[i * G + c].
-  // Computed by one warp.
+  // stage, for every column of the tile: st[i * G + c] (computed by one warp).
   static constexpr int kSteps = G * SH::radix(SH::kLast);
   GB_HD static void steps(cf* st, int col0, int logN, int lane) {
     for (int x = lane; x < kSteps; x += 32) {
@@ -248,7 +292,7 @@ GB_UNROLL
 GB_UNROLL
     for (int q = 0; q < NB; ++q) {
       int c, jb;
-      coords<map_of(S)>(q * T + tid, c, jb);
+      coords<S>(q * T + tid, c, jb);
       cf* p = wb + (jb / G2) * (cols * G2) + c * G2 + jb % G2;
 GB_UNROLL
       for (int i = 0; i < RR; ++i)
@@ -264,12 +308,44 @@ GB_UNROLL
 GB_UNROLL
     for (int q = 0; q < NB; ++q) {
       int c, jb;
-      coords<map_of(S)>(q * T + tid, c, jb);
+      coords<S>(q * T + tid, c, jb);
       cf* p = base + (int64_t)jb * e + c;
 GB_UNROLL
       for (int i = 0; i < RR; ++i) {
         const cf x = v[q * RR + i];
         Mem::stout(p, i * Ns * e, INV ? mk(x.y, x.x) : x);
+      }
+    }
+  }
+  // Last stage of a row pass / of a frame's column pass.
+  GB_HD static void store_rows(const cf (&v)[R], cf* base, int64_t valid, int tid) {
+    constexpr int S = SH::kLast, RR = SH::radix(S), NB = R / RR, Ns = SH::ns(S);
+GB_UNROLL
+    for (int q = 0; q < NB; ++q) {
+      int c, jb;
+      coords<S>(q * T + tid, c, jb);
+      cf* p = base + c * L + jb;
+      if (c < valid) {
+GB_UNROLL
+        for (int i = 0; i < RR; ++i) Mem::stw(p, i * Ns, v[q * RR + i]);
+      }
+    }
+  }
+  template <bool INV>
+  GB_HD static void store_frame(const cf (&v)[R], cf* buf, int64_t col0, int64_t cols, int lc,
+                                int tid) {
+    constexpr int S = SH::kLast, RR = SH::radix(S), NB = R / RR, Ns = SH::ns(S);
+GB_UNROLL
+    for (int q = 0; q < NB; ++q) {
+      int c, jb;
+      coords<S>(q * T + tid, c, jb);
+      cf* p = buf + frame_col(col0 + c, lc) + (jb << lc);
+      if (col0 + c < cols) {
+GB_UNROLL
+        for (int i = 0; i < RR; ++i) {
+          const cf x = v[q * RR + i];
+          Mem::stout(p, (i * Ns) << lc, INV ? mk(x.y, x.x) : x);
+        }
       }
     }
   }
@@ -286,15 +362,24 @@ struct JoinPairOf {
   static constexpr int kG1 = S1::kG, kG2 = S2::kG;
   static constexpr int kThreads = S1::kThreads, kTileLog = S1::kTileLog, kTile = S1::kTile;
   static constexpr int kTiles = kN / kTile;  // tiles of one transform, per pass
-  // shared-memory elements: the larger tile, then the first pass's steps
-  static constexpr int kSlots = S1::kSlotsRow > S2::kSlotsCol ? S1::kSlotsRow : S2::kSlotsCol;
-  static constexpr int kTileSlots = kSlots;
   static constexpr int kSteps = S1::kG << S1::rlog(S1::kLast);
 };
 template <int TL> using Join128 = JoinShape<TL, 7, 4, 3>;
 template <int TL> using Join256 = JoinShape<TL, 8, 4, 4>;
 template <int TL> using Join512 = JoinShape<TL, 9, 5, 4>;
 template <int TL> using Join1024 = JoinShape<TL, 10, 5, 5>;
+// Every length a row (2^4 .. 2^13) or column (2^4 .. 2^11) pass of frames has.
+template <int TL, int LOGL> struct JoinLen;
+template <int TL> struct JoinLen<TL, 4> { using S = JoinShape<TL, 4, 2, 2>; };
+template <int TL> struct JoinLen<TL, 5> { using S = JoinShape<TL, 5, 3, 2>; };
+template <int TL> struct JoinLen<TL, 6> { using S = JoinShape<TL, 6, 3, 3>; };
+template <int TL> struct JoinLen<TL, 7> { using S = Join128<TL>; };
+template <int TL> struct JoinLen<TL, 8> { using S = Join256<TL>; };
+template <int TL> struct JoinLen<TL, 9> { using S = Join512<TL>; };
+template <int TL> struct JoinLen<TL, 10> { using S = Join1024<TL>; };
+template <int TL> struct JoinLen<TL, 11> { using S = JoinShape<TL, 11, 4, 4, 3>; };
+template <int TL> struct JoinLen<TL, 12> { using S = JoinShape<TL, 12, 4, 4, 4>; };
+template <int TL> struct JoinLen<TL, 13> { using S = JoinShape<TL, 13, 5, 4, 4>; };
 template <int LOGN> struct JoinPair;
 template <> struct JoinPair<15> : JoinPairOf<Join128<12>, Join256<12>> {};
 template <> struct JoinPair<16> : JoinPairOf<Join256<12>, Join256<12>> {};
@@ -307,6 +392,11 @@ constexpr int kJoinMinLog = 15, kJoinMaxLog = 20;
 // elements in all).
 GB_HD constexpr int join_tile_log(int logn) { return logn <= 16 ? 12 : logn <= 19 ? 13 : 14; }
 GB_HD constexpr int join_blocks_log(int tile_log) { return 14 - tile_log; }
+// Frames: rows of 2^lc, columns of 2^lr.
+GB_HD constexpr bool join_frame(int lr, int lc) {
+  return lr >= 4 && lr <= 11 && lc >= 4 && lc <= 13;
+}
+GB_HD constexpr int join_frame_tile_log(int lr, int lc) { return lr <= 8 && lc <= 12 ? 12 : 13; }
 // Fewest elements a plan joins its passes for.
 constexpr int64_t kJoinMinElems = int64_t(1) << 21;
 
@@ -315,47 +405,54 @@ constexpr int64_t kJoinMinElems = int64_t(1) << 21;
 // so a tile only ever waits for tiles handed out before it, which running
 // blocks hold: no wait depends on blocks that have not started.
 //
-// Transform b's second pass follows its first by `lag` transforms; in between,
-// first-pass tiles of later transforms keep every block busy while the last
-// tiles of b's first pass finish.  The workspace is a ring of `ring` >= lag + 1
-// transforms, so what the second pass reads was written a few tens of MB
-// earlier and is still in L2, and the next user of the slot overwrites it
-// there: the intermediate need not reach HBM.
+// A unit is a transform, a frame, or a tile's worth of smaller frames.  The
+// second pass follows the first by `lag` tiles: a unit's, and as many more as
+// keep every block busy on later units while the last tiles of its first pass
+// finish.  So what the second pass reads was written a few tens of MB earlier
+// and is still in L2.  The workspace of four-step transforms is a ring of
+// `ring` units, large enough that a slot's second pass is over when its next
+// first pass comes up: the intermediate is overwritten in L2 and need not reach
+// HBM.  (Frames have their intermediate in the output; there the ring only
+// numbers the counters.)
 struct JoinOrder {
-  int64_t nb;  // transforms
-  int32_t tpt_log;  // log2 tiles per transform and pass
-  int32_t lag, ring;
+  int64_t nb;       // units
+  int32_t tpt_log;  // log2 tiles per unit and pass
+  int32_t ring;
+  int64_t lag;      // tiles, at most nb << tpt_log
 };
 struct JoinTicket {
   int pass;     // 0 or 1
-  int64_t b;    // transform
+  int64_t b;    // unit
   int32_t tile;
 };
 GB_HD int64_t join_tickets(const JoinOrder& o) { return (2 * o.nb) << o.tpt_log; }
+// lag tiles of the first pass, then second and first pass in turn, then the
+// last lag tiles of the second.
 GB_HD JoinTicket join_ticket(const JoinOrder& o, int64_t t) {
   JoinTicket k;
-  const int64_t lead = (int64_t)o.lag << o.tpt_log;
-  const int32_t mask = (1 << o.tpt_log) - 1;
-  if (t < lead) {  // the first `lag` transforms' first passes
-    k.pass = 0;
-    k.b = t >> o.tpt_log;
-    k.tile = (int32_t)t & mask;
-    return k;
+  const int64_t tiles = o.nb << o.tpt_log, both = t - o.lag;
+  int64_t i = t;
+  k.pass = 0;
+  if (both >= 2 * (tiles - o.lag)) {
+    k.pass = 1;
+    i = t - tiles;
+  } else if (both >= 0) {
+    k.pass = both & 1 ? 0 : 1;
+    i = (both >> 1) + (k.pass ? 0 : o.lag);
   }
-  t -= lead;
-  const int64_t mid = (2 * (o.nb - o.lag)) << o.tpt_log;
-  if (t < mid) {  // second pass of b, first pass of b + lag, tile by tile
-    const int64_t b = t >> (o.tpt_log + 1);
-    k.pass = (t & 1) ? 0 : 1;
-    k.b = k.pass ? b : b + o.lag;
-    k.tile = (int32_t)(t >> 1) & mask;
-    return k;
-  }
-  t -= mid;
-  k.pass = 1;
-  k.b = o.nb - o.lag + (t >> o.tpt_log);
-  k.tile = (int32_t)t & mask;
+  k.b = i >> o.tpt_log;
+  k.tile = (int32_t)(i - (k.b << o.tpt_log));
   return k;
+}
+// The lag and the ring for `batch` units of 2^tpt_log tiles with `resident`
+// blocks at work: a margin of 1.125 tiles per block (measured: 0.6 costs up to
+// 20% in waits, 2.5 as much in L2 misses).
+GB_HD void join_plan(int64_t batch, int tpt_log, int64_t resident, int64_t& lag, int64_t& ring) {
+  const int64_t unit = int64_t(1) << tpt_log, margin = resident + resident / 8;
+  lag = unit + margin;
+  if (lag > batch * unit) lag = batch * unit;
+  ring = 2 + (2 * margin + unit - 1) / unit;
+  if (ring > batch) ring = batch;
 }
 // What ticket k waits for: `count` finished tiles of ring slot `slot` in pass
 // `pass` (counted over the slot's users so far); count 0: nothing.

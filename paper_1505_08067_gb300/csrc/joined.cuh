@@ -91,144 +91,275 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   return done;
 }
 
-// Brings a first-pass tile's input into L2 (one thread; asynchronous).
-template <class PR>
-__device__ __forceinline__ void join_prefetch(const JoinDesc& d, const JoinTicket& k) {
-  constexpr int BR = PR::kN1 < 256 ? PR::kN1 : 256;
-  const uint64_t map = reinterpret_cast<uint64_t>(&d.tmap_in[0]);
-#pragma unroll 1
-  for (int j = 0; j < PR::kN1 / BR; ++j)
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map),
-                 "r"(k.tile * PR::kG1), "r"((int)(k.b * PR::kN1) + j * BR)
-                 : "memory");
+// The kernel's last warp hands out the tiles.  While the others work on one it
+// raises the count of the tile before (the release waits for that tile's stores
+// to reach L2; nobody else has to), takes the next ticket, waits for what that
+// depends on and prepares it.  A wait may be for this block's own tile, so it
+// raises that as soon as it is stored.  prefetch(k): one thread, as early as
+// possible; prepare(k, set): the warp, for the tile after the one at work.
+template <class Prefetch, class Prepare>
+__device__ __forceinline__ void join_dispatch(const JoinDesc& d, uint64_t* stored,
+                                              unsigned* s_ticket, int lane, Prefetch prefetch,
+                                              Prepare prepare) {
+  const unsigned total = (unsigned)join_tickets(d.o);
+  unsigned* finished = nullptr;
+  for (int n = 0;; ++n) {
+    unsigned t = 0;
+    if (lane == 0) {
+      t = atomicAdd(d.ctr, 1u);
+      if (t < total) {
+        const JoinTicket k = join_ticket(d.o, t);
+        if (k.pass == 0) prefetch(k);
+        const JoinDep dep = join_dep(d.o, k);
+        const unsigned* c = join_done(d, dep.pass, dep.slot);
+        bool ok = dep.count == 0;
+        for (uint32_t it = 0; it < kJoinPolls && !ok; ++it) {
+          ok = ld_acquire_gpu(c) >= dep.count;
+          if (!ok && finished && mbar_test(stored, (n - 1) & 1)) {
+            red_release_gpu(finished);
+            finished = nullptr;
+          }
+          if (!ok && it > 16) __nanosleep(64);
+        }
+        if (!ok) {
+          atomicExch(d.status, 1);
+          t = total;
+        }
+      }
+      s_ticket[n & 1] = t;
+    }
+    t = __shfl_sync(~0u, t, 0);
+    const JoinTicket k = join_ticket(d.o, t < total ? t : 0);
+    if (t < total) prepare(k, n & 1);
+    __syncthreads();  // the tile before is stored, this one may start
+    if (lane == 0 && finished) red_release_gpu(finished);
+    if (t >= total) break;
+    finished = join_done(d, k.pass, (int)(k.b % d.o.ring));
+  }
+  unsigned last = 0;
+  if (lane == 0) {
+    __threadfence();
+    last = atomicAdd(d.ctr + 1, 1u) == gridDim.x - 1;
+  }
+  if (__shfl_sync(~0u, last, 0))
+    for (int i = lane; i < 2 + 2 * d.o.ring; i += 32) d.ctr[i] = 0;
 }
 
-template <int LOGN, bool INV>
-__global__ void __launch_bounds__(JoinPair<LOGN>::kThreads + 32, 1 << join_blocks_log(JoinPair<LOGN>::kTileLog))
-joined_pass(const cf* in, cf* out, cf* work, const __grid_constant__ JoinDesc d) {
-  using PR = JoinPair<LOGN>;
-  using B1 = JoinBody<typename PR::P1, true, JoinMem>;
-  using B2 = JoinBody<typename PR::P2, false, JoinMem>;
-  constexpr int T = PR::kThreads;
-  extern __shared__ __align__(16) unsigned char smem_join[];
-  cf* sm = reinterpret_cast<cf*>(smem_join);
-  cf* steps = sm + PR::kTileSlots;  // two sets
-  __shared__ uint64_t stored;       // completes a phase when a tile's stores are issued
-  __shared__ unsigned s_ticket[2];
-  const int tid = threadIdx.x;
+// The other warps: tile(k, set) for every ticket the last warp publishes.
+template <class Tile>
+__device__ __forceinline__ void join_work(const JoinDesc& d, uint64_t* stored,
+                                          const unsigned* s_ticket, int tid, Tile tile) {
   const unsigned total = (unsigned)join_tickets(d.o);
-  if (tid == 0) mbar_init(&stored, T / 32);
-  __syncthreads();
-
-  if (tid >= T) {
-    // The last warp hands out the tiles.  While the others work on one it
-    // raises the count of the tile before (the release waits for that tile's
-    // stores to reach L2; nobody else has to), takes the next ticket, waits for
-    // what that depends on and computes its steps.  A wait may be for this
-    // block's own tile, so it raises that as soon as it is stored.
-    const int lane = tid - T;
-    unsigned* finished = nullptr;
-    for (int n = 0;; ++n) {
-      unsigned t = 0;
-      if (lane == 0) {
-        t = atomicAdd(d.ctr, 1u);
-        if (t < total) {
-          const JoinTicket k = join_ticket(d.o, t);
-          if (k.pass == 0 && d.mapped) join_prefetch<PR>(d, k);
-          const JoinDep dep = join_dep(d.o, k);
-          const unsigned* c = join_done(d, dep.pass, dep.slot);
-          bool ok = dep.count == 0;
-          for (uint32_t it = 0; it < kJoinPolls && !ok; ++it) {
-            ok = ld_acquire_gpu(c) >= dep.count;
-            if (!ok && finished && mbar_test(&stored, (n - 1) & 1)) {
-              red_release_gpu(finished);
-              finished = nullptr;
-            }
-            if (!ok && it > 16) __nanosleep(64);
-          }
-          if (!ok) {
-            atomicExch(d.status, 1);
-            t = total;
-          }
-        }
-        s_ticket[n & 1] = t;
-      }
-      t = __shfl_sync(~0u, t, 0);
-      const JoinTicket k = join_ticket(d.o, t < total ? t : 0);
-      if (t < total && k.pass == 0) B1::steps(steps + (n & 1) * PR::kSteps, k.tile * PR::kG1, LOGN, lane);
-      __syncthreads();  // the tile before is stored, this one may start
-      if (lane == 0 && finished) red_release_gpu(finished);
-      if (t >= total) break;
-      finished = join_done(d, k.pass, (int)(k.b % d.o.ring));
-    }
-    unsigned last = 0;
-    if (lane == 0) {
-      __threadfence();
-      last = atomicAdd(d.ctr + 1, 1u) == gridDim.x - 1;
-    }
-    if (__shfl_sync(~0u, last, 0))
-      for (int i = lane; i < 2 + 2 * d.o.ring; i += 32) d.ctr[i] = 0;
-    return;
-  }
-
   for (int n = 0;; ++n) {
     __syncthreads();  // every thread has read the last tile's shared memory
     const unsigned t = s_ticket[n & 1];
     if (t >= total) break;
-    const JoinTicket k = join_ticket(d.o, t);
+    tile(join_ticket(d.o, t), n & 1);
+    __syncwarp();
+    if ((tid & 31) == 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(stored)) : "memory");
+  }
+}
+
+// The stages of a tile between its loads and its stores; TW4 as JoinBody::turn.
+template <class SH, int KIND, bool TW4>
+__device__ __forceinline__ void join_stages(cf (&v)[kJoinR], cf* sm, const cf* tw, int col0,
+                                            int logN, int tid) {
+  using B = JoinBody<SH, KIND, JoinMem>;
+  B::dft0(v);
+  B::template put<0>(v, sm, tid);
+  join_sync<SH::kThreads>();
+  if constexpr (SH::kNst == 3) {
+    B::template get<1>(v, sm, tid);
+    B::template turn<1, false>(v, tw, 0, 0, tid);
+    join_sync<SH::kThreads>();
+    B::template put<1>(v, sm, tid);
+    join_sync<SH::kThreads>();
+  }
+  B::template get<SH::kLast>(v, sm, tid);
+  B::template turn<SH::kLast, TW4>(v, tw, col0, logN, tid);
+}
+
+// Four-step transforms of 2^LOGN points.
+template <int LOGN, bool INV>
+__global__ void __launch_bounds__(JoinPair<LOGN>::kThreads + 32,
+                                  1 << join_blocks_log(JoinPair<LOGN>::kTileLog))
+joined_pass(const cf* in, cf* out, cf* work, const __grid_constant__ JoinDesc d) {
+  using PR = JoinPair<LOGN>;
+  using B1 = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>;
+  using B2 = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>;
+  constexpr int T = PR::kThreads;
+  constexpr int kSlots = B1::kSlots > B2::kSlots ? B1::kSlots : B2::kSlots;
+  extern __shared__ __align__(16) unsigned char smem_join[];
+  cf* sm = reinterpret_cast<cf*>(smem_join);
+  cf* steps = sm + kSlots;     // two sets
+  __shared__ uint64_t stored;  // completes a phase when a tile's stores are issued
+  __shared__ unsigned s_ticket[2];
+  const int tid = threadIdx.x;
+  if (tid == 0) mbar_init(&stored, T / 32);
+  __syncthreads();
+  if (tid >= T) {
+    join_dispatch(
+        d, &stored, s_ticket, tid - T,
+        [&](const JoinTicket& k) {  // the tile's columns, asynchronously into L2
+          if (!d.mapped) return;
+          constexpr int BR = PR::kN1 < 256 ? PR::kN1 : 256;
+          const uint64_t map = reinterpret_cast<uint64_t>(&d.tmap_in[0]);
+#pragma unroll 1
+          for (int j = 0; j < PR::kN1 / BR; ++j)
+            asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map),
+                         "r"(k.tile * PR::kG1), "r"((int)(k.b * PR::kN1) + j * BR)
+                         : "memory");
+        },
+        [&](const JoinTicket& k, int set) {
+          if (k.pass == 0) B1::steps(steps + set * PR::kSteps, k.tile * PR::kG1, LOGN, tid - T);
+        });
+    return;
+  }
+  join_work(d, &stored, s_ticket, tid, [&](const JoinTicket& k, int set) {
     cf* w = work + (int64_t)(k.b % d.o.ring) * PR::kN;
-    const cf* st = steps + (n & 1) * PR::kSteps;
     cf v[kJoinR];
     if (k.pass == 0) {
       const int col0 = k.tile * PR::kG1;
       B1::template first<INV, false>(v, in + k.b * PR::kN + col0, PR::kN2, tid);
-      B1::dft0(v);
-      B1::template put<0>(v, sm, tid);
-      join_sync<T>();
-      if constexpr (PR::P1::kNst == 3) {
-        B1::template get<1>(v, sm, tid);
-        B1::template turn<1, false>(v, d.tw1, 0, 0, tid);
-        join_sync<T>();
-        B1::template put<1>(v, sm, tid);
-        join_sync<T>();
-      }
-      B1::template get<PR::P1::kLast>(v, sm, tid);
-      B1::template turn<PR::P1::kLast, true>(v, d.tw1, col0, LOGN, tid);
-      B1::template store_block<PR::kG2>(v, w + col0 * PR::kG2, st, PR::kN2, tid);
+      join_stages<typename PR::P1, JOIN_FIRST, true>(v, sm, d.tw1, col0, LOGN, tid);
+      B1::template store_block<PR::kG2>(v, w + col0 * PR::kG2, steps + set * PR::kSteps, PR::kN2,
+                                        tid);
     } else {
       B2::template first<false, true>(v, w + k.tile * PR::kTile, PR::kG2, tid);
-      B2::dft0(v);
-      B2::template put<0>(v, sm, tid);
-      join_sync<T>();
-      if constexpr (PR::P2::kNst == 3) {
-        B2::template get<1>(v, sm, tid);
-        B2::template turn<1, false>(v, d.tw2, 0, 0, tid);
-        join_sync<T>();
-        B2::template put<1>(v, sm, tid);
-        join_sync<T>();
-      }
-      B2::template get<PR::P2::kLast>(v, sm, tid);
-      B2::template turn<PR::P2::kLast, false>(v, d.tw2, 0, 0, tid);
+      join_stages<typename PR::P2, JOIN_COLS, false>(v, sm, d.tw2, 0, 0, tid);
       B2::template store_cols<INV>(v, out + k.b * PR::kN + k.tile * PR::kG2, PR::kN1, tid);
     }
-    __syncwarp();
-    if ((tid & 31) == 0)
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&stored)) : "memory");
+  });
+}
+
+// One tile of rows (from in to out) or of columns (in place) of frames.
+template <int TL, int LOGL, bool INV>
+__device__ __forceinline__ void join_rows(const cf* in, cf* out, const JoinDesc& d, int64_t tile,
+                                          cf* sm, int tid) {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  using B = JoinBody<SH, JOIN_ROWS, JoinMem>;
+  const int64_t valid = (d.total >> LOGL) - tile * B::G;
+  cf v[kJoinR];
+  B::template first_rows<INV>(v, in + (tile << TL), valid, tid);
+  join_stages<SH, JOIN_ROWS, false>(v, sm, d.tw1, 0, 0, tid);
+  B::store_rows(v, out + (tile << TL), valid, tid);
+}
+template <int TL, int LOGL, bool INV>
+__device__ __forceinline__ void join_cols(cf* buf, const JoinDesc& d, int64_t tile, cf* sm,
+                                          int tid) {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  using B = JoinBody<SH, JOIN_COLS, JoinMem>;
+  cf v[kJoinR];
+  B::first_frame(v, buf, tile * B::G, d.total >> LOGL, d.lc, tid);
+  join_stages<SH, JOIN_COLS, false>(v, sm, d.tw2, 0, 0, tid);
+  B::template store_frame<INV>(v, buf, tile * B::G, d.total >> LOGL, d.lc, tid);
+}
+
+// 2D frames of 2^lr rows of 2^lc elements: row pass from in to out, column pass
+// in out.  One kernel for all lengths (a block uses two of the bodies below):
+// the column passes had compile-time shapes for 4096 rows only, and the
+// run-time-parameter kernel is bound by its address arithmetic and its load
+// queue.  Column passes read 64 bytes per row at 1024 rows and 32 at 2048;
+// 4096 rows and more (16 bytes) keep the staged column kernel and its tensor-map
+// loads.  Tiles of 4096 elements up to 256 rows (measured as for transforms
+// above), else 8192.
+// Measured, 2^25 elements, before (a launch per pass) and now: 16 x 16 390 ->
+// 139 us, 64 x 64 242 -> 123, 256 x 1024 201 -> 144, 512 x 512 247 -> 148,
+// 1024 x 1024 271 -> 161, 1024 x 8192 293 -> 223, 2048 x 1024 272 -> 209,
+// 2048 x 8192 297 -> 270; 2^21 elements: 20.6-39.9 -> 16.7-24.7 us.
+template <int TL, bool INV>
+__global__ void __launch_bounds__((1 << TL) / kJoinR + 32, 1 << join_blocks_log(TL))
+joined_frames(const cf* in, cf* out, const __grid_constant__ JoinDesc d) {
+  constexpr int T = (1 << TL) / kJoinR;
+  extern __shared__ __align__(16) unsigned char smem_join[];
+  cf* sm = reinterpret_cast<cf*>(smem_join);
+  __shared__ uint64_t stored;
+  __shared__ unsigned s_ticket[2];
+  const int tid = threadIdx.x;
+  if (tid == 0) mbar_init(&stored, T / 32);
+  __syncthreads();
+  if (tid >= T) {
+    join_dispatch(
+        d, &stored, s_ticket, tid - T,
+        [&](const JoinTicket& k) {
+          if (!d.mapped) return;
+          const int64_t at = (((k.b << d.o.tpt_log) + k.tile)) << TL;
+          const int64_t n = d.total - at < (1 << TL) ? d.total - at : (1 << TL);
+          if (n > 0)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(in + at),
+                         "r"((unsigned)n * 8)
+                         : "memory");
+        },
+        [](const JoinTicket&, int) {});
+    return;
   }
+  join_work(d, &stored, s_ticket, tid, [&](const JoinTicket& k, int) {
+    const int64_t tile = (k.b << d.o.tpt_log) + k.tile;
+    if (k.pass == 0) {
+      switch (d.lc) {
+        case 4: join_rows<TL, 4, INV>(in, out, d, tile, sm, tid); break;
+        case 5: join_rows<TL, 5, INV>(in, out, d, tile, sm, tid); break;
+        case 6: join_rows<TL, 6, INV>(in, out, d, tile, sm, tid); break;
+        case 7: join_rows<TL, 7, INV>(in, out, d, tile, sm, tid); break;
+        case 8: join_rows<TL, 8, INV>(in, out, d, tile, sm, tid); break;
+        case 9: join_rows<TL, 9, INV>(in, out, d, tile, sm, tid); break;
+        case 10: join_rows<TL, 10, INV>(in, out, d, tile, sm, tid); break;
+        case 11: join_rows<TL, 11, INV>(in, out, d, tile, sm, tid); break;
+        case 12: join_rows<TL, 12, INV>(in, out, d, tile, sm, tid); break;
+        default:
+          if constexpr (TL >= 13) join_rows<TL, 13, INV>(in, out, d, tile, sm, tid);
+          break;
+      }
+    } else {
+      switch (d.lr) {
+        case 4: join_cols<TL, 4, INV>(out, d, tile, sm, tid); break;
+        case 5: join_cols<TL, 5, INV>(out, d, tile, sm, tid); break;
+        case 6: join_cols<TL, 6, INV>(out, d, tile, sm, tid); break;
+        case 7: join_cols<TL, 7, INV>(out, d, tile, sm, tid); break;
+        case 8: join_cols<TL, 8, INV>(out, d, tile, sm, tid); break;
+        default:
+          if constexpr (TL >= 13) {
+            if (d.lr == 9) join_cols<TL, 9, INV>(out, d, tile, sm, tid);
+            else if (d.lr == 10) join_cols<TL, 10, INV>(out, d, tile, sm, tid);
+            else join_cols<TL, 11, INV>(out, d, tile, sm, tid);
+          }
+          break;
+      }
+    }
+  });
 }
 
 template <int LOGN>
 inline void joined_fn(bool inv, JoinedLaunch& j) {
   using PR = JoinPair<LOGN>;
+  using B1 = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>;
+  using B2 = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>;
   j.fn = inv ? (const void*)joined_pass<LOGN, true> : (const void*)joined_pass<LOGN, false>;
-  j.smem = (PR::kTileSlots + 2 * PR::kSteps) * sizeof(cf);
+  j.smem = ((B1::kSlots > B2::kSlots ? B1::kSlots : B2::kSlots) + 2 * PR::kSteps) * sizeof(cf);
   j.block = PR::kThreads + 32;
   j.d.o.tpt_log = LOGN - PR::kTileLog;
   j.n1 = PR::kN1;
   j.n2 = PR::kN2;
   j.g1 = PR::kG1;
   j.box_rows = PR::kN1 < 256 ? PR::kN1 : 256;
+}
 
+// Shared memory of the frame kernels: the largest tile of their bodies.
+template <int TL, int LOGL, int TOP>
+constexpr int join_frame_slots() {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  constexpr int rows = JoinBody<SH, JOIN_ROWS, JoinMem>::kSlots;
+  constexpr int cols = JoinBody<SH, JOIN_COLS, JoinMem>::kSlots;
+  constexpr int here = rows > cols ? rows : cols;
+  if constexpr (LOGL == TOP) return here;
+  else return here > join_frame_slots<TL, LOGL + 1, TOP>() ? here : join_frame_slots<TL, LOGL + 1, TOP>();
+}
+template <int TL>
+inline void joined_frames_fn(bool inv, JoinedLaunch& j) {
+  j.fn = inv ? (const void*)joined_frames<TL, true> : (const void*)joined_frames<TL, false>;
+  j.smem = join_frame_slots<TL, 4, TL < 13 ? 12 : 13>() * sizeof(cf);
+  j.block = (1 << TL) / kJoinR + 32;
 }
 
 }  // namespace gbfft

@@ -8,30 +8,39 @@
 
 namespace gbfft {
 
-// The joined two-pass kernel (joined.cuh).
+// The joined kernels (joined.cuh): both passes of a four-step transform, or of
+// 2D frames, in one launch.
 struct JoinDesc {
-  const cf* tw1;  // w_{N1}^j, w_{N2}^j
+  const cf* tw1;  // w_L^j of the first pass's length, and of the second's
   const cf* tw2;
   JoinOrder o;
   unsigned* ctr;  // 2 + 2 ring counters, zero between launches
   int* status;
-  // when `mapped`, a tensor map of the input viewed as rows of N2 complex64
-  // elements in boxes of G1 columns: first-pass tiles are prefetched into L2
+  // frames: log2 rows and columns, elements of the whole batch
+  int lr, lc;
+  int64_t total;
+  // first-pass tiles are prefetched into L2 when `mapped`: for transforms by a
+  // tensor map of the input viewed as rows of N2 elements in boxes of G1
+  // columns; frames only need a 16-byte-aligned input
   int mapped;
   alignas(64) unsigned char tmap_in[128];
 };
 struct JoinedLaunch {
   const void* fn = nullptr;  // null: the plan's passes run as launches of their own
+  bool frames = false;
   int max_grid = 0;          // resident blocks
   int block = 0;
   size_t smem = 0;
   int n1 = 0, n2 = 0, g1 = 0, box_rows = 0;
   JoinDesc d{};
 };
-// Kernel for N = 2^logn, its opt-in shared memory and resident blocks.
+// Kernel for transforms of 2^logn, or frames of 2^lr x 2^lc, its opt-in shared
+// memory, resident blocks and tiles per unit.
 cudaError_t prepare_joined(int logn, bool inverse, int sm_count, JoinedLaunch* j);
-cudaError_t launch_joined(const JoinedLaunch& j, int64_t nb, const void* in, void* out, void* work,
-                          cudaStream_t st);
+cudaError_t prepare_joined_frames(int lr, int lc, bool inverse, int sm_count, JoinedLaunch* j);
+// `batch` transforms or frames; `work`: the ring of a four-step plan.
+cudaError_t launch_joined(const JoinedLaunch& j, int64_t batch, const void* in, void* out,
+                          void* work, cudaStream_t st);
 // Tensor map (128 bytes) over `rows` rows of `cols` complex64 elements at `p`,
 // boxes of box_cols x box_rows; false if `p` or the driver does not allow it.
 bool encode_rows_map(const void* p, int64_t cols, int64_t rows, int box_cols, int box_rows,

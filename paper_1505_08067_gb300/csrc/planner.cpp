@@ -207,19 +207,18 @@ static PassSpec contiguous_pass(int logL, int64_t batch, int64_t units_per_batch
   return p;
 }
 
-// Does a two-pass plan of `batch` transforms per sub-batch run its passes as
-// one launch, and in what order (fft_join.h)?
-static void plan_joined(PlanSpec& s, int logN, int64_t batch, const Caps& caps) {
-  if (logN < kJoinMinLog || logN > kJoinMaxLog) return;
-  if (batch << logN < kJoinMinElems) return;
-  // ticks of the lag: 2.5 times the tiles in work at once (join_blocks_log)
-  const int tl = join_tile_log(logN);
-  const int64_t tiles = int64_t(1) << (logN - tl);  // per transform and pass
-  const int64_t resident = (int64_t)caps.sm_count << join_blocks_log(tl);
-  const int64_t lag = std::max<int64_t>(1, (5 * resident + 4 * tiles - 1) / (4 * tiles));
+// Do the two passes of a plan of `batch` transforms of 2^logE elements (1D:
+// per sub-batch; 2D: frames) run as one launch of tiles of 2^tile_log, and in
+// what order (fft_join.h)?
+static void plan_joined(PlanSpec& s, int logE, int tile_log, int64_t batch, const Caps& caps) {
+  if (batch << logE < kJoinMinElems) return;
+  const int tpt_log = std::max(0, logE - tile_log);
+  const int64_t per_unit = int64_t(1) << std::max(0, tile_log - logE);
+  const int64_t units = (batch + per_unit - 1) / per_unit;
+  int64_t ring;
+  join_plan(units, tpt_log, (int64_t)caps.sm_count << join_blocks_log(tile_log), s.join_lag, ring);
+  s.join_ring = (int)ring;
   s.joined = true;
-  s.join_lag = (int)std::min(lag, batch);
-  s.join_ring = (int)std::min(2 * lag, batch);
 }
 
 void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direction,
@@ -284,6 +283,8 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
   s.max_block_log2 = bmax;
   s.generic_only = o.generic != 0;
   const int inv = direction == FFT_INVERSE;
+  const bool defaults = !o.radix && !o.schedule && o.max_block_log2 <= 0 && !o.tile &&
+                        !o.generic && !o.variant && !o.epilogue && !o.split_log2;
 
   if (conv) {
     // Fast convolution: every line on one SM, forward stages, filter, forward
@@ -485,9 +486,8 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       const int64_t chunk = two_pass_chunk(N);
       s.chunk_batch = batch > chunk ? chunk : 0;
       s.work_elems = std::min(batch, chunk) * N;
-      const bool defaults = !o.radix && !o.schedule && o.max_block_log2 <= 0 && !o.tile &&
-                            !o.generic && !o.variant && !o.epilogue && !o.split_log2;
-      if (defaults) plan_joined(s, logN, std::min(batch, chunk), caps);
+      if (defaults && logN >= kJoinMinLog && logN <= kJoinMaxLog)
+        plan_joined(s, logN, join_tile_log(logN), std::min(batch, chunk), caps);
     }
   } else {
     const int64_t rows = n[0], cols = n[1];
@@ -527,6 +527,8 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       p.conj_out = inv;
       s.passes.push_back(p);
     }
+    if (defaults && join_frame(lr, lc))
+      plan_joined(s, lr + lc, join_frame_tile_log(lr, lc), batch, caps);
   }
 
   // launch shapes and twiddle tables
@@ -568,14 +570,13 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
     }
   }
   if (s.joined) {
-    const int logN = ilog2(s.n[0]);
-    const int64_t N1 = int64_t(1) << (logN / 2), N2 = s.n[0] / N1;
+    const int64_t L1 = int64_t(1) << s.passes[0].logL, L2 = int64_t(1) << s.passes[1].logL;
     s.join_tw1 = off;
-    s.tables.push_back(TwSegment{off, N1, N1, 1, 1, 1});
-    off += N1;
+    s.tables.push_back(TwSegment{off, L1, L1, 1, 1, 1});
+    off += L1;
     s.join_tw2 = off;
-    s.tables.push_back(TwSegment{off, N2, N2, 1, 1, 1});
-    off += N2;
+    s.tables.push_back(TwSegment{off, L2, L2, 1, 1, 1});
+    off += L2;
   }
   s.table_elems = off;
   for (auto& p : s.passes) {

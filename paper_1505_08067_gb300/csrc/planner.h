@@ -118,10 +118,11 @@ struct PlanSpec {
   // two-pass 1D plans execute in sub-batches of at most chunk_batch transforms
   // (0: no sub-batching); work_elems holds one sub-batch
   int64_t chunk_batch = 0;
-  // two-pass 1D plans whose passes run as one launch (fft_join.h): the order
-  // of its tiles and the offsets of its twiddle tables w_{N1}^j, w_{N2}^j
+  // plans whose two passes run as one launch (fft_join.h): the order of its
+  // tiles and the offsets of its twiddle tables w_L^j for the passes' lengths
   bool joined = false;
-  int join_lag = 1, join_ring = 1;
+  int64_t join_lag = 1;
+  int join_ring = 1;
   int64_t join_tw1 = 0, join_tw2 = 0;
   // six-step plans: the second workspace buffer starts work2_off elements in
   int64_t work2_off = 0;

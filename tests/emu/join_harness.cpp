@@ -11,6 +11,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -103,31 +104,36 @@ std::vector<cf> roots(int n) {
   return t;
 }
 
-template <class SH, bool ROWL, class First, class Store>
+template <class SH, int KIND, class First, class Store>
 void tile(cf* sm, cf* st, const cf* tw, int col0, int logN, First first, Store store) {
-  using B = JoinBody<SH, ROWL, CheckMem>;
+  using B = JoinBody<SH, KIND, CheckMem>;
   std::vector<cf> regs((size_t)SH::kThreads * kJoinR);
   auto v = [&](int t) -> cf (&)[kJoinR] { return *reinterpret_cast<cf(*)[kJoinR]>(&regs[(size_t)t * kJoinR]); };
   auto each = [&](auto f) { for (int t = 0; t < SH::kThreads; ++t) f(v(t), t); };
   ++g.phase;
-  if (ROWL)
+  if (KIND == JOIN_FIRST)
     for (int lane = 0; lane < 32; ++lane) B::steps(st, col0, logN, lane);
   each([&](cf (&r)[kJoinR], int t) { first(r, t); B::dft0(r); B::template put<0>(r, sm, t); });
+  if constexpr (SH::kNst == 3) {  // rows and columns of frames: no steps to keep
+    each([&](cf (&r)[kJoinR], int t) { B::template get<1>(r, sm, t); B::template turn<1, false>(r, tw, 0, 0, t); });
+    ++g.phase;
+    each([&](cf (&r)[kJoinR], int t) { B::template put<1>(r, sm, t); });
+  }
   each([&](cf (&r)[kJoinR], int t) {
     B::template get<SH::kLast>(r, sm, t);
-    B::template turn<SH::kLast, ROWL>(r, tw, col0, logN, t);  // pass 1 carries the four-step twiddle
+    B::template turn<SH::kLast, KIND == JOIN_FIRST>(r, tw, col0, logN, t);  // pass 1 carries the four-step twiddle
     store(r, t);
   });
 }
 
 template <int LOGN, bool INV>
-int64_t run(int64_t nb, int lag, int ring, const cf* in, cf* out) {
+int64_t run(int64_t nb, int64_t lag, int ring, const cf* in, cf* out) {
   using PR = JoinPair<LOGN>;
-  using B1 = JoinBody<typename PR::P1, true, CheckMem>;
-  using B2 = JoinBody<typename PR::P2, false, CheckMem>;
+  using B1 = JoinBody<typename PR::P1, JOIN_FIRST, CheckMem>;
+  using B2 = JoinBody<typename PR::P2, JOIN_COLS, CheckMem>;
   g = Ctx{};
   std::vector<cf> t1 = roots(PR::kN1), t2 = roots(PR::kN2), work((size_t)ring * PR::kN),
-                  sm(PR::kTileSlots + PR::kSteps);
+                  sm(std::max(B1::kSlots, B2::kSlots) + PR::kSteps);
   g.in = in;
   g.out = out;
   g.in_len = g.out_len = nb * PR::kN;
@@ -142,9 +148,9 @@ int64_t run(int64_t nb, int lag, int ring, const cf* in, cf* out) {
   g.sm = sm.data();
   g.smem_len = (int)sm.size();
   g.phase_of.assign(sm.size(), -1);
-  cf* st = sm.data() + PR::kTileSlots;
+  cf* st = sm.data() + std::max(B1::kSlots, B2::kSlots);
   static_assert(join_tile_log(LOGN) == PR::kTileLog, "the planner's tile");
-  JoinOrder o{nb, LOGN - PR::kTileLog, lag < nb ? lag : (int)nb, ring};
+  JoinOrder o{nb, LOGN - PR::kTileLog, ring, std::min<int64_t>(lag, nb * PR::kTiles)};
   std::vector<uint32_t> done(2 * ring, 0);
   for (int64_t t = 0; t < join_tickets(o); ++t) {
     const JoinTicket k = join_ticket(o, t);
@@ -156,12 +162,12 @@ int64_t run(int64_t nb, int lag, int ring, const cf* in, cf* out) {
     g.b = k.b;
     if (k.pass == 0) {
       const int col0 = k.tile * PR::kG1;
-      tile<typename PR::P1, true>(
+      tile<typename PR::P1, JOIN_FIRST>(
           sm.data(), st, g.tw1, col0, LOGN,
           [&](cf (&v)[kJoinR], int i) { B1::template first<INV, false>(v, in + k.b * PR::kN + col0, PR::kN2, i); },
           [&](cf (&v)[kJoinR], int i) { B1::template store_block<PR::kG2>(v, w + col0 * PR::kG2, st, PR::kN2, i); });
     } else {
-      tile<typename PR::P2, false>(
+      tile<typename PR::P2, JOIN_COLS>(
           sm.data(), st, g.tw2, 0, 0,
           [&](cf (&v)[kJoinR], int i) { B2::template first<false, true>(v, w + k.tile * PR::kTile, PR::kG2, i); },
           [&](cf (&v)[kJoinR], int i) { B2::template store_cols<INV>(v, out + k.b * PR::kN + k.tile * PR::kG2, PR::kN1, i); });
@@ -173,9 +179,79 @@ int64_t run(int64_t nb, int lag, int ring, const cf* in, cf* out) {
   return g.errors;
 }
 
+template <int TL, int LOGL, bool INV>
+void rows(const cf* in, cf* out, int64_t total, int64_t t, cf* sm) {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  using B = JoinBody<SH, JOIN_ROWS, CheckMem>;
+  const int64_t valid = (total >> LOGL) - t * B::G;
+  tile<SH, JOIN_ROWS>(
+      sm, sm, g.tw1, 0, 0,
+      [&](cf (&v)[kJoinR], int i) { B::template first_rows<INV>(v, in + (t << TL), valid, i); },
+      [&](cf (&v)[kJoinR], int i) { B::store_rows(v, out + (t << TL), valid, i); });
+}
+template <int TL, int LOGL, bool INV>
+void cols(cf* mid, cf* out, int64_t total, int64_t t, int lc, cf* sm) {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  using B = JoinBody<SH, JOIN_COLS, CheckMem>;
+  tile<SH, JOIN_COLS>(
+      sm, sm, g.tw2, 0, 0,
+      [&](cf (&v)[kJoinR], int i) { B::first_frame(v, mid, t * B::G, total >> LOGL, lc, i); },
+      [&](cf (&v)[kJoinR], int i) { B::template store_frame<INV>(v, out, t * B::G, total >> LOGL, lc, i); });
+}
+
+// Frames: the row pass writes `mid` (the output buffer on the GPU, kept apart
+// here so that reads and writes of it can be checked on their own).
+template <int TL, bool INV>
+int64_t run_frames(int64_t batch, int lr, int lc, const cf* in, cf* out) {
+  g = Ctx{};
+  const int64_t total = batch << (lr + lc);
+  std::vector<cf> t1 = roots(1 << lc), t2 = roots(1 << lr), mid(total), sm(1 << 15);
+  const int tpt_log = std::max(0, lr + lc - TL);
+  const int64_t nb = (total + (int64_t(1) << (TL + tpt_log)) - 1) >> (TL + tpt_log);
+  int64_t lag, ring;
+  join_plan(nb, tpt_log, 6, lag, ring);
+  JoinOrder o{nb, tpt_log, (int)ring, lag};
+  g.in = in;
+  g.out = out;
+  g.work = mid.data();
+  g.in_len = g.out_len = g.work_len = total;
+  g.out_hits.assign(total, 0);
+  g.work_owner.assign(total, -1);
+  g.b = 0;
+  g.tw1 = t1.data();
+  g.tw2 = t2.data();
+  g.tw1_len = 1 << lc;
+  g.tw2_len = 1 << lr;
+  g.sm = sm.data();
+  g.smem_len = (int)sm.size();
+  g.phase_of.assign(sm.size(), -1);
+  std::vector<uint32_t> done(2 * ring, 0);
+  for (int64_t t = 0; t < join_tickets(o); ++t) {
+    const JoinTicket k = join_ticket(o, t);
+    const JoinDep dep = join_dep(o, k);
+    if (k.b < 0 || k.b >= nb || k.tile < 0 || k.tile >> tpt_log) { err("ticket out of range", t); break; }
+    if (done[dep.pass * ring + dep.slot] < dep.count) err("a ticket waits for a later one", t);
+    const int64_t at = (k.b << tpt_log) + k.tile;
+    switch (k.pass ? 100 + lr : lc) {
+#define GB_R(L) case L: rows<TL, L, INV>(in, mid.data(), total, at, sm.data()); break;
+#define GB_C(L) case 100 + L: cols<TL, L, INV>(mid.data(), out, total, at, lc, sm.data()); break;
+      GB_R(4) GB_R(5) GB_R(6) GB_R(7) GB_R(8) GB_R(9) GB_R(10) GB_R(11) GB_R(12)
+      GB_C(4) GB_C(5) GB_C(6) GB_C(7) GB_C(8)
+      default:
+        if constexpr (TL == 13) switch (k.pass ? 100 + lr : lc) { GB_R(13) GB_C(9) GB_C(10) GB_C(11) default: break; }
+#undef GB_R
+#undef GB_C
+    }
+    ++done[k.pass * ring + (int)(k.b % ring)];
+  }
+  for (int64_t i = 0; i < total; ++i)
+    if (g.out_hits[i] != 1 || g.work_owner[i] != 0) { err("element not written exactly once", i); break; }
+  return g.errors;
+}
+
 }  // namespace
 
-extern "C" int64_t join_run(int logn, int64_t nb, int inverse, int lag, int ring, const float* in,
+extern "C" int64_t join_run(int logn, int64_t nb, int inverse, int64_t lag, int ring, const float* in,
                             float* out, char* msg, size_t len) {
   const cf* x = reinterpret_cast<const cf*>(in);
   cf* y = reinterpret_cast<cf*>(out);
@@ -187,6 +263,18 @@ extern "C" int64_t join_run(int logn, int64_t nb, int inverse, int lag, int ring
 #undef GB_RUN
     default: break;
   }
+  snprintf(msg, len, "%s", g.first.c_str());
+  return e;
+}
+
+extern "C" int64_t join_run_frames(int64_t batch, int lr, int lc, int inverse, const float* in,
+                                   float* out, char* msg, size_t len) {
+  const cf* x = reinterpret_cast<const cf*>(in);
+  cf* y = reinterpret_cast<cf*>(out);
+  if (!join_frame(lr, lc)) return -1;
+  const int64_t e = join_frame_tile_log(lr, lc) == 12
+                        ? (inverse ? run_frames<12, true>(batch, lr, lc, x, y) : run_frames<12, false>(batch, lr, lc, x, y))
+                        : (inverse ? run_frames<13, true>(batch, lr, lc, x, y) : run_frames<13, false>(batch, lr, lc, x, y));
   snprintf(msg, len, "%s", g.first.c_str());
   return e;
 }

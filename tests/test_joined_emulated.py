@@ -24,22 +24,41 @@ def joined():
         subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-shared", "-fPIC",
                         "-Wno-unknown-pragmas", "-I" + CSRC, "-o", tmp, src], check=True)
         os.replace(tmp, lib)
-    f = ctypes.CDLL(lib).join_run
-    f.restype = ctypes.c_int64
-    f.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_int,
-                  ctypes.c_void_p, ctypes.c_void_p, ctypes.c_char_p, ctypes.c_size_t]
+    f = ctypes.CDLL(lib)
+    f.join_run.restype = f.join_run_frames.restype = ctypes.c_int64
+    f.join_run.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int, ctypes.c_int64, ctypes.c_int,
+                           ctypes.c_void_p, ctypes.c_void_p, ctypes.c_char_p, ctypes.c_size_t]
+    f.join_run_frames.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_int,
+                                  ctypes.c_void_p, ctypes.c_void_p, ctypes.c_char_p, ctypes.c_size_t]
     return f
 
 
 # one transform, a ring that is reused, a lag of several transforms, no reuse
-@pytest.mark.parametrize("logn,batch,lag,ring", [(15, 7, 2, 3), (15, 1, 4, 1), (16, 3, 1, 2),
-                                                 (17, 3, 2, 3), (18, 3, 1, 2), (19, 2, 1, 2),
-                                                 (20, 1, 1, 1)])
+# (lag in tiles: 8 to 64 per transform)
+@pytest.mark.parametrize("logn,batch,lag,ring", [(15, 7, 19, 4), (15, 1, 40, 1), (16, 3, 16, 2),
+                                                 (17, 3, 33, 3), (18, 3, 32, 2), (19, 2, 64, 2),
+                                                 (20, 1, 64, 1)])
 @pytest.mark.parametrize("direction", [-1, 1])
 def test_joined(oracle, joined, logn, batch, lag, ring, direction):
     x = synth.uniform(60 + logn, batch, 2 ** logn)
     y = np.zeros_like(x)
     msg = ctypes.create_string_buffer(256)
-    n = joined(logn, batch, int(direction > 0), lag, ring, x.ctypes.data, y.ctypes.data, msg, 256)
+    n = joined.join_run(logn, batch, int(direction > 0), lag, ring, x.ctypes.data, y.ctypes.data, msg, 256)
     assert n == 0, msg.value.decode()
     assert np.max(oracle.rel_l2(y, oracle.fft(x, direction))) <= 1e-6 * logn
+
+
+# every column length and row length, frames smaller than a tile with a ragged
+# last one, both tile sizes
+@pytest.mark.parametrize("lr,lc,batch", [(4, 4, 37), (5, 6, 7), (6, 5, 3), (7, 7, 2), (8, 8, 2),
+                                         (4, 12, 2), (9, 4, 3), (10, 5, 2), (11, 6, 1), (8, 9, 1),
+                                         (5, 10, 2), (4, 11, 1), (5, 13, 1), (9, 9, 1), (10, 4, 5)])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_joined_frames(oracle, joined, lr, lc, batch, direction):
+    x = synth.uniform(80 + lr, batch, 2 ** (lr + lc)).reshape(batch, 2 ** lr, 2 ** lc)
+    y = np.zeros_like(x)
+    msg = ctypes.create_string_buffer(256)
+    n = joined.join_run_frames(batch, lr, lc, int(direction > 0), x.ctypes.data, y.ctypes.data, msg, 256)
+    assert n == 0, msg.value.decode()
+    ref = oracle.fft2d(x, direction).reshape(batch, -1)
+    assert np.max(oracle.rel_l2(y.reshape(batch, -1), ref)) <= 1e-6 * (lr + lc)

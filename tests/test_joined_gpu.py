@@ -77,3 +77,41 @@ def test_two_plans_on_two_streams(gb, oracle):
                 plan.execute(x, y, stream=s)
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(want, got))
+
+
+@pytest.mark.parametrize("shape,batch", [((16, 16), 8193), ((32, 64), 1031), ((64, 128), 257),
+                                         ((512, 16), 257), ((256, 8192), 1), ((16, 4096), 33),
+                                         ((32, 2048), 35), ((128, 32), 513), ((1024, 512), 5),
+                                         ((2048, 16), 65), ((2048, 2048), 1), ((256, 256), 33)])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_joined_frames(gb, oracle, shape, batch, direction):
+    """Frames smaller than a tile with a ragged last one, frames of one tile and
+    of many, both tile sizes, both ends of the length ranges."""
+    n = shape[0] * shape[1]
+    x_np = synth.uniform(800 + shape[0], batch, n).reshape((batch,) + shape)
+    idx = np.unique([0, batch // 2, batch - 1])
+    buf = torch.empty(batch * n + 1, dtype=torch.complex64, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    with gb.Plan(shape, batch, direction) as p:
+        assert p.describe()["joined"] == 1 and p.launch_count == 1
+        first = None
+        for shift in (0, 1):
+            x = buf[shift:shift + batch * n].view((batch,) + shape)
+            x.copy_(torch.from_numpy(x_np))
+            y = torch.full_like(x, float("nan"))
+            p.execute(x, y)
+            first = y if first is None else first
+            assert torch.equal(first, y)
+        p.execute(x, x)
+        gb.fft_plan_sync_status(p.handle, s)
+        assert torch.equal(first, x)
+    ref = oracle.fft2d(x_np[idx], direction).reshape(len(idx), n)
+    got = first[torch.from_numpy(idx).cuda()].cpu().numpy().reshape(len(idx), n)
+    assert np.max(oracle.rel_l2(got, ref)) <= 1e-6 * np.log2(n)
+
+
+@pytest.mark.parametrize("shape,batch", [((512, 16), 255), ((8, 4096), 80), ((4096, 512), 1),
+                                         ((64, 16384), 3), ((4096, 8192), 1)])
+def test_frames_not_joined(gb, shape, batch):
+    with gb.Plan(shape, batch) as p:
+        assert p.describe()["joined"] == 0 and p.launch_count == 2
