@@ -88,8 +88,10 @@ cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, i
                         unsigned* counters, JoinedLaunch* j) {
   const int l0 = s.passes[0].logL, l1 = s.passes[1].logL;
   const bool inv = s.direction == FFT_INVERSE;
-  const cudaError_t e = s.dims == 2 ? prepare_joined_frames(l1, l0, inv, caps.sm_count, j)
-                                    : prepare_joined(l0 + l1, inv, caps.sm_count, j);
+  const cudaError_t e = s.dims == 2 ? prepare_joined_frames(l1, l0, s.join_tile_log, inv,
+                                                            caps.sm_count, j)
+                                    : prepare_joined(l0 + l1, s.join_tile_log, inv,
+                                                     caps.sm_count, j);
   if (e != cudaSuccess) return e;
   j->d.tw1 = tables + s.join_tw1;
   j->d.tw2 = tables + s.join_tw2;

@@ -380,25 +380,43 @@ template <int TL> struct JoinLen<TL, 10> { using S = Join1024<TL>; };
 template <int TL> struct JoinLen<TL, 11> { using S = JoinShape<TL, 11, 4, 4, 3>; };
 template <int TL> struct JoinLen<TL, 12> { using S = JoinShape<TL, 12, 4, 4, 4>; };
 template <int TL> struct JoinLen<TL, 13> { using S = JoinShape<TL, 13, 5, 4, 4>; };
-template <int LOGN> struct JoinPair;
-template <> struct JoinPair<15> : JoinPairOf<Join128<12>, Join256<12>> {};
-template <> struct JoinPair<16> : JoinPairOf<Join256<12>, Join256<12>> {};
-template <> struct JoinPair<17> : JoinPairOf<Join256<13>, Join512<13>> {};
-template <> struct JoinPair<18> : JoinPairOf<Join512<13>, Join512<13>> {};
-template <> struct JoinPair<19> : JoinPairOf<Join512<13>, Join1024<13>> {};
-template <> struct JoinPair<20> : JoinPairOf<Join1024<14>, Join1024<14>> {};
+// TL: log2 of the tile (join_tile_log).
+template <int LOGN, int TL> struct JoinPair;
+template <int TL> struct JoinPair<15, TL> : JoinPairOf<Join128<TL>, Join256<TL>> {};
+template <int TL> struct JoinPair<16, TL> : JoinPairOf<Join256<TL>, Join256<TL>> {};
+template <int TL> struct JoinPair<17, TL> : JoinPairOf<Join256<TL>, Join512<TL>> {};
+template <int TL> struct JoinPair<18, TL> : JoinPairOf<Join512<TL>, Join512<TL>> {};
+template <int TL> struct JoinPair<19, TL> : JoinPairOf<Join512<TL>, Join1024<TL>> {};
+template <int TL> struct JoinPair<20, TL> : JoinPairOf<Join1024<TL>, Join1024<TL>> {};
 constexpr int kJoinMinLog = 15, kJoinMaxLog = 20;
-// log2 of the tile, and of the blocks per SM it allows (512 threads of 32
-// elements in all).
-GB_HD constexpr int join_tile_log(int logn) { return logn <= 16 ? 12 : logn <= 19 ? 13 : 14; }
+// Tiles of a transform of 2^logn points in a batch of `elems` elements.  With
+// work for several tiles per block, the tile is the smallest whose row segments
+// are 128 bytes wide (64 in one of the two passes of 2^17 .. 2^19); with less,
+// smaller tiles spread it over more SMs (2^21 elements, 8192 against 4096 per
+// tile: 2^17 19.8 and 18.5 us, 2^18 20.5 and 20.1, 2^19 19.8 and 20.7).
+GB_HD constexpr int join_tile_log(int logn, int64_t elems) {
+  return elems < int64_t(1) << 22 ? (logn <= 18 ? 12 : 13) : logn <= 16 ? 12 : logn <= 19 ? 13 : 14;
+}
+// log2 of the blocks per SM (512 threads of 32 elements in all).
 GB_HD constexpr int join_blocks_log(int tile_log) { return 14 - tile_log; }
-// Frames: rows of 2^lc, columns of 2^lr.
-GB_HD constexpr bool join_frame(int lr, int lc) {
-  return lr >= 4 && lr <= 11 && lc >= 4 && lc <= 13;
+// Do such transforms run joined?  Measured against two launches: always faster
+// (2^17 x 1 13.8 -> 10.3 us, 2^18 x 2 16.5 -> 12.6; 2^15 alike) but for a little
+// over one wave of first-pass tiles, where the second pass then starts late
+// (2^20 elements: 2^16 14.4 -> 16.5 us, 2^20 18.4 -> 19.8; 2^18 18.0 -> 17.5).
+GB_HD constexpr bool join_transform(int logn, int64_t elems) {
+  return logn >= kJoinMinLog && logn <= kJoinMaxLog &&
+         (elems >= int64_t(1) << 21 || logn == 18 || (logn > 15 && elems < int64_t(1) << 20));
+}
+
+// Frames: rows of 2^lc, columns of 2^lr, `elems` elements in all.  The same
+// band is excluded where the passes had fast kernels (256 rows and fewer of 256
+// elements and more: 16 x 1024 x 64 15.9 -> 16.7 us); 1.1 to 2.6 times faster
+// elsewhere (64 x 64 x 64 20.7 -> 10.4 us).
+GB_HD constexpr bool join_frame(int lr, int lc, int64_t elems) {
+  return lr >= 4 && lr <= 11 && lc >= 4 && lc <= 13 &&
+         (lr > 8 || lc < 8 || elems < int64_t(1) << 20 || elems >= int64_t(1) << 21);
 }
 GB_HD constexpr int join_frame_tile_log(int lr, int lc) { return lr <= 8 && lc <= 12 ? 12 : 13; }
-// Fewest elements a plan joins its passes for.
-constexpr int64_t kJoinMinElems = int64_t(1) << 21;
 
 // ------------------------------------------------------------- the order --
 // Tiles are handed out in one order to whichever block asks next (a counter),

@@ -181,11 +181,10 @@ __device__ __forceinline__ void join_stages(cf (&v)[kJoinR], cf* sm, const cf* t
 }
 
 // Four-step transforms of 2^LOGN points.
-template <int LOGN, bool INV>
-__global__ void __launch_bounds__(JoinPair<LOGN>::kThreads + 32,
-                                  1 << join_blocks_log(JoinPair<LOGN>::kTileLog))
+template <int LOGN, int TL, bool INV>
+__global__ void __launch_bounds__((1 << TL) / kJoinR + 32, 1 << join_blocks_log(TL))
 joined_pass(const cf* in, cf* out, cf* work, const __grid_constant__ JoinDesc d) {
-  using PR = JoinPair<LOGN>;
+  using PR = JoinPair<LOGN, TL>;
   using B1 = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>;
   using B2 = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>;
   constexpr int T = PR::kThreads;
@@ -330,19 +329,21 @@ joined_frames(const cf* in, cf* out, const __grid_constant__ JoinDesc d) {
   });
 }
 
-template <int LOGN>
-inline void joined_fn(bool inv, JoinedLaunch& j) {
-  using PR = JoinPair<LOGN>;
+template <int LOGN, int TL>
+inline bool joined_fn(bool inv, JoinedLaunch& j) {
+  using PR = JoinPair<LOGN, TL>;
   using B1 = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>;
   using B2 = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>;
-  j.fn = inv ? (const void*)joined_pass<LOGN, true> : (const void*)joined_pass<LOGN, false>;
+  j.fn = inv ? (const void*)joined_pass<LOGN, TL, true> : (const void*)joined_pass<LOGN, TL, false>;
   j.smem = ((B1::kSlots > B2::kSlots ? B1::kSlots : B2::kSlots) + 2 * PR::kSteps) * sizeof(cf);
   j.block = PR::kThreads + 32;
-  j.d.o.tpt_log = LOGN - PR::kTileLog;
+  j.d.o.tpt_log = LOGN - TL;
+  j.tile_log = TL;
   j.n1 = PR::kN1;
   j.n2 = PR::kN2;
   j.g1 = PR::kG1;
   j.box_rows = PR::kN1 < 256 ? PR::kN1 : 256;
+  return true;
 }
 
 // Shared memory of the frame kernels: the largest tile of their bodies.

@@ -1,14 +1,14 @@
-// Joined two-pass kernels of 2^15 .. 2^18 points (joined.cuh).
+// Joined kernels of transforms of 2^15 .. 2^17 points (joined.cuh).
 #include "joined.cuh"
 
 namespace gbfft {
 
-bool joined_kernel_a(int logn, bool inv, JoinedLaunch& j) {
-  switch (logn) {
-    case 15: joined_fn<15>(inv, j); return true;
-    case 16: joined_fn<16>(inv, j); return true;
-    case 17: joined_fn<17>(inv, j); return true;
-    case 18: joined_fn<18>(inv, j); return true;
+bool joined_kernel_a(int logn, int tile_log, bool inv, JoinedLaunch& j) {
+  switch (logn * 100 + tile_log) {
+    case 1512: return joined_fn<15, 12>(inv, j);
+    case 1612: return joined_fn<16, 12>(inv, j);
+    case 1712: return joined_fn<17, 12>(inv, j);
+    case 1713: return joined_fn<17, 13>(inv, j);
     default: return false;
   }
 }

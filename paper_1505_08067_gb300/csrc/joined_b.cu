@@ -1,17 +1,20 @@
-// Joined two-pass kernels of 2^19 and 2^20 points (joined.cuh), and the launch.
+// Joined two-pass kernels of 2^18 .. 2^20 points (joined.cuh), and the launch.
 #include <algorithm>
 
 #include "joined.cuh"
 
 namespace gbfft {
 
-bool joined_kernel_a(int logn, bool inv, JoinedLaunch& j);
+bool joined_kernel_a(int logn, int tile_log, bool inv, JoinedLaunch& j);
 void joined_frames_kernel(int tile_log, bool inv, JoinedLaunch& j);
 
-static bool joined_kernel_b(int logn, bool inv, JoinedLaunch& j) {
-  switch (logn) {
-    case 19: joined_fn<19>(inv, j); return true;
-    case 20: joined_fn<20>(inv, j); return true;
+static bool joined_kernel_b(int logn, int tile_log, bool inv, JoinedLaunch& j) {
+  switch (logn * 100 + tile_log) {
+    case 1812: return joined_fn<18, 12>(inv, j);
+    case 1813: return joined_fn<18, 13>(inv, j);
+    case 1913: return joined_fn<19, 13>(inv, j);
+    case 2013: return joined_fn<20, 13>(inv, j);
+    case 2014: return joined_fn<20, 14>(inv, j);
     default: return false;
   }
 }
@@ -28,17 +31,18 @@ static cudaError_t prepare(int sm_count, JoinedLaunch* j) {
   return cudaSuccess;
 }
 
-cudaError_t prepare_joined(int logn, bool inv, int sm_count, JoinedLaunch* j) {
-  if (!joined_kernel_a(logn, inv, *j) && !joined_kernel_b(logn, inv, *j))
+cudaError_t prepare_joined(int logn, int tile_log, bool inv, int sm_count, JoinedLaunch* j) {
+  if (!joined_kernel_a(logn, tile_log, inv, *j) && !joined_kernel_b(logn, tile_log, inv, *j))
     return cudaErrorInvalidValue;
   return prepare(sm_count, j);
 }
 
-cudaError_t prepare_joined_frames(int lr, int lc, bool inv, int sm_count, JoinedLaunch* j) {
-  if (!join_frame(lr, lc)) return cudaErrorInvalidValue;
-  const int tl = join_frame_tile_log(lr, lc);
+cudaError_t prepare_joined_frames(int lr, int lc, int tl, bool inv, int sm_count,
+                                  JoinedLaunch* j) {
+  if (!join_frame(lr, lc, 0) || tl != join_frame_tile_log(lr, lc)) return cudaErrorInvalidValue;
   joined_frames_kernel(tl, inv, *j);
   j->frames = true;
+  j->tile_log = tl;
   j->d.lr = lr;
   j->d.lc = lc;
   j->d.o.tpt_log = std::max(0, lr + lc - tl);
@@ -52,8 +56,8 @@ cudaError_t launch_joined(const JoinedLaunch& j, int64_t batch, const void* in, 
   d.o.nb = batch;
   if (j.frames) {
     d.total = batch << (d.lr + d.lc);
-    const int tl = join_frame_tile_log(d.lr, d.lc);
-    d.o.nb = (d.total + (int64_t(1) << (tl + d.o.tpt_log)) - 1) >> (tl + d.o.tpt_log);
+    const int unit = j.tile_log + d.o.tpt_log;
+    d.o.nb = (d.total + (int64_t(1) << unit) - 1) >> unit;
     d.mapped = ((uintptr_t)in & 15) == 0;
   } else {
     d.mapped = encode_rows_map(in, j.n2, batch * j.n1, j.g1, j.box_rows, d.tmap_in);

@@ -31,13 +31,15 @@ struct JoinedLaunch {
   int max_grid = 0;          // resident blocks
   int block = 0;
   size_t smem = 0;
+  int tile_log = 0;
   int n1 = 0, n2 = 0, g1 = 0, box_rows = 0;
   JoinDesc d{};
 };
-// Kernel for transforms of 2^logn, or frames of 2^lr x 2^lc, its opt-in shared
-// memory, resident blocks and tiles per unit.
-cudaError_t prepare_joined(int logn, bool inverse, int sm_count, JoinedLaunch* j);
-cudaError_t prepare_joined_frames(int lr, int lc, bool inverse, int sm_count, JoinedLaunch* j);
+// Kernel for transforms of 2^logn, or frames of 2^lr x 2^lc, in tiles of
+// 2^tile_log, its opt-in shared memory, resident blocks and tiles per unit.
+cudaError_t prepare_joined(int logn, int tile_log, bool inverse, int sm_count, JoinedLaunch* j);
+cudaError_t prepare_joined_frames(int lr, int lc, int tile_log, bool inverse, int sm_count,
+                                  JoinedLaunch* j);
 // `batch` transforms or frames; `work`: the ring of a four-step plan.
 cudaError_t launch_joined(const JoinedLaunch& j, int64_t batch, const void* in, void* out,
                           void* work, cudaStream_t st);

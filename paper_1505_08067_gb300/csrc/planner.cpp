@@ -211,13 +211,13 @@ static PassSpec contiguous_pass(int logL, int64_t batch, int64_t units_per_batch
 // per sub-batch; 2D: frames) run as one launch of tiles of 2^tile_log, and in
 // what order (fft_join.h)?
 static void plan_joined(PlanSpec& s, int logE, int tile_log, int64_t batch, const Caps& caps) {
-  if (batch << logE < kJoinMinElems) return;
   const int tpt_log = std::max(0, logE - tile_log);
   const int64_t per_unit = int64_t(1) << std::max(0, tile_log - logE);
   const int64_t units = (batch + per_unit - 1) / per_unit;
   int64_t ring;
   join_plan(units, tpt_log, (int64_t)caps.sm_count << join_blocks_log(tile_log), s.join_lag, ring);
   s.join_ring = (int)ring;
+  s.join_tile_log = tile_log;
   s.joined = true;
 }
 
@@ -486,8 +486,8 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       const int64_t chunk = two_pass_chunk(N);
       s.chunk_batch = batch > chunk ? chunk : 0;
       s.work_elems = std::min(batch, chunk) * N;
-      if (defaults && logN >= kJoinMinLog && logN <= kJoinMaxLog)
-        plan_joined(s, logN, join_tile_log(logN), std::min(batch, chunk), caps);
+      if (defaults && batch > 0 && join_transform(logN, s.work_elems))
+        plan_joined(s, logN, join_tile_log(logN, s.work_elems), std::min(batch, chunk), caps);
     }
   } else {
     const int64_t rows = n[0], cols = n[1];
@@ -527,7 +527,7 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       p.conj_out = inv;
       s.passes.push_back(p);
     }
-    if (defaults && join_frame(lr, lc))
+    if (defaults && batch > 0 && join_frame(lr, lc, batch << (lr + lc)))
       plan_joined(s, lr + lc, join_frame_tile_log(lr, lc), batch, caps);
   }
 

@@ -122,7 +122,7 @@ struct PlanSpec {
   // tiles and the offsets of its twiddle tables w_L^j for the passes' lengths
   bool joined = false;
   int64_t join_lag = 1;
-  int join_ring = 1;
+  int join_ring = 1, join_tile_log = 0;
   int64_t join_tw1 = 0, join_tw2 = 0;
   // six-step plans: the second workspace buffer starts work2_off elements in
   int64_t work2_off = 0;

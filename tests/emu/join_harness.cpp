@@ -126,9 +126,9 @@ void tile(cf* sm, cf* st, const cf* tw, int col0, int logN, First first, Store s
   });
 }
 
-template <int LOGN, bool INV>
+template <int LOGN, int TL, bool INV>
 int64_t run(int64_t nb, int64_t lag, int ring, const cf* in, cf* out) {
-  using PR = JoinPair<LOGN>;
+  using PR = JoinPair<LOGN, TL>;
   using B1 = JoinBody<typename PR::P1, JOIN_FIRST, CheckMem>;
   using B2 = JoinBody<typename PR::P2, JOIN_COLS, CheckMem>;
   g = Ctx{};
@@ -149,7 +149,6 @@ int64_t run(int64_t nb, int64_t lag, int ring, const cf* in, cf* out) {
   g.smem_len = (int)sm.size();
   g.phase_of.assign(sm.size(), -1);
   cf* st = sm.data() + std::max(B1::kSlots, B2::kSlots);
-  static_assert(join_tile_log(LOGN) == PR::kTileLog, "the planner's tile");
   JoinOrder o{nb, LOGN - PR::kTileLog, ring, std::min<int64_t>(lag, nb * PR::kTiles)};
   std::vector<uint32_t> done(2 * ring, 0);
   for (int64_t t = 0; t < join_tickets(o); ++t) {
@@ -251,15 +250,17 @@ int64_t run_frames(int64_t batch, int lr, int lc, const cf* in, cf* out) {
 
 }  // namespace
 
-extern "C" int64_t join_run(int logn, int64_t nb, int inverse, int64_t lag, int ring, const float* in,
+extern "C" int64_t join_run(int logn, int tile_log, int64_t nb, int inverse, int64_t lag, int ring, const float* in,
                             float* out, char* msg, size_t len) {
   const cf* x = reinterpret_cast<const cf*>(in);
   cf* y = reinterpret_cast<cf*>(out);
   int64_t e = -1;
-  switch (logn) {
-#define GB_RUN(L) \
-  case L: e = inverse ? run<L, true>(nb, lag, ring, x, y) : run<L, false>(nb, lag, ring, x, y); break;
-    GB_RUN(15) GB_RUN(16) GB_RUN(17) GB_RUN(18) GB_RUN(19) GB_RUN(20)
+  switch (logn * 100 + tile_log) {
+#define GB_RUN(L, TL) \
+  case L * 100 + TL:  \
+    e = inverse ? run<L, TL, true>(nb, lag, ring, x, y) : run<L, TL, false>(nb, lag, ring, x, y); break;
+    GB_RUN(15, 12) GB_RUN(16, 12) GB_RUN(17, 12) GB_RUN(17, 13) GB_RUN(18, 12) GB_RUN(18, 13)
+    GB_RUN(19, 13) GB_RUN(20, 13) GB_RUN(20, 14)
 #undef GB_RUN
     default: break;
   }
@@ -271,7 +272,7 @@ extern "C" int64_t join_run_frames(int64_t batch, int lr, int lc, int inverse, c
                                    float* out, char* msg, size_t len) {
   const cf* x = reinterpret_cast<const cf*>(in);
   cf* y = reinterpret_cast<cf*>(out);
-  if (!join_frame(lr, lc)) return -1;
+  if (!join_frame(lr, lc, 0)) return -1;
   const int64_t e = join_frame_tile_log(lr, lc) == 12
                         ? (inverse ? run_frames<12, true>(batch, lr, lc, x, y) : run_frames<12, false>(batch, lr, lc, x, y))
                         : (inverse ? run_frames<13, true>(batch, lr, lc, x, y) : run_frames<13, false>(batch, lr, lc, x, y));

@@ -26,24 +26,26 @@ def joined():
         os.replace(tmp, lib)
     f = ctypes.CDLL(lib)
     f.join_run.restype = f.join_run_frames.restype = ctypes.c_int64
-    f.join_run.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int, ctypes.c_int64, ctypes.c_int,
-                           ctypes.c_void_p, ctypes.c_void_p, ctypes.c_char_p, ctypes.c_size_t]
+    f.join_run.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int64, ctypes.c_int, ctypes.c_int64,
+                           ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_char_p, ctypes.c_size_t]
     f.join_run_frames.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                   ctypes.c_void_p, ctypes.c_void_p, ctypes.c_char_p, ctypes.c_size_t]
     return f
 
 
-# one transform, a ring that is reused, a lag of several transforms, no reuse
-# (lag in tiles: 8 to 64 per transform)
-@pytest.mark.parametrize("logn,batch,lag,ring", [(15, 7, 19, 4), (15, 1, 40, 1), (16, 3, 16, 2),
-                                                 (17, 3, 33, 3), (18, 3, 32, 2), (19, 2, 64, 2),
-                                                 (20, 1, 64, 1)])
+# every transform length in every tile it runs in; one transform, a ring that is
+# reused, a lag of several transforms, no reuse (lag in tiles: 8 to 128 a transform)
+@pytest.mark.parametrize("logn,tile,batch,lag,ring",
+                         [(15, 12, 7, 19, 4), (15, 12, 1, 40, 1), (16, 12, 3, 16, 2),
+                          (17, 12, 1, 32, 1), (17, 13, 3, 33, 4), (18, 12, 1, 64, 1),
+                          (18, 13, 3, 32, 2), (19, 13, 2, 64, 2), (20, 13, 1, 128, 1),
+                          (20, 14, 1, 64, 1)])
 @pytest.mark.parametrize("direction", [-1, 1])
-def test_joined(oracle, joined, logn, batch, lag, ring, direction):
+def test_joined(oracle, joined, logn, tile, batch, lag, ring, direction):
     x = synth.uniform(60 + logn, batch, 2 ** logn)
     y = np.zeros_like(x)
     msg = ctypes.create_string_buffer(256)
-    n = joined.join_run(logn, batch, int(direction > 0), lag, ring, x.ctypes.data, y.ctypes.data, msg, 256)
+    n = joined.join_run(logn, tile, batch, int(direction > 0), lag, ring, x.ctypes.data, y.ctypes.data, msg, 256)
     assert n == 0, msg.value.decode()
     assert np.max(oracle.rel_l2(y, oracle.fft(x, direction))) <= 1e-6 * logn
 

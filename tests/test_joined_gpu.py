@@ -16,8 +16,9 @@ def _check(oracle, y, x_np, idx, direction, logn):
     assert np.max(oracle.rel_l2(y[torch.from_numpy(idx).cuda()].cpu().numpy(), ref)) <= 1e-6 * logn
 
 
-@pytest.mark.parametrize("logn,batch", [(15, 64), (15, 391), (16, 193), (17, 16), (17, 75), (18, 8),
-                                        (18, 39), (19, 4), (19, 17), (20, 2), (20, 9)])
+@pytest.mark.parametrize("logn,batch", [(15, 64), (15, 391), (16, 7), (16, 193), (17, 1),
+                                        (17, 16), (17, 75), (18, 1), (18, 4), (18, 39), (19, 1),
+                                        (19, 4), (19, 17), (20, 2), (20, 3), (20, 9)])
 @pytest.mark.parametrize("direction", [-1, 1])
 def test_joined(gb, oracle, logn, batch, direction):
     n = 2 ** logn
@@ -41,7 +42,7 @@ def test_joined(gb, oracle, logn, batch, direction):
         assert torch.equal(first, x)
 
 
-@pytest.mark.parametrize("logn,batch", [(15, 63), (20, 1), (21, 2)])
+@pytest.mark.parametrize("logn,batch", [(15, 1), (15, 63), (16, 16), (20, 1), (21, 2)])
 def test_not_joined(gb, logn, batch):
     with gb.Plan(2 ** logn, batch) as p:
         assert p.describe()["joined"] == 0 and p.launch_count == 2
@@ -79,7 +80,8 @@ def test_two_plans_on_two_streams(gb, oracle):
         assert all(torch.equal(a, b) for a, b in zip(want, got))
 
 
-@pytest.mark.parametrize("shape,batch", [((16, 16), 8193), ((32, 64), 1031), ((64, 128), 257),
+@pytest.mark.parametrize("shape,batch", [((16, 16), 1), ((16, 16), 8193), ((64, 64), 3),
+                                         ((1024, 16), 1), ((32, 64), 1031), ((64, 128), 257),
                                          ((512, 16), 257), ((256, 8192), 1), ((16, 4096), 33),
                                          ((32, 2048), 35), ((128, 32), 513), ((1024, 512), 5),
                                          ((2048, 16), 65), ((2048, 2048), 1), ((256, 256), 33)])
@@ -110,7 +112,7 @@ def test_joined_frames(gb, oracle, shape, batch, direction):
     assert np.max(oracle.rel_l2(got, ref)) <= 1e-6 * np.log2(n)
 
 
-@pytest.mark.parametrize("shape,batch", [((512, 16), 255), ((8, 4096), 80), ((4096, 512), 1),
+@pytest.mark.parametrize("shape,batch", [((8, 4096), 80), ((256, 256), 16), ((4096, 512), 1),
                                          ((64, 16384), 3), ((4096, 8192), 1)])
 def test_frames_not_joined(gb, shape, batch):
     with gb.Plan(shape, batch) as p:
