@@ -366,7 +366,7 @@ fft_status_t fft_plan_workspace_bytes(fft_plan_t plan, size_t* bytes) {
 fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches) {
   if (!plan_ok(plan)) return fail(FFT_ERR_BAD_PLAN, "null or destroyed plan");
   if (!launches) return fail(FFT_ERR_INVALID_ARG, "launches is null");
-  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined ? 1 : (int)plan->spec.passes.size();
+  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined ? 1 : plan->spec.tc_cols ? 2 : (int)plan->spec.passes.size();
   return FFT_OK;
 }
 

@@ -87,6 +87,47 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
 cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
                         unsigned* counters, JoinedLaunch* j) {
   const int l0 = s.passes[0].logL, l1 = s.passes[1].logL;
+  if (s.tc_cols) {
+    // the column forms of the two row passes (pass 1 and 3 of the five)
+    const int n = s.passes.size(), logN = s.passes[1].logL + s.passes[3].logL;
+    for (int h = 0; h < 2; ++h) {
+      const PassSpec& p = s.passes[1 + 2 * h];
+      PassLaunch l = launches[1 + 2 * h];
+      l.fn = h ? resolve_umma_cols2(p.logL, p.tc_prec, p.io16)
+               : resolve_umma_cols1(p.logL, p.tc_prec, p.io16);
+      if (!l.fn) return cudaErrorInvalidDeviceFunction;
+      cudaError_t e = prepare_launch(l);
+      if (e != cudaSuccess) return e;
+      int per_sm = 0;
+      e = resident_blocks(l.fn, l.block, l.smem, umma_tmem_cols(p.logL), &per_sm);
+      if (e != cudaSuccess) return e;
+      l.ctas_per_sm = per_sm;
+      l.persistent_grid = std::max(per_sm, 1) * caps.sm_count;
+      l.d.epi_logN = logN;
+      l.d.conj_in = h == 0 && s.direction == FFT_INVERSE;
+      l.d.conj_out = h == 1 && s.direction == FFT_INVERSE;
+      launches[n + h] = l;
+    }
+  }
+  return cudaSuccess;
+}
+
+// The two column launches of a six-step plan for nb transforms.
+static cudaError_t enqueue_tc_cols(const PlanSpec& s, const PassLaunch* launches, const void* in,
+                                   void* out, void* work, int64_t nb, cudaStream_t st) {
+  for (int h = 0; h < 2; ++h) {
+    PassLaunch l = launches[s.passes.size() + h];
+    const PassSpec& p = s.passes[1 + 2 * h];
+    const int logN = l.d.epi_logN, le = logN - p.logL;
+    l.d.tiles = nb << (logN - 12);  // tiles of 4096 elements
+    l.d.count_inner = nb << le;
+    l.grid = (int)std::min<int64_t>(l.persistent_grid, l.d.tiles);
+    if (h == 0)
+      encode_tc_cols_map(l.d, in, nb << p.logL, le, elem_bytes(s.precision), 1 << (12 - p.logL),
+                         std::min(1 << p.logL, 256));
+    const cudaError_t e = launch_pass(l, h ? work : in, h ? out : work, st);
+    if (e != cudaSuccess) return e;
+  }
   const bool inv = s.direction == FFT_INVERSE;
   const cudaError_t e = s.dims == 2 ? prepare_joined_frames(l1, l0, s.join_tile_log, inv,
                                                             caps.sm_count, j)
@@ -152,6 +193,7 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
     return b == BUF_IN ? const_cast<void*>(in) : b == BUF_OUT ? out : b == BUF_WORK2 ? work2 : work;
   };
   for (int i = 0; i < s.passes.size(); ++i) {
+  if (s.tc_cols && work) return enqueue_tc_cols(s, launches, in, out, work, nb, st);
     const PassSpec& p = s.passes[i];
     const void* src = buf(p.src);
     void* dst = buf(p.dst);

@@ -125,17 +125,19 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 bool encode_rows_map(const void* p, int64_t cols, int64_t rows, int box_cols, int box_rows,
-                     unsigned char (&map)[128]) {
+                     unsigned char (&map)[128], int esz) {
   if ((uintptr_t)p & 15) return false;
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
   CUtensorMap m;
   static_assert(sizeof(CUtensorMap) == sizeof(map), "tensor map size");
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)cols * 8};
+  const cuuint64_t strides[1] = {(cuuint64_t)cols * esz};
   const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
   const cuuint32_t elem_strides[2] = {1, 1};
-  if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void*>(p), dims, strides, box,
+  const CUtensorMapDataType type =
+      esz == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32 : CU_TENSOR_MAP_DATA_TYPE_UINT64;
+  if (enc(&m, type, 2, const_cast<void*>(p), dims, strides, box,
           elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return false;
@@ -180,6 +182,11 @@ cudaError_t launch_staged(const StagedLaunch& s, const PassDesc& d, const void* 
   }
   k<<<s.grid, s.block, s.smem, st>>>(static_cast<const cf*>(in), static_cast<cf*>(out), dm);
   return cudaGetLastError();
+}
+
+void encode_tc_cols_map(PassDesc& d, const void* in, int64_t rows, int le, int esz, int cols,
+                        int box_rows) {
+  d.tmap_in_ok = encode_rows_map(in, int64_t(1) << le, rows, cols, box_rows, d.tmap_in, esz);
 }
 
 cudaError_t prepare_launch(PassLaunch& p) {

@@ -45,8 +45,9 @@ cudaError_t launch_joined(const JoinedLaunch& j, int64_t batch, const void* in, 
                           void* work, cudaStream_t st);
 // Tensor map (128 bytes) over `rows` rows of `cols` complex64 elements at `p`,
 // boxes of box_cols x box_rows; false if `p` or the driver does not allow it.
+// (esz: bytes per element, 8 or 4)
 bool encode_rows_map(const void* p, int64_t cols, int64_t rows, int box_cols, int box_rows,
-                     unsigned char (&map)[128]);
+                     unsigned char (&map)[128], int esz = 8);
 
 // Job table of a coalesced launch (see stockham_grouped): up to kMaxGroup jobs
 // of one contiguous single-pass shape, each with its own buffers.
@@ -122,6 +123,14 @@ cudaError_t resident_blocks(const void* fn, int block, size_t smem, int tmem_col
 // The tcgen05 form of the FP16 class with complex32 input and output.
 const void* resolve_umma_c32(int logL, size_t* smem);
 // The kernel of a tensor-core pass of the given variant (0 tcgen05, 1 warp MMA);
+// The tcgen05 column forms (first and second pass of four-step plans) for
+// lengths 2^7 .. 2^10; io16: complex32.
+const void* resolve_umma_cols1(int logL, int prec, int io16);
+const void* resolve_umma_cols2(int logL, int prec, int io16);
+// Tensor map of a first pass's input (d.tmap_in; sets d.tmap_in_ok): `rows`
+// rows of 2^le elements of `esz` bytes, boxes of `cols` x `box_rows`.
+void encode_tc_cols_map(PassDesc& d, const void* in, int64_t rows, int le, int esz, int cols,
+                        int box_rows);
 // io16: complex32 input and output (tcgen05, FP16 only).
 inline const void* resolve_tc_pass(int logL, int prec, int variant, int io16 = 0) {
   size_t sm = 0;

@@ -407,6 +407,7 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
           t.dst = dst;
           return t;
         };
+        s.tc_cols = tc_columns(logN) && !o.generic;
         PassSpec f1 = tc_pass(l1, N2), f2 = tc_pass(l2, N1);
         f1.src = f1.dst = BUF_WORK;
         f2.src = f2.dst = BUF_WORK2;
@@ -643,6 +644,7 @@ std::string describe(const PlanSpec& s) {
       << (p.kind == PASS_FFT ? "fft" : p.kind == PASS_COPY ? "copy" : "transpose") << "\"";
     if (p.kind == PASS_TRANSPOSE)
       o << ",\"rows\":" << p.tr_rows << ",\"cols\":" << p.tr_cols << ",\"twiddle_logN\":"
+    << ",\"tc_columns\":" << (s.tc_cols ? 1 : 0)
         << p.tr_logN << ",\"io16\":" << p.io16;
     if (p.kind == PASS_FFT) {
       o << ",\"L\":" << (1 << p.logL) << ",\"R\":" << p.R << ",\"G\":" << p.G

@@ -40,7 +40,7 @@ using Sched = SmallVec<int, 15>;
 
 enum { BUF_IN = 0, BUF_OUT = 1, BUF_WORK = 2, BUF_WORK2 = 3 };
 enum { PASS_FFT = 0, PASS_COPY = 1, PASS_TRANSPOSE = 2 };
-constexpr int kMaxPasses = 6;
+constexpr int kMaxPasses = 8;  // and launches (exec.cpp: a six-step plan's two column launches follow its five)
 
 struct Caps {
   int sm_count = 152;
@@ -125,6 +125,8 @@ struct PlanSpec {
   int join_ring = 1, join_tile_log = 0;
   int64_t join_tw1 = 0, join_tw2 = 0;
   // six-step plans: the second workspace buffer starts work2_off elements in
+  // six-step plans that execute as two tensor-core column passes instead
+  bool tc_cols = false;
   int64_t work2_off = 0;
   fft_status_t status = FFT_OK;
   char error[256] = {0};

@@ -26,6 +26,10 @@
 // reads finish (tcgen05.wait::ld) before the barrier after which the next
 // stage overwrites the accumulators.
 //
+// The column forms (MODE 1 and 2, UmmaBody) are the two passes of four-step
+// plans of 2^15 .. 2^20 points: tiles of adjacent columns, staged by tensor-map
+// boxes where contiguous tiles are staged by one bulk copy.
+//
 // Every wait is bounded: a give-up sets the pass's status word, waits (again
 // bounded) for the UMMAs and the staging copy in flight, frees the tensor
 // memory and returns.
@@ -199,12 +203,12 @@ struct UmmaStagedMem : Base {
   }
 };
 
-template <int LOGL, int PREC, bool H = false>
+template <int LOGL, int PREC, bool H = false, int MODE = 0>
 struct Umma {
   using G = UmmaGeo<LOGL>;
   using Mem = std::conditional_t<H, UmmaDevMemH, UmmaDevMem>;
-  using Body = UmmaBody<LOGL, PREC, Mem>;
-  using BodyS = UmmaBody<LOGL, PREC, UmmaStagedMem<Mem>>;  // loader from the staging buffer
+  using Body = UmmaBody<LOGL, PREC, Mem, MODE>;
+  using BodyS = UmmaBody<LOGL, PREC, UmmaStagedMem<Mem>, MODE>;  // loader from the staging buffer
   static constexpr int P = Body::P;
   static constexpr bool SPLIT = Body::SPLIT;
   static constexpr int SMEM = (SPLIT ? 2 : 1) * G::A_BYTES + 2 * G::B_BYTES + 16;
@@ -235,13 +239,13 @@ struct Umma {
   template <int t>
   static __device__ __forceinline__ void epilogue(const PassDesc& d, cf* gout, int valid,
                                                   uint32_t tmem, uint32_t a_hi, uint32_t a_lo,
-                                                  int warp, int lane) {
+                                                  int warp, int lane, int col0) {
     const int q = warp & 3;
 #pragma unroll 1
     for (int rb = warp >> 2; rb < G::RB; rb += G::NWARP / 4) {
       const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + 32u * rb;
       const int m = rb * 128 + q * 32 + lane;
-      typename Body::RowPart rp = Body::template row_part<t>(d, m);
+      typename Body::RowPart rp = Body::template row_part<t>(d, m, col0);
       uint32_t r[16];
       tmem_ld16(ta, r);  // outputs 0..7
       Body::template epilogue_part<t, 0, 8>(d, gout, valid, rp, r, a_hi, a_lo);
@@ -251,10 +255,10 @@ struct Umma {
   }
 };
 
-template <int LOGL, int PREC, bool H>
+template <int LOGL, int PREC, bool H, int MODE = 0>
 __global__ void __launch_bounds__(32 * umma_warps(LOGL), umma_warps(LOGL) == 16 ? 2 : 4)
 stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc d) {
-  using U = Umma<LOGL, PREC, H>;
+  using U = Umma<LOGL, PREC, H, MODE>;
   using Body = typename U::Body;
   using Mem = typename U::Mem;
   constexpr int ESZ = H ? 4 : 8;  // bytes per stored element
@@ -276,13 +280,37 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
   const uint32_t st_rel = ((b_lo + G::B_BYTES - base) + 16u + 127u) & ~127u;
   const cf* stg = reinterpret_cast<const cf*>(gbase + st_rel);
   uint64_t* lbar = reinterpret_cast<uint64_t*>(gbase + st_rel + kStageBytes);
-  const bool staged = kStaged && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
   // bytes of tile t's valid transforms (every transform L * ESZ >= 64 bytes)
   auto tile_bytes = [&](int64_t t) -> uint32_t {
     const int64_t rem = d.count_inner - t * G::TPT;
     return (uint32_t)((rem < G::TPT ? rem : G::TPT) * G::L * ESZ);
   };
-
+  const bool staged =
+      kStaged && (MODE == 1 ? d.tmap_in_ok != 0 : (reinterpret_cast<uintptr_t>(in) & 15) == 0);
+  // the column forms' tiles (UmmaBody): tiles per transform, log2
+  const int tpt_log = MODE ? d.epi_logN - G::LOGT : 0;
+  // this thread's copy of tile t into the staging buffer
+  auto stage_copy = [&](int64_t t) {
+    if constexpr (MODE == 1) {
+      constexpr int BR = G::L < 256 ? G::L : 256;
+      const uint64_t map = reinterpret_cast<uint64_t>(&d.tmap_in[0]);
+      const int x = (int)(t & ((int64_t(1) << tpt_log) - 1)) * G::TPT;
+      const int y = (int)(t >> tpt_log) << LOGL;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(lbar)),
+                   "r"(kStageBytes)
+                   : "memory");
+#pragma unroll 1
+      for (int j = 0; j < G::L / BR; ++j)
+        asm volatile(
+            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(stg) + j * BR * G::TPT * ESZ),
+            "l"(map), "r"(x), "r"(y + j * BR), "r"(smem_u32(lbar))
+            : "memory");
+    } else {
+      tma_load(const_cast<cf*>(stg), Mem::at(in, t * G::TPT * G::L), tile_bytes(t), lbar);
+    }
+  };
   if (warp == 0) tmem_alloc(tslot, G::TMEM_COLS);
   // the DFT matrix (and its low part) in the B layout, once per CTA
   for (int e = tid; e < 1024; e += G::THREADS) {
@@ -305,13 +333,11 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
   const uint32_t tmem = *tslot;
   // the first tile's copy; `pending`: a copy is in flight that no wait has seen
   bool pending = staged && blockIdx.x < d.tiles;
-  if (pending && tid == 0)
-    tma_load(const_cast<cf*>(stg), Mem::at(in, (int64_t)blockIdx.x * G::TPT * G::L),
-             tile_bytes(blockIdx.x), lbar);
+  if (pending && tid == 0) stage_copy(blockIdx.x);
   uint32_t lparity = 0;
 
   // the loader's parts of this thread's blocks of items
-  const int et = umma_load_item<LOGL>(lane, warp);
+  const int et = umma_load_item<LOGL, MODE>(lane, warp);
   auto parts = [&](int b) { return Body::block_part_of(et, b); };
   auto parts_s = [&](int b) { return U::BodyS::block_part_of(et, b); };
 
@@ -320,9 +346,11 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
   for (int64_t tile = blockIdx.x; tile < d.tiles && !failed; tile += gridDim.x) {
     const int64_t first = tile * G::TPT;
     const int64_t rem = d.count_inner - first;
-    const int valid = rem < G::TPT ? (int)rem : G::TPT;
-    const cf* gin = Mem::at(in, first * G::L);
-    cf* gout = Mem::at(out, first * G::L);
+    const int valid = MODE || rem >= G::TPT ? G::TPT : (int)rem;
+    const int64_t unit = tile >> tpt_log;  // column forms: the transform, and the tile's column
+    const int col0 = MODE ? (int)(tile - (unit << tpt_log)) * G::TPT : 0;
+    const cf* gin = Mem::at(in, MODE == 1 ? (unit << d.epi_logN) + col0 : first * G::L);
+    cf* gout = Mem::at(out, MODE ? (unit << d.epi_logN) + col0 : first * G::L);
     // the tile this CTA takes next, into L2 while this one is computed
     // (whole 16-byte units inside the tile only; none for a ragged tile).
     // Measured per form: it pays for complex32 storage, for tiles of 4096
@@ -331,13 +359,27 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
     // it, DRAM reads were 17% above the tile bytes: prefetched lines read
     // again).
     constexpr bool kPrefetchL2 = H || LOGL < 13 || (U::SPLIT && LOGL == 13);
-    if (kPrefetchL2 && !staged && tid == 0 && tile + gridDim.x < d.tiles) {
+    if (MODE != 1 && kPrefetchL2 && !staged && tid == 0 && tile + gridDim.x < d.tiles) {
       const int64_t nfirst = (tile + gridDim.x) * G::TPT;
       if (nfirst + G::TPT <= d.count_inner) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(Mem::at(in, nfirst * G::L));
         const uintptr_t a16 = (a + 15) & ~uintptr_t(15);
         const uintptr_t e16 = (a + (uintptr_t)G::T * ESZ) & ~uintptr_t(15);
         if (e16 > a16) prefetch_l2(reinterpret_cast<const void*>(a16), (uint32_t)(e16 - a16));
+      }
+    }
+    if constexpr (MODE == 1) {  // the same for columns: boxes of the input's tensor map
+      if (!staged && d.tmap_in_ok && tid == 0 && tile + gridDim.x < d.tiles) {
+        constexpr int BR = G::L < 256 ? G::L : 256;
+        const int64_t t = tile + gridDim.x;
+        const int x = (int)(t & ((int64_t(1) << tpt_log) - 1)) * G::TPT;
+        const int y = (int)(t >> tpt_log) << LOGL;
+#pragma unroll 1
+        for (int j = 0; j < G::L / BR; ++j)
+          asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                           reinterpret_cast<uint64_t>(&d.tmap_in[0])),
+                       "r"(x), "r"(y + j * BR)
+                       : "memory");
       }
     }
     bool direct = true;
@@ -351,13 +393,14 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
         }
         lparity ^= 1u;
         pending = false;
-        if (valid == G::TPT) U::BodyS::template load_tile<true>(d, stg, valid, a_hi, a_lo, parts_s);
-        else U::BodyS::template load_tile<false>(d, stg, valid, a_hi, a_lo, parts_s);
+        if (MODE || valid == G::TPT)
+          U::BodyS::template load_tile<true, true>(d, stg, valid, a_hi, a_lo, parts_s);
+        else U::BodyS::template load_tile<false, true>(d, stg, valid, a_hi, a_lo, parts_s);
         direct = false;
       }
     }
     if (direct) {
-      if (valid == G::TPT) Body::template load_tile<true>(d, gin, valid, a_hi, a_lo, parts);
+      if (MODE || valid == G::TPT) Body::template load_tile<true>(d, gin, valid, a_hi, a_lo, parts);
       else Body::template load_tile<false>(d, gin, valid, a_hi, a_lo, parts);
     }
     fence_smem_async();
@@ -366,9 +409,7 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
     // every thread has read the staging buffer: the next tile's copy
     if (staged && tile + gridDim.x < d.tiles) {
       pending = true;
-      if (tid == 0)
-        tma_load(const_cast<cf*>(stg), Mem::at(in, (tile + gridDim.x) * G::TPT * G::L),
-                 tile_bytes(tile + gridDim.x), lbar);
+      if (tid == 0) stage_copy(tile + gridDim.x);
     }
     auto stage = [&](auto t_) {
       constexpr int t = decltype(t_)::value;
@@ -388,7 +429,7 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
       }
       parity ^= 1u;
       tc05_fence_after();
-      U::template epilogue<t>(d, gout, valid, tmem, a_hi, a_lo, warp, lane);
+      U::template epilogue<t>(d, gout, valid, tmem, a_hi, a_lo, warp, lane, col0);
       fence_smem_async();
       tc05_fence_before();
       __syncthreads();

@@ -46,8 +46,19 @@ namespace gbfft {
 // umma_perm_code(L, t): bit k of the A row index of tensor-core stage t holds
 // bit nibble_k of the butterfly index u = tr * (L/16) + jb (tr: transform
 // within the tile, jb: butterfly within the transform).
-GB_HD constexpr uint64_t umma_perm_code(int logL, int t) {
+//
+// Column forms (mode, see UmmaBody): the last stage puts the transform index
+// (adjacent columns) in the low row bits, so that a warp's stores of one output
+// are runs of adjacent columns; the stage before was chosen for that.
+GB_HD constexpr uint64_t umma_perm_code(int logL, int t, int mode = 0) {
   // nibble k = butterfly-index bit held by row bit k
+  if (mode) {
+    if (logL == 7) return 0x21076543ull;
+    if (logL == 8) return t ? 0x32107654ull : mode == 1 ? 0x73210654ull : 0x76543210ull;
+    if (logL == 9) return t ? 0x43210765ull : mode == 1 ? 0x43021765ull : 0x76054321ull;
+    if (logL == 10) return t ? 0x54321076ull : mode == 1 ? 0x54130762ull : 0x75164302ull;
+    return 0;
+  }
   if (logL == 4) return t == 0 ? 0x76543210ull : 0;
   if (logL == 5) return t == 0 ? 0x76543210ull : 0;
   if (logL == 6) return t == 0 ? 0x76543210ull : 0;
@@ -66,8 +77,17 @@ GB_HD constexpr uint64_t umma_perm_code(int logL, int t) {
 // lane bit k selects.  Work items are tile elements (r0 = 1) or first-stage
 // butterflies (r0 > 1); bits 0 and 1 are always lane bits, so every 32-byte
 // sector a warp load touches is used whole.
-GB_HD constexpr uint32_t umma_load_lanes_code(int logL) {
+// Mode 1 (columns) puts the transform bits there instead: adjacent columns.
+GB_HD constexpr uint32_t umma_load_lanes_code(int logL, int mode = 0) {
   // nibble k = bit of the loader's work item selected by lane bit k
+  if (mode == 1) {
+    if (logL == 7) return 0x87654u;
+    if (logL == 8) return 0xba984u;
+    if (logL == 9) return 0xa9854u;
+    if (logL == 10) return 0x98540u;
+    return 0;
+  }
+  if (mode == 2 && logL == 9) return 0x54210u;
   if (logL == 4) return 0x43210u;
   if (logL == 5) return 0x43210u;
   if (logL == 6) return 0x43210u;
@@ -98,6 +118,19 @@ GB_HD constexpr int umma_staging_bytes(int logL, int eb, bool split) {
   return logL <= 12 && !split ? 128 + 4096 * eb + 16 : 0;
 }
 
+// Do tensor-core plans of 2^logn points (six steps: transposes and row passes)
+// run as two passes over column tiles?  A tile of 4096 elements holds
+// 4096 / L >= 4 adjacent columns for passes of up to 1024 points, whole 32-byte
+// sectors per row (complex32: 16 bytes at 1024 points, still far ahead of five
+// passes); 2048-point passes would leave 16 bytes and 8.
+// What bounds the six steps is memory: five passes, 80 bytes an element, of
+// which the transposes take 60%.  The column forms read and write each element
+// twice; their stages are the ones of the contiguous kernel, which bound them.
+// Measured, 2^25 elements, six steps and now: 2^16 FP16 451 -> 201 us, BF16
+// 452 -> 201, BF16x3 497 -> 231, complex32 322 -> 144; 2^20 462 -> 229,
+// 460 -> 227, 515 -> 332, 331 -> 212.
+GB_HD constexpr bool tc_columns(int logn) { return logn >= 15 && logn <= 20; }
+
 template <int LOGL>
 struct UmmaGeo {
   static_assert(LOGL >= 4 && LOGL <= 14, "tensor-core lengths are 2^4 .. 2^14");
@@ -125,18 +158,18 @@ struct UmmaGeo {
 };
 
 // Bit permutation of the A rows of stage t: row -> butterfly, butterfly -> row.
-template <int LOGL>
+template <int LOGL, int MODE = 0>
 GB_HD int umma_u_of_row(int t, int m) {
   int u = 0;
-  const uint64_t c = umma_perm_code(LOGL, t);
+  const uint64_t c = umma_perm_code(LOGL, t, MODE);
 GB_UNROLL
   for (int k = 0; k < UmmaGeo<LOGL>::ROWB; ++k) u |= ((m >> k) & 1) << ((c >> (4 * k)) & 15);
   return u;
 }
-template <int LOGL>
+template <int LOGL, int MODE = 0>
 GB_HD int umma_row_of_u(int t, int u) {
   int m = 0;
-  const uint64_t c = umma_perm_code(LOGL, t);
+  const uint64_t c = umma_perm_code(LOGL, t, MODE);
 GB_UNROLL
   for (int k = 0; k < UmmaGeo<LOGL>::ROWB; ++k) m |= ((u >> ((c >> (4 * k)) & 15)) & 1) << k;
   return m;
@@ -198,11 +231,11 @@ GB_HD void umma_next(int t, int u, int o, int& u2, int& i2, int& tw) {
 
 // Work item e of the loader: the tile element (r0 = 1) or the first-stage
 // butterfly (r0 > 1) that lane bits and (warp, iteration) bits select.
-template <int LOGL>
+template <int LOGL, int MODE = 0>
 GB_HD int umma_load_item(int lane, int rest) {
   int e = 0, r = rest;
   int pos = 0;
-  constexpr uint32_t c = umma_load_lanes_code(LOGL);
+  constexpr uint32_t c = umma_load_lanes_code(LOGL, MODE);
 GB_UNROLL
   for (int b = 0; (1 << b) < UmmaGeo<LOGL>::ITEMS; ++b) {
     int k = -1;
@@ -250,7 +283,13 @@ GB_HD void umma_first_target(int e, int o, int& u, int& i, int& tw) {
 // ldtw (twiddle table), sts32 (a 32-bit store at a byte address of the A
 // operands) and kHalfIO (complex32 storage).  a_hi / a_lo are the byte
 // addresses of the two A operands (a_lo only for the split class).
-template <int LOGL, int PREC, class Mem>
+//
+// MODE 0: batches of contiguous transforms.  1 and 2: the passes of a four-step
+// plan (N = N1 N2, x[n1 N2 + n2]).  1: a tile holds adjacent columns n2, read and
+// written as columns of rows of 2^le = N2 elements, the outputs multiplied by
+// the four-step twiddle w_N^{n2 k1}.  2: a tile holds adjacent rows k1, read as
+// rows and written as columns of rows of 2^le = N1 elements.
+template <int LOGL, int PREC, class Mem, int MODE = 0>
 struct UmmaBody {
   using G = UmmaGeo<LOGL>;
   static constexpr int P = PREC == TC_BF16X3 ? TC_BF16 : PREC;
@@ -293,12 +332,12 @@ struct UmmaBody {
   GB_HD static uint32_t off_of(int e) {  // r0 = 1: A-operand offset of tile element e
     int u, i;
     umma_load_target<LOGL>(e, u, i);
-    return umma_aoff(umma_row_of_u<LOGL>(0, u), i);
+    return umma_aoff(umma_row_of_u<LOGL, MODE>(0, u), i);
   }
   GB_HD static void first_of(int e, int o, uint32_t& off, int& i, int& tw) {  // r0 > 1
     int u;
     umma_first_target<LOGL>(e, o, u, i, tw);
-    off = umma_aoff(umma_row_of_u<LOGL>(0, u), i);
+    off = umma_aoff(umma_row_of_u<LOGL, MODE>(0, u), i);
   }
 
   // The parts of block b of CH items of the thread whose item part is et
@@ -312,7 +351,7 @@ struct UmmaBody {
   };
   GB_HD static BlockPart block_part_of(int et, int b) {
     BlockPart p{};
-    p.eb = et | umma_load_item<LOGL>(0, b * CH * G::NWARP);
+    p.eb = et | umma_load_item<LOGL, MODE>(0, b * CH * G::NWARP);
     p.xb = elem_of(p.eb);
     if (G::R0B == 0) p.offb = off_of(p.eb);
     else first_of(p.eb, 0, p.offb, p.ib, p.twb);
@@ -321,46 +360,53 @@ struct UmmaBody {
 
   // FULL: every transform of the tile is valid (no per-item check).
   // parts(b) gives the thread's BlockPart of block b.
-  template <bool FULL, class Parts>
+  // STAGED: gin is the staging buffer (MODE 1: element a of column c at
+  // a * TPT + c, as tensor-map boxes bring it).
+  template <bool FULL, bool STAGED = false, class Parts>
   GB_HD static void load_tile(const PassDesc& d, const cf* gin, int valid, uint32_t a_hi,
                               uint32_t a_lo, const Parts& parts) {
     const bool swap = d.conj_in != 0;
+    // offset of tile element x; the parts of disjoint bits add up
+    const int le = MODE == 1 && !STAGED ? d.epi_logN - LOGL : LOGL == 12 ? 0 : 12 - LOGL;
+    auto at = [&](int x) {
+      return MODE == 1 ? ((x & (G::L - 1)) << le) + (x >> LOGL) : x;
+    };
 #pragma unroll 1
     for (int b = 0; b < KB; ++b) {
       const BlockPart bp = parts(b);
-      const cf* gb = Mem::at(gin, bp.xb);
+      const cf* gb = Mem::at(gin, at(bp.xb));
       if constexpr (Mem::kHalfIO && !LOAD_SCALE && P == TC_FP16 && !SPLIT && G::R0B == 0) {
         // complex32 into an FP16 operand, unscaled: the loaded pair is the
         // operand's pair (swapped for the inverse), no conversion
         uint32_t h[CH];
 GB_UNROLL
         for (int j = 0; j < CH; ++j) {
-          const int ej = umma_load_item<LOGL>(0, j * G::NWARP);
-          h[j] = FULL || tr_of(bp.eb | ej) < valid ? Mem::ldg_pair(gb, ej, swap) : 0u;
+          const int ej = umma_load_item<LOGL, MODE>(0, j * G::NWARP);
+          h[j] = FULL || tr_of(bp.eb | ej) < valid ? Mem::ldg_pair(gb, at(ej), swap) : 0u;
         }
 GB_UNROLL
         for (int j = 0; j < CH; ++j)
-          Mem::sts32(a_hi + (bp.offb ^ off_of(umma_load_item<LOGL>(0, j * G::NWARP))), h[j]);
+          Mem::sts32(a_hi + (bp.offb ^ off_of(umma_load_item<LOGL, MODE>(0, j * G::NWARP))), h[j]);
       } else if (G::R0B == 0) {
         cf v[CH];
 GB_UNROLL
         for (int j = 0; j < CH; ++j) {
-          const int ej = umma_load_item<LOGL>(0, j * G::NWARP);
-          v[j] = FULL || tr_of(bp.eb | ej) < valid ? Mem::ldg_sw(gb, ej, swap) : mk(0.f, 0.f);
+          const int ej = umma_load_item<LOGL, MODE>(0, j * G::NWARP);
+          v[j] = FULL || tr_of(bp.eb | ej) < valid ? Mem::ldg_sw(gb, at(ej), swap) : mk(0.f, 0.f);
         }
 GB_UNROLL
         for (int j = 0; j < CH; ++j)
-          put_a<LOAD_SCALE>(a_hi, a_lo, bp.offb ^ off_of(umma_load_item<LOGL>(0, j * G::NWARP)), v[j]);
+          put_a<LOAD_SCALE>(a_hi, a_lo, bp.offb ^ off_of(umma_load_item<LOGL, MODE>(0, j * G::NWARP)), v[j]);
       } else {
         const cf* tw = d.tw + d.tw_off[1];
 GB_UNROLL
         for (int j = 0; j < CH; ++j) {
-          const int ej = umma_load_item<LOGL>(0, j * G::NWARP);
+          const int ej = umma_load_item<LOGL, MODE>(0, j * G::NWARP);
           const bool ok = FULL || tr_of(bp.eb | ej) < valid;
           cf y[G::R0];
 GB_UNROLL
           for (int q = 0; q < G::R0; ++q)
-            y[q] = ok ? Mem::ldg_sw(gb, elem_of(ej) + q * (G::L / G::R0), swap) : mk(0.f, 0.f);
+            y[q] = ok ? Mem::ldg_sw(gb, at(elem_of(ej) + q * (G::L / G::R0)), swap) : mk(0.f, 0.f);
           if (G::R0 == 2) dft_small<2, 1>(y);
           else if (G::R0 == 4) dft_small<4, 1>(y);
           else dft_pq<2, 4>(y);
@@ -410,17 +456,24 @@ GB_UNROLL
   // c = w^{i' k} and s = w^{i' Ns} = (c s) * conj(c): two table loads per
   // row, then a running product (at most 16 further roundings, ~1e-6).  For
   // FP16, c carries the next stage's exact 1/16.
+  // MODE 1, last stage: w_N^{n2 k1} of output o (k1 = pos + o Ns) likewise, from
+  // the exact angles of the column col0 + tr.
   template <int t>
-  GB_HD static RowPart row_part(const PassDesc& d, int m) {
+  GB_HD static RowPart row_part(const PassDesc& d, int m, int col0 = 0) {
     RowPart rp{};
-    const int u = umma_u_of_row<LOGL>(t, m);
+    const int u = umma_u_of_row<LOGL, MODE>(t, m);
     if (t == G::NTC - 1) {
       rp.tr = u >> G::BPSB;
-      rp.pos = (rp.tr << LOGL) | umma_out_pos(G::ns_log(t), u & ((1 << G::BPSB) - 1), 0);
+      const int pos = umma_out_pos(G::ns_log(t), u & ((1 << G::BPSB) - 1), 0);
+      rp.pos = MODE ? (pos << (d.epi_logN - LOGL)) + rp.tr : (rp.tr << LOGL) | pos;
+      if constexpr (MODE == 1) {
+        rp.run = Mem::rotor((int64_t)(col0 + rp.tr) * pos, d.epi_logN);
+        rp.step = Mem::rotor((int64_t)(col0 + rp.tr) << G::ns_log(t), d.epi_logN);
+      }
     } else {
       int u2, i2;
       umma_next<LOGL>(t, u, 0, u2, i2, rp.tw);
-      rp.off = umma_aoff(umma_row_of_u<LOGL>(t + 1, u2), i2);
+      rp.off = umma_aoff(umma_row_of_u<LOGL, MODE>(t + 1, u2), i2);
       int u2o, i2o, two;
       umma_next<LOGL>(t, 0, 1, u2o, i2o, two);  // output 1's part of the table index
       const cf* tw = d.tw + d.tw_off[ST0 + t + 1];
@@ -453,7 +506,12 @@ GB_UNROLL
           const float sc = (float)(1 << (4 * SCALED_STAGES));
           v = mk(v.x * sc, v.y * sc);
         }
-        Mem::stg_sw(o_base, o << G::ns_log(t), v, swap);
+        if constexpr (MODE == 1) {
+          v = cmul(v, rp.run);
+          rp.run = cmul(rp.run, rp.step);
+        }
+        if constexpr (MODE != 0) Mem::stg_sw(o_base, (o << G::ns_log(t)) << (d.epi_logN - LOGL), v, swap);
+        else Mem::stg_sw(o_base, o << G::ns_log(t), v, swap);
       }
     } else {
 GB_UNROLL
@@ -461,7 +519,7 @@ GB_UNROLL
         const int o = O0 + j;
         int u2o, i2o, two;
         umma_next<LOGL>(t, 0, o, u2o, i2o, two);
-        const uint32_t off = rp.off ^ umma_aoff(umma_row_of_u<LOGL>(t + 1, u2o), i2o);
+        const uint32_t off = rp.off ^ umma_aoff(umma_row_of_u<LOGL, MODE>(t + 1, u2o), i2o);
         cf v = mk(u32_as_f32(r[2 * j]), u32_as_f32(r[2 * j + 1]));
         v = cmul(v, rp.run);               // c * s^o
         rp.run = cmul(rp.run, rp.step);

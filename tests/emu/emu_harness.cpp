@@ -607,9 +607,10 @@ GB_HD uint32_t umma_hw_offset(int m, int k) {
   return (uint32_t)((m / 8) * 512 + (m % 8) * 64 + (((k / 8) ^ ((m % 8) / 2)) & 3) * 16 + (k % 8) * 2);
 }
 
-template <int LOGL, int PREC>
+// MODE 1, 2: the column forms (UmmaBody); a copied tile becomes plain loads.
+template <int LOGL, int PREC, int MODE = 0>
 void run_umma_t(const PassDesc& d, const cf* in, cf* out) {
-  using Body = UmmaBody<LOGL, PREC, UmmaCheckMem>;
+  using Body = UmmaBody<LOGL, PREC, UmmaCheckMem, MODE>;
   using G = UmmaGeo<LOGL>;
   constexpr int P = Body::P;
   constexpr bool SPLIT = Body::SPLIT;
@@ -640,12 +641,15 @@ void run_umma_t(const PassDesc& d, const cf* in, cf* out) {
   for (int64_t tile = 0; tile < d.tiles; ++tile) {
     const int64_t first = tile * G::TPT;
     const int valid = (int)std::min<int64_t>(G::TPT, d.count_inner - first);
-    const cf* gin = in + first * G::L;
-    cf* gout = out + first * G::L;
+    const int tpt_log = MODE ? d.epi_logN - G::LOGT : 0;
+    const int64_t unit = tile >> tpt_log;
+    const int col0 = MODE ? (int)(tile - (unit << tpt_log)) * G::TPT : 0;
+    const cf* gin = in + (MODE == 1 ? (unit << d.epi_logN) + col0 : first * G::L);
+    cf* gout = out + (MODE ? (unit << d.epi_logN) + col0 : first * G::L);
     ++g_umma.phase;
     for (int warp = 0; warp < G::NWARP; ++warp)
       for (int lane = 0; lane < 32; ++lane) {
-        const int et = umma_load_item<LOGL>(lane, warp);
+        const int et = umma_load_item<LOGL, MODE>(lane, warp);
         auto parts = [&](int b) { return Body::block_part_of(et, b); };
         if (valid == G::TPT) Body::template load_tile<true>(d, gin, valid, a_hi, a_lo, parts);
         else Body::template load_tile<false>(d, gin, valid, a_hi, a_lo, parts);
@@ -671,7 +675,7 @@ void run_umma_t(const PassDesc& d, const cf* in, cf* out) {
             const int m = rb * 128 + (warp & 3) * 32 + lane;
             ++row_reads[m];
             // as the kernel: one row part, the row read in two halves
-            typename Body::RowPart rp = Body::template row_part<t>(d, m);
+            typename Body::RowPart rp = Body::template row_part<t>(d, m, col0);
             uint32_t r[16];
             memcpy(r, &D[(size_t)m * 32], sizeof r);
             Body::template epilogue_part<t, 0, 8>(d, gout, valid, rp, r, a_hi, a_lo);
@@ -700,6 +704,44 @@ bool run_umma(int logL, int prec, const PassDesc& d, const cf* in, cf* out) {
   GB_UM(13) GB_UM(14)
 #undef GB_UM
   return false;
+}
+
+// A tensor-core plan above 2^14 as the two column passes it executes as.
+template <int PREC>
+bool run_tc_cols_t(const PlanSpec& s, const cf* tables, int64_t batch, const cf* in, cf* work, cf* out) {
+  const int logN = s.passes[1].logL + s.passes[3].logL;
+  const int64_t E = batch << logN;
+  for (int h = 0; h < 2; ++h) {
+    const PassSpec& p = s.passes[1 + 2 * h];
+    PassDesc d = pass_desc(p, 0, batch, batch);
+    d.tw = tables;
+    d.epi_logN = logN;
+    d.conj_in = h == 0 && s.direction == FFT_INVERSE;
+    d.conj_out = h == 1 && s.direction == FFT_INVERSE;
+    d.tiles = batch << (logN - 12);
+    d.count_inner = batch << (logN - p.logL);
+    const cf* src = h ? work : in;
+    cf* dst = h ? out : work;
+    g.in = src;
+    g.in_len = E;
+    g.out = dst;
+    g.out_len = E;
+    std::vector<uint8_t> hits(E, 0);
+    g.out_hits = &hits;
+    g.tw = tables;
+    g.tw_len = s.table_elems;
+    switch (p.logL * 10 + h) {
+#define GB_UC(LG) \
+  case LG * 10: run_umma_t<LG, PREC, 1>(d, src, dst); break; \
+  case LG * 10 + 1: run_umma_t<LG, PREC, 2>(d, src, dst); break;
+      GB_UC(7) GB_UC(8) GB_UC(9) GB_UC(10)
+#undef GB_UC
+      default: return false;
+    }
+    for (int64_t i = 0; i < E; ++i)
+      if (hits[i] != 1) { err("output element not written exactly once", i); break; }
+  }
+  return true;
 }
 
 template <int LM, int SM>
@@ -929,6 +971,31 @@ int emu_ring_replay(uint64_t seed, int slots, int jobs, int exact, char* msg, si
     }
   }
   return 0;
+}
+
+int64_t emu_tc_cols_run(int64_t n, int64_t batch, int direction, int precision, const float* in_f,
+                        float* out_f, char* msg, size_t msg_len) {
+  static PlanSpec s;
+  Caps caps;
+  make_plan(s, &n, 1, batch, direction, precision, nullptr, caps);
+  g = Ctx{};
+  if (s.status != FFT_OK || !s.tc_cols) {
+    snprintf(msg, msg_len, "no column plan: %s", s.error);
+    return -1;
+  }
+  std::vector<cf> tables(std::max<int64_t>(1, s.table_elems));
+  for (const TwSegment& t : s.tables)
+    for (int64_t j = 0; j < t.count; ++j)
+      tables[t.off + j] = root(t.mode == 0 ? (j / t.r) * (j % t.r) : j * t.mult, t.den);
+  std::vector<cf> work(batch * n);
+  const cf* in = reinterpret_cast<const cf*>(in_f);
+  cf* out = reinterpret_cast<cf*>(out_f);
+  const bool ok = precision == 1   ? run_tc_cols_t<1>(s, tables.data(), batch, in, work.data(), out)
+                  : precision == 2 ? run_tc_cols_t<2>(s, tables.data(), batch, in, work.data(), out)
+                                   : run_tc_cols_t<3>(s, tables.data(), batch, in, work.data(), out);
+  if (!ok) err("no replay for these passes", n);
+  snprintf(msg, msg_len, "%s", g.first_error.c_str());
+  return g.errors;
 }
 
 }  // extern "C"
