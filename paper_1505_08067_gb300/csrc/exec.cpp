@@ -81,12 +81,6 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
     }
     launches[i] = l;
   }
-  return cudaSuccess;
-}
-
-cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
-                        unsigned* counters, JoinedLaunch* j) {
-  const int l0 = s.passes[0].logL, l1 = s.passes[1].logL;
   if (s.tc_cols) {
     // the column forms of the two row passes (pass 1 and 3 of the five)
     const int n = s.passes.size(), logN = s.passes[1].logL + s.passes[3].logL;
@@ -128,6 +122,12 @@ static cudaError_t enqueue_tc_cols(const PlanSpec& s, const PassLaunch* launches
     const cudaError_t e = launch_pass(l, h ? work : in, h ? out : work, st);
     if (e != cudaSuccess) return e;
   }
+  return cudaSuccess;
+}
+
+cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
+                        unsigned* counters, JoinedLaunch* j) {
+  const int l0 = s.passes[0].logL, l1 = s.passes[1].logL;
   const bool inv = s.direction == FFT_INVERSE;
   const cudaError_t e = s.dims == 2 ? prepare_joined_frames(l1, l0, s.join_tile_log, inv,
                                                             caps.sm_count, j)
@@ -187,13 +187,13 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
     if (a == b || a + bytes <= b || b + bytes <= a)
       return launch_joined(*joined, nb, in, out, work, st);
   }
+  if (s.tc_cols && work) return enqueue_tc_cols(s, launches, in, out, work, nb, st);
   // the second workspace buffer of six-step plans
   void* work2 = work ? static_cast<char*>(work) + work2_off * elem_bytes(s.precision) : nullptr;
   auto buf = [&](int b) -> void* {
     return b == BUF_IN ? const_cast<void*>(in) : b == BUF_OUT ? out : b == BUF_WORK2 ? work2 : work;
   };
   for (int i = 0; i < s.passes.size(); ++i) {
-  if (s.tc_cols && work) return enqueue_tc_cols(s, launches, in, out, work, nb, st);
     const PassSpec& p = s.passes[i];
     const void* src = buf(p.src);
     void* dst = buf(p.dst);

@@ -122,7 +122,6 @@ int umma_tmem_cols(int logL);
 cudaError_t resident_blocks(const void* fn, int block, size_t smem, int tmem_cols, int* blocks);
 // The tcgen05 form of the FP16 class with complex32 input and output.
 const void* resolve_umma_c32(int logL, size_t* smem);
-// The kernel of a tensor-core pass of the given variant (0 tcgen05, 1 warp MMA);
 // The tcgen05 column forms (first and second pass of four-step plans) for
 // lengths 2^7 .. 2^10; io16: complex32.
 const void* resolve_umma_cols1(int logL, int prec, int io16);
@@ -131,6 +130,7 @@ const void* resolve_umma_cols2(int logL, int prec, int io16);
 // rows of 2^le elements of `esz` bytes, boxes of `cols` x `box_rows`.
 void encode_tc_cols_map(PassDesc& d, const void* in, int64_t rows, int le, int esz, int cols,
                         int box_rows);
+// The kernel of a tensor-core pass of the given variant (0 tcgen05, 1 warp MMA);
 // io16: complex32 input and output (tcgen05, FP16 only).
 inline const void* resolve_tc_pass(int logL, int prec, int variant, int io16 = 0) {
   size_t sm = 0;

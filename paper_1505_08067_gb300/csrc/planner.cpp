@@ -636,6 +636,7 @@ std::string describe(const PlanSpec& s) {
     << ",\"generic\":" << (s.generic_only ? 1 : 0) << ",\"conv\":" << (s.conv ? 1 : 0)
     << ",\"workspace_bytes\":" << s.work_elems * 8 << ",\"table_elems\":" << s.table_elems
     << ",\"chunk_batch\":" << s.chunk_batch << ",\"joined\":" << (s.joined ? 1 : 0)
+    << ",\"tc_columns\":" << (s.tc_cols ? 1 : 0)
     << ",\"passes\":[";
   for (size_t i = 0; i < s.passes.size(); ++i) {
     const PassSpec& p = s.passes[i];
@@ -644,7 +645,6 @@ std::string describe(const PlanSpec& s) {
       << (p.kind == PASS_FFT ? "fft" : p.kind == PASS_COPY ? "copy" : "transpose") << "\"";
     if (p.kind == PASS_TRANSPOSE)
       o << ",\"rows\":" << p.tr_rows << ",\"cols\":" << p.tr_cols << ",\"twiddle_logN\":"
-    << ",\"tc_columns\":" << (s.tc_cols ? 1 : 0)
         << p.tr_logN << ",\"io16\":" << p.io16;
     if (p.kind == PASS_FFT) {
       o << ",\"L\":" << (1 << p.logL) << ",\"R\":" << p.R << ",\"G\":" << p.G

@@ -124,9 +124,9 @@ struct PlanSpec {
   int64_t join_lag = 1;
   int join_ring = 1, join_tile_log = 0;
   int64_t join_tw1 = 0, join_tw2 = 0;
-  // six-step plans: the second workspace buffer starts work2_off elements in
   // six-step plans that execute as two tensor-core column passes instead
   bool tc_cols = false;
+  // six-step plans: the second workspace buffer starts work2_off elements in
   int64_t work2_off = 0;
   fft_status_t status = FFT_OK;
   char error[256] = {0};
