@@ -5,6 +5,11 @@
 
 namespace gbfft {
 
+// Blocks of a short-line launch: tiles of 4096 elements.
+static int lines_grid(const PassDesc& d, int logL) {
+  return (int)std::min<int64_t>(((d.count_inner << logL) + 4095) >> 12, 0x7fffffff);
+}
+
 cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
                           PassLaunch* launches) {
   for (int i = 0; i < s.passes.size(); ++i) {
@@ -30,6 +35,7 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
         l.specialised = true;
       } else {
         l.fn = resolve_kernel(l.R, l.lmap, l.smap, l.d, s.generic_only, &l.specialised);
+        if (p.line_off >= 0 && resolve_lines(p.logL, &l)) l.grid = lines_grid(l.d, p.logL);
       }
       cudaError_t e = prepare_launch(l);
       if (e != cudaSuccess) return e;
@@ -213,13 +219,16 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
         d.status = l.d.status;
         d.h = l.d.h;
         l.d = d;
-        l.fn = p.tc_prec ? resolve_tc_pass(p.logL, p.tc_prec, p.variant, p.io16)
+        if (!l.lines)
+          l.fn = p.tc_prec ? resolve_tc_pass(p.logL, p.tc_prec, p.variant, p.io16)
                          : resolve_kernel(l.R, l.lmap, l.smap, l.d, s.generic_only, &l.specialised);
         e = prepare_launch(l);
         if (e != cudaSuccess) return e;
         d.l2_prefetch = launches[i].d.l2_prefetch;
         l.d.l2_prefetch = d.l2_prefetch;
-        l.grid = (int)std::min<int64_t>(d.tiles, l.persistent_grid ? l.persistent_grid : 0x7fffffff);
+        l.grid = l.lines ? lines_grid(d, p.logL)
+                         : (int)std::min<int64_t>(d.tiles, l.persistent_grid ? l.persistent_grid
+                                                                              : 0x7fffffff);
       }
       if (l.d.tiles == 0) continue;
       if (l.has_staged && ((uintptr_t)src & 15) == 0) {

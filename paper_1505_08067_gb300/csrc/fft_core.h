@@ -156,6 +156,7 @@ struct PassDesc {
   int32_t nst;         // number of radix stages
   int32_t rlog[15];    // log2 of each stage's radix (1..4)
   int32_t tw_off[15];  // stage s twiddles start at tw + tw_off[s]: [k][i], Ns*r entries
+  int32_t tw_line;     // short lines (lines.cu): w_L^j, j < L, at tw + tw_line
   int32_t G;           // transforms per tile
   int32_t T;           // threads per transform = L / R
   int32_t pitch;       // shared-memory pitch per transform (row layout)

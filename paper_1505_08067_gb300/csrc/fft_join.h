@@ -318,6 +318,7 @@ GB_UNROLL
     }
   }
   // Last stage of a row pass / of a frame's column pass.
+  template <bool INV = false>
   GB_HD static void store_rows(const cf (&v)[R], cf* base, int64_t valid, int tid) {
     constexpr int S = SH::kLast, RR = SH::radix(S), NB = R / RR, Ns = SH::ns(S);
 GB_UNROLL
@@ -327,7 +328,10 @@ GB_UNROLL
       cf* p = base + c * L + jb;
       if (c < valid) {
 GB_UNROLL
-        for (int i = 0; i < RR; ++i) Mem::stw(p, i * Ns, v[q * RR + i]);
+        for (int i = 0; i < RR; ++i) {
+          const cf x = v[q * RR + i];
+          Mem::stw(p, i * Ns, INV ? mk(x.y, x.x) : x);
+        }
       }
     }
   }
@@ -368,8 +372,10 @@ template <int TL> using Join128 = JoinShape<TL, 7, 4, 3>;
 template <int TL> using Join256 = JoinShape<TL, 8, 4, 4>;
 template <int TL> using Join512 = JoinShape<TL, 9, 5, 4>;
 template <int TL> using Join1024 = JoinShape<TL, 10, 5, 5>;
-// Every length a row (2^4 .. 2^13) or column (2^4 .. 2^11) pass of frames has.
+// Every length a row (2^4 .. 2^13) or column (2^4 .. 2^11) pass of frames has,
+// and short lines (2^3 .. 2^10, lines.cu).
 template <int TL, int LOGL> struct JoinLen;
+template <int TL> struct JoinLen<TL, 3> { using S = JoinShape<TL, 3, 1, 2>; };
 template <int TL> struct JoinLen<TL, 4> { using S = JoinShape<TL, 4, 2, 2>; };
 template <int TL> struct JoinLen<TL, 5> { using S = JoinShape<TL, 5, 3, 2>; };
 template <int TL> struct JoinLen<TL, 6> { using S = JoinShape<TL, 6, 3, 3>; };
@@ -402,19 +408,20 @@ GB_HD constexpr int join_blocks_log(int tile_log) { return 14 - tile_log; }
 // Do such transforms run joined?  Measured against two launches: always faster
 // (2^17 x 1 13.8 -> 10.3 us, 2^18 x 2 16.5 -> 12.6; 2^15 alike) but for a little
 // over one wave of first-pass tiles, where the second pass then starts late
-// (2^20 elements: 2^16 14.4 -> 16.5 us, 2^20 18.4 -> 19.8; 2^18 18.0 -> 17.5).
+// (2^20 elements: 2^16 14.4 -> 16.5 us, 2^18 16.5 -> 17.5, 2^20 18.4 -> 19.8).
 GB_HD constexpr bool join_transform(int logn, int64_t elems) {
   return logn >= kJoinMinLog && logn <= kJoinMaxLog &&
-         (elems >= int64_t(1) << 21 || logn == 18 || (logn > 15 && elems < int64_t(1) << 20));
+         (elems >= int64_t(1) << 21 || (logn > 15 && elems < int64_t(1) << 20));
 }
 
 // Frames: rows of 2^lc, columns of 2^lr, `elems` elements in all.  The same
 // band is excluded where the passes had fast kernels (256 rows and fewer of 256
-// elements and more: 16 x 1024 x 64 15.9 -> 16.7 us); 1.1 to 2.6 times faster
-// elsewhere (64 x 64 x 64 20.7 -> 10.4 us).
+// elements and more, and rows of 2048 and more: 16 x 1024 x 64 15.9 -> 16.7 us,
+// 512 x 2048 18.6 -> 19.4); 1.1 to 2.6 times faster elsewhere (64 x 64 x 64
+// 20.7 -> 10.4 us).
 GB_HD constexpr bool join_frame(int lr, int lc, int64_t elems) {
   return lr >= 4 && lr <= 11 && lc >= 4 && lc <= 13 &&
-         (lr > 8 || lc < 8 || elems < int64_t(1) << 20 || elems >= int64_t(1) << 21);
+         ((lr > 8 ? lc < 11 : lc < 8) || elems < int64_t(1) << 20 || elems >= int64_t(1) << 21);
 }
 GB_HD constexpr int join_frame_tile_log(int lr, int lc) { return lr <= 8 && lc <= 12 ? 12 : 13; }
 

@@ -73,6 +73,7 @@ struct PassLaunch {
   size_t smem;      // dynamic shared memory in bytes
   const void* fn = nullptr;  // resolved kernel (specialised or generic)
   bool specialised = false;
+  bool lines = false;        // the short-line kernel (resolve_lines): a tile of 4096 elements per block
   bool has_staged = false;   // a staged kernel exists for this shape (see below)
   int persistent_grid = 0;   // nonzero: grid capped at resident blocks (L2-prefetch variant)
   int ctas_per_sm = 0;       // persistent kernels: resident blocks per SM the grid assumes
@@ -144,6 +145,10 @@ inline const void* resolve_tc_pass(int logL, int prec, int variant, int io16 = 0
 // multiples of 32.
 cudaError_t launch_transpose(const void* in, void* out, int64_t batch, int64_t rows, int64_t cols,
                              int logN, int sign, int h16, int sm_count, cudaStream_t st);
+
+// The short-line kernel of a contiguous pass of 2^logL points (lines.cu): sets
+// fn, block and smem; false if there is none.
+bool resolve_lines(int logL, PassLaunch* l);
 
 // Per-kernel attributes a launch needs (opt-in shared memory); call once after
 // resolving, before the first launch_pass.

@@ -1,0 +1,61 @@
+// Batches of short contiguous transforms (2^3 .. 2^10 points): a tile of 4096
+// elements per 128-thread block as a row pass of fft_join.h, 32 elements and one
+// exchange per thread.
+//
+// Lengths below 256 ran the run-time-parameter kernel, bound by its address
+// arithmetic and, at 16 points (one transform per thread), by loads that touch
+// a 128-byte line per lane.  Here a transform's first stage has at least four
+// lanes, so every load fills whole 32-byte sectors, and memory is the bound.
+// Four blocks per SM: five (96 registers) and six (80) measured 3% and 20%
+// slower at 64 points and up, as for the joined kernels (L1).
+// Measured, 2^26 elements, before and now: 8 points 297 -> 221 us, 16 516 -> 170,
+// 32 333 -> 161, 64 213 -> 156, 128 201 -> 160 (2^26 elements of HBM: 160 us);
+// 256 .. 1024 158 -> 158, 160 -> 160, 159 -> 160 there and one launch quantum
+// less below 2^19 elements (6.2 -> 4.2 us), where 128-thread blocks of one
+// exchange finish sooner.  Not 4 points (272 -> 283 us: two lanes per
+// transform), nor 2048 and 4096 (166 -> 171, 164 -> 186: a third stage).
+#include "joined.cuh"
+
+namespace gbfft {
+
+template <int LOGL>
+__global__ void __launch_bounds__(128, 4)
+short_lines(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc d) {
+  using SH = typename JoinLen<12, LOGL>::S;
+  using B = JoinBody<SH, JOIN_ROWS, JoinMem>;
+  extern __shared__ __align__(16) unsigned char smem_lines[];
+  cf* sm = reinterpret_cast<cf*>(smem_lines);
+  const int tid = threadIdx.x;
+  const int64_t at = (int64_t)blockIdx.x << 12, valid = d.count_inner - (int64_t)blockIdx.x * B::G;
+  cf v[kJoinR];
+  if (d.conj_in) B::template first_rows<true>(v, in + at, valid, tid);
+  else B::template first_rows<false>(v, in + at, valid, tid);
+  join_stages<SH, JOIN_ROWS, false>(v, sm, d.tw + d.tw_line, 0, 0, tid);
+  if (d.conj_out) B::template store_rows<true>(v, out + at, valid, tid);
+  else B::template store_rows<false>(v, out + at, valid, tid);
+}
+
+template <int LOGL>
+static bool lines_fn(PassLaunch* l) {
+  l->fn = (const void*)short_lines<LOGL>;
+  l->smem = JoinBody<typename JoinLen<12, LOGL>::S, JOIN_ROWS, JoinMem>::kSlots * sizeof(cf);
+  l->block = 128;
+  l->lines = true;
+  return true;
+}
+
+bool resolve_lines(int logL, PassLaunch* l) {
+  switch (logL) {
+    case 3: return lines_fn<3>(l);
+    case 4: return lines_fn<4>(l);
+    case 5: return lines_fn<5>(l);
+    case 6: return lines_fn<6>(l);
+    case 7: return lines_fn<7>(l);
+    case 8: return lines_fn<8>(l);
+    case 9: return lines_fn<9>(l);
+    case 10: return lines_fn<10>(l);
+    default: return false;
+  }
+}
+
+}  // namespace gbfft

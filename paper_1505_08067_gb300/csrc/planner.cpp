@@ -570,6 +570,13 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       off = (off + 1) & ~int64_t(1);
     }
   }
+  for (auto& p : s.passes)
+    if (defaults && p.kind == PASS_FFT && p.batch_is_tiles && !p.tc_prec && !p.conv &&
+        p.logL >= 3 && p.logL <= 10) {
+      p.line_off = off;
+      s.tables.push_back(TwSegment{off, int64_t(1) << p.logL, int64_t(1) << p.logL, 1, 1, 1});
+      off += int64_t(1) << p.logL;
+    }
   if (s.joined) {
     const int64_t L1 = int64_t(1) << s.passes[0].logL, L2 = int64_t(1) << s.passes[1].logL;
     s.join_tw1 = off;
@@ -621,6 +628,7 @@ PassDesc pass_desc(const PassSpec& p, int64_t b0, int64_t nb, int64_t n_total) {
   d.epi_logN = p.epi_logN;
   d.conv = p.conv;
   d.h_scale = p.h_scale;
+  d.tw_line = (int32_t)p.line_off;
   d.h_lines = p.h_lines > 0 ? p.h_lines : 1;
   // line u of a sub-batch starting at entry b0 is line b0 * units + u overall
   d.h_first = p.batch_is_tiles ? (b0 * p.units_per_batch) % d.h_lines : 0;

@@ -86,6 +86,7 @@ struct PassSpec {
   // twiddle-table offsets (complex entries) inside the plan's table allocation
   SmallVec<int32_t, 15> tw_off;  // per stage (stage 0 unused)
   int64_t epi_hi_off = 0, epi_lo_off = 0;
+  int64_t line_off = -1;  // contiguous pass run by the short-line kernel: its table w_L^j
 };
 
 struct TwSegment {  // one twiddle_gen launch (mode 0: exponent (j / r) * (j % r))

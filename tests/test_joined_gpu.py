@@ -17,7 +17,7 @@ def _check(oracle, y, x_np, idx, direction, logn):
 
 
 @pytest.mark.parametrize("logn,batch", [(15, 64), (15, 391), (16, 7), (16, 193), (17, 1),
-                                        (17, 16), (17, 75), (18, 1), (18, 4), (18, 39), (19, 1),
+                                        (17, 16), (17, 75), (18, 1), (18, 3), (18, 39), (19, 1),
                                         (19, 4), (19, 17), (20, 2), (20, 3), (20, 9)])
 @pytest.mark.parametrize("direction", [-1, 1])
 def test_joined(gb, oracle, logn, batch, direction):
@@ -42,7 +42,7 @@ def test_joined(gb, oracle, logn, batch, direction):
         assert torch.equal(first, x)
 
 
-@pytest.mark.parametrize("logn,batch", [(15, 1), (15, 63), (16, 16), (20, 1), (21, 2)])
+@pytest.mark.parametrize("logn,batch", [(15, 1), (15, 63), (16, 16), (18, 4), (20, 1), (21, 2)])
 def test_not_joined(gb, logn, batch):
     with gb.Plan(2 ** logn, batch) as p:
         assert p.describe()["joined"] == 0 and p.launch_count == 2
