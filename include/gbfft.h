@@ -72,8 +72,9 @@ enum { FFT_FORWARD = -1, FFT_INVERSE = +1 };
  * and 2^15 .. 2^24 in six steps (transpose, tensor-core rows of N1, transpose
  * with the twiddle w_N^{n2 k1}, rows of N2, transpose; N = N1 N2, a workspace
  * of 2 min(batch, c) n elements, c = max(1, 2^28 / n); 2^15 .. 2^20 execute the
- * two row passes on column tiles instead, without the transposes -- "tc_columns"
- * in the plan's description):
+ * two row passes on column tiles instead, without the first and last transpose,
+ * and without the middle one for BF16X3 and complex32 -- "tc_columns" in the
+ * plan's description):
  *   FFT_PREC_TC_FP16    stage inputs and DFT matrix rounded to FP16 (each
  *                       stage's input scaled by 1/16, exactly undone at the end)
  *   FFT_PREC_TC_BF16    rounded to BF16

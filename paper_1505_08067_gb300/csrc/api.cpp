@@ -16,6 +16,7 @@
 #include "kernels.h"
 #include "planner.h"
 #include "trace.h"
+#include "umma_stage.h"
 
 using namespace gbfft;
 
@@ -363,10 +364,14 @@ fft_status_t fft_plan_workspace_bytes(fft_plan_t plan, size_t* bytes) {
   return FFT_OK;
 }
 
+static int tc_cols_launches(const PlanSpec& s) {
+  return tc_columns_fused(s.passes[1].tc_prec, s.passes[1].io16) ? 2 : 3;
+}
+
 fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches) {
   if (!plan_ok(plan)) return fail(FFT_ERR_BAD_PLAN, "null or destroyed plan");
   if (!launches) return fail(FFT_ERR_INVALID_ARG, "launches is null");
-  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined ? 1 : plan->spec.tc_cols ? 2 : (int)plan->spec.passes.size();
+  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined ? 1 : plan->spec.tc_cols ? tc_cols_launches(plan->spec) : (int)plan->spec.passes.size();
   return FFT_OK;
 }
 

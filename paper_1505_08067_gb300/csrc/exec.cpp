@@ -1,6 +1,8 @@
 // See exec.h.
 #include "exec.h"
 
+#include "umma_stage.h"
+
 #include <algorithm>
 
 namespace gbfft {
@@ -104,18 +106,29 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
       l.ctas_per_sm = per_sm;
       l.persistent_grid = std::max(per_sm, 1) * caps.sm_count;
       l.d.epi_logN = logN;
-      l.d.conj_in = h == 0 && s.direction == FFT_INVERSE;
-      l.d.conj_out = h == 1 && s.direction == FFT_INVERSE;
+      if (tc_columns_fused(p.tc_prec, p.io16)) {  // else both passes swap, as in the six steps
+        l.d.conj_in = h == 0 && s.direction == FFT_INVERSE;
+        l.d.conj_out = h == 1 && s.direction == FFT_INVERSE;
+      }
       launches[n + h] = l;
     }
   }
   return cudaSuccess;
 }
 
-// The two column launches of a six-step plan for nb transforms.
+// The two column launches of a six-step plan for nb transforms, with the
+// twiddle transpose between them where the first does not multiply.
 static cudaError_t enqueue_tc_cols(const PlanSpec& s, const PassLaunch* launches, const void* in,
-                                   void* out, void* work, int64_t nb, cudaStream_t st) {
+                                   void* out, void* work, void* work2, int64_t nb,
+                                   cudaStream_t st) {
+  const bool fused = tc_columns_fused(s.passes[1].tc_prec, s.passes[1].io16);
   for (int h = 0; h < 2; ++h) {
+    if (h && !fused) {
+      const PassSpec& t = s.passes[2];
+      const cudaError_t e = launch_transpose(work, work2, nb, t.tr_rows, t.tr_cols, t.tr_logN,
+                                             t.tr_sign, t.io16, launches[2].grid, st);
+      if (e != cudaSuccess) return e;
+    }
     PassLaunch l = launches[s.passes.size() + h];
     const PassSpec& p = s.passes[1 + 2 * h];
     const int logN = l.d.epi_logN, le = logN - p.logL;
@@ -125,7 +138,7 @@ static cudaError_t enqueue_tc_cols(const PlanSpec& s, const PassLaunch* launches
     if (h == 0)
       encode_tc_cols_map(l.d, in, nb << p.logL, le, elem_bytes(s.precision), 1 << (12 - p.logL),
                          std::min(1 << p.logL, 256));
-    const cudaError_t e = launch_pass(l, h ? work : in, h ? out : work, st);
+    const cudaError_t e = launch_pass(l, !h ? in : fused ? work : work2, h ? out : work, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -193,9 +206,9 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
     if (a == b || a + bytes <= b || b + bytes <= a)
       return launch_joined(*joined, nb, in, out, work, st);
   }
-  if (s.tc_cols && work) return enqueue_tc_cols(s, launches, in, out, work, nb, st);
   // the second workspace buffer of six-step plans
   void* work2 = work ? static_cast<char*>(work) + work2_off * elem_bytes(s.precision) : nullptr;
+  if (s.tc_cols && work) return enqueue_tc_cols(s, launches, in, out, work, work2, nb, st);
   auto buf = [&](int b) -> void* {
     return b == BUF_IN ? const_cast<void*>(in) : b == BUF_OUT ? out : b == BUF_WORK2 ? work2 : work;
   };

@@ -26,7 +26,7 @@
 // reads finish (tcgen05.wait::ld) before the barrier after which the next
 // stage overwrites the accumulators.
 //
-// The column forms (MODE 1 and 2, UmmaBody) are the two passes of four-step
+// The column forms (MODE 1 to 3, UmmaBody) are the two passes of four-step
 // plans of 2^15 .. 2^20 points: tiles of adjacent columns, staged by tensor-map
 // boxes where contiguous tiles are staged by one bulk copy.
 //
@@ -286,12 +286,12 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
     return (uint32_t)((rem < G::TPT ? rem : G::TPT) * G::L * ESZ);
   };
   const bool staged =
-      kStaged && (MODE == 1 ? d.tmap_in_ok != 0 : (reinterpret_cast<uintptr_t>(in) & 15) == 0);
+      kStaged && (MODE % 2 ? d.tmap_in_ok != 0 : (reinterpret_cast<uintptr_t>(in) & 15) == 0);
   // the column forms' tiles (UmmaBody): tiles per transform, log2
   const int tpt_log = MODE ? d.epi_logN - G::LOGT : 0;
   // this thread's copy of tile t into the staging buffer
   auto stage_copy = [&](int64_t t) {
-    if constexpr (MODE == 1) {
+    if constexpr (MODE % 2 == 1) {
       constexpr int BR = G::L < 256 ? G::L : 256;
       const uint64_t map = reinterpret_cast<uint64_t>(&d.tmap_in[0]);
       const int x = (int)(t & ((int64_t(1) << tpt_log) - 1)) * G::TPT;
@@ -349,8 +349,8 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
     const int valid = MODE || rem >= G::TPT ? G::TPT : (int)rem;
     const int64_t unit = tile >> tpt_log;  // column forms: the transform, and the tile's column
     const int col0 = MODE ? (int)(tile - (unit << tpt_log)) * G::TPT : 0;
-    const cf* gin = Mem::at(in, MODE == 1 ? (unit << d.epi_logN) + col0 : first * G::L);
-    cf* gout = Mem::at(out, MODE ? (unit << d.epi_logN) + col0 : first * G::L);
+    const cf* gin = Mem::at(in, MODE % 2 ? (unit << d.epi_logN) + col0 : first * G::L);
+    cf* gout = Mem::at(out, MODE == 1 || MODE == 2 ? (unit << d.epi_logN) + col0 : first * G::L);
     // the tile this CTA takes next, into L2 while this one is computed
     // (whole 16-byte units inside the tile only; none for a ragged tile).
     // Measured per form: it pays for complex32 storage, for tiles of 4096
@@ -359,7 +359,7 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
     // it, DRAM reads were 17% above the tile bytes: prefetched lines read
     // again).
     constexpr bool kPrefetchL2 = H || LOGL < 13 || (U::SPLIT && LOGL == 13);
-    if (MODE != 1 && kPrefetchL2 && !staged && tid == 0 && tile + gridDim.x < d.tiles) {
+    if (MODE % 2 == 0 && kPrefetchL2 && !staged && tid == 0 && tile + gridDim.x < d.tiles) {
       const int64_t nfirst = (tile + gridDim.x) * G::TPT;
       if (nfirst + G::TPT <= d.count_inner) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(Mem::at(in, nfirst * G::L));
@@ -368,7 +368,7 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
         if (e16 > a16) prefetch_l2(reinterpret_cast<const void*>(a16), (uint32_t)(e16 - a16));
       }
     }
-    if constexpr (MODE == 1) {  // the same for columns: boxes of the input's tensor map
+    if constexpr (MODE % 2 == 1) {  // the same for columns: boxes of the input's tensor map
       if (!staged && d.tmap_in_ok && tid == 0 && tile + gridDim.x < d.tiles) {
         constexpr int BR = G::L < 256 ? G::L : 256;
         const int64_t t = tile + gridDim.x;

@@ -52,6 +52,7 @@ namespace gbfft {
 // are runs of adjacent columns; the stage before was chosen for that.
 GB_HD constexpr uint64_t umma_perm_code(int logL, int t, int mode = 0) {
   // nibble k = butterfly-index bit held by row bit k
+  if (mode == 3) mode = 1;
   if (mode) {
     if (logL == 7) return 0x21076543ull;
     if (logL == 8) return t ? 0x32107654ull : mode == 1 ? 0x73210654ull : 0x76543210ull;
@@ -80,7 +81,7 @@ GB_HD constexpr uint64_t umma_perm_code(int logL, int t, int mode = 0) {
 // Mode 1 (columns) puts the transform bits there instead: adjacent columns.
 GB_HD constexpr uint32_t umma_load_lanes_code(int logL, int mode = 0) {
   // nibble k = bit of the loader's work item selected by lane bit k
-  if (mode == 1) {
+  if (mode % 2) {
     if (logL == 7) return 0x87654u;
     if (logL == 8) return 0xba984u;
     if (logL == 9) return 0xa9854u;
@@ -119,17 +120,22 @@ GB_HD constexpr int umma_staging_bytes(int logL, int eb, bool split) {
 }
 
 // Do tensor-core plans of 2^logn points (six steps: transposes and row passes)
-// run as two passes over column tiles?  A tile of 4096 elements holds
+// run over column tiles, without the first and last transpose?  A tile of 4096 elements holds
 // 4096 / L >= 4 adjacent columns for passes of up to 1024 points, whole 32-byte
 // sectors per row (complex32: 16 bytes at 1024 points, still far ahead of five
 // passes); 2048-point passes would leave 16 bytes and 8.
 // What bounds the six steps is memory: five passes, 80 bytes an element, of
 // which the transposes take 60%.  The column forms read and write each element
 // twice; their stages are the ones of the contiguous kernel, which bound them.
-// Measured, 2^25 elements, six steps and now: 2^16 FP16 451 -> 201 us, BF16
-// 452 -> 201, BF16x3 497 -> 231, complex32 322 -> 144; 2^20 462 -> 229,
-// 460 -> 227, 515 -> 332, 331 -> 212.
+// The twiddle moves into the first pass's last stage for BF16x3 and complex32
+// (tc_columns_fused).  FP16 and BF16 with complex64 data keep the twiddle
+// transpose as a pass of its own: twiddles rounded differently in the last bit
+// flip roundings to 16 bits downstream, and moved the outputs by 2e-5 and 6e-5.
+// Measured, 2^25 elements, six steps and now: 2^16 BF16x3 497 -> 231 us, complex32
+// 322 -> 144; 2^20 515 -> 332, 331 -> 212; FP16 and BF16 (bit for bit the six
+// steps' outputs) 2^15 451 -> 408, 2^16 451 -> 375, 2^18 462 -> 319, 2^20 462 -> 316.
 GB_HD constexpr bool tc_columns(int logn) { return logn >= 15 && logn <= 20; }
+GB_HD constexpr bool tc_columns_fused(int prec, int io16) { return prec == TC_BF16X3 || io16; }
 
 template <int LOGL>
 struct UmmaGeo {
@@ -288,7 +294,9 @@ GB_HD void umma_first_target(int e, int o, int& u, int& i, int& tw) {
 // plan (N = N1 N2, x[n1 N2 + n2]).  1: a tile holds adjacent columns n2, read and
 // written as columns of rows of 2^le = N2 elements, the outputs multiplied by
 // the four-step twiddle w_N^{n2 k1}.  2: a tile holds adjacent rows k1, read as
-// rows and written as columns of rows of 2^le = N1 elements.
+// rows and written as columns of rows of 2^le = N1 elements.  3: as 1, but the
+// outputs of each column n2 are written as one contiguous row and not
+// multiplied (a twiddle transpose follows).
 template <int LOGL, int PREC, class Mem, int MODE = 0>
 struct UmmaBody {
   using G = UmmaGeo<LOGL>;
@@ -367,9 +375,9 @@ struct UmmaBody {
                               uint32_t a_lo, const Parts& parts) {
     const bool swap = d.conj_in != 0;
     // offset of tile element x; the parts of disjoint bits add up
-    const int le = MODE == 1 && !STAGED ? d.epi_logN - LOGL : LOGL == 12 ? 0 : 12 - LOGL;
+    const int le = MODE % 2 && !STAGED ? d.epi_logN - LOGL : LOGL == 12 ? 0 : 12 - LOGL;
     auto at = [&](int x) {
-      return MODE == 1 ? ((x & (G::L - 1)) << le) + (x >> LOGL) : x;
+      return MODE % 2 ? ((x & (G::L - 1)) << le) + (x >> LOGL) : x;
     };
 #pragma unroll 1
     for (int b = 0; b < KB; ++b) {
@@ -465,7 +473,7 @@ GB_UNROLL
     if (t == G::NTC - 1) {
       rp.tr = u >> G::BPSB;
       const int pos = umma_out_pos(G::ns_log(t), u & ((1 << G::BPSB) - 1), 0);
-      rp.pos = MODE ? (pos << (d.epi_logN - LOGL)) + rp.tr : (rp.tr << LOGL) | pos;
+      rp.pos = MODE == 1 || MODE == 2 ? (pos << (d.epi_logN - LOGL)) + rp.tr : (rp.tr << LOGL) | pos;
       if constexpr (MODE == 1) {
         rp.run = Mem::rotor((int64_t)(col0 + rp.tr) * pos, d.epi_logN);
         rp.step = Mem::rotor((int64_t)(col0 + rp.tr) << G::ns_log(t), d.epi_logN);
@@ -510,7 +518,7 @@ GB_UNROLL
           v = cmul(v, rp.run);
           rp.run = cmul(rp.run, rp.step);
         }
-        if constexpr (MODE != 0) Mem::stg_sw(o_base, (o << G::ns_log(t)) << (d.epi_logN - LOGL), v, swap);
+        if constexpr (MODE == 1 || MODE == 2) Mem::stg_sw(o_base, (o << G::ns_log(t)) << (d.epi_logN - LOGL), v, swap);
         else Mem::stg_sw(o_base, o << G::ns_log(t), v, swap);
       }
     } else {

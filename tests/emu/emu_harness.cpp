@@ -644,8 +644,8 @@ void run_umma_t(const PassDesc& d, const cf* in, cf* out) {
     const int tpt_log = MODE ? d.epi_logN - G::LOGT : 0;
     const int64_t unit = tile >> tpt_log;
     const int col0 = MODE ? (int)(tile - (unit << tpt_log)) * G::TPT : 0;
-    const cf* gin = in + (MODE == 1 ? (unit << d.epi_logN) + col0 : first * G::L);
-    cf* gout = out + (MODE ? (unit << d.epi_logN) + col0 : first * G::L);
+    const cf* gin = in + (MODE % 2 ? (unit << d.epi_logN) + col0 : first * G::L);
+    cf* gout = out + (MODE == 1 || MODE == 2 ? (unit << d.epi_logN) + col0 : first * G::L);
     ++g_umma.phase;
     for (int warp = 0; warp < G::NWARP; ++warp)
       for (int lane = 0; lane < 32; ++lane) {
@@ -716,8 +716,12 @@ bool run_tc_cols_t(const PlanSpec& s, const cf* tables, int64_t batch, const cf*
     PassDesc d = pass_desc(p, 0, batch, batch);
     d.tw = tables;
     d.epi_logN = logN;
-    d.conj_in = h == 0 && s.direction == FFT_INVERSE;
-    d.conj_out = h == 1 && s.direction == FFT_INVERSE;
+    constexpr bool kFused = tc_columns_fused(PREC, 0);
+    constexpr int kFirst = kFused ? 1 : 3;
+    if (kFused) {
+      d.conj_in = h == 0 && s.direction == FFT_INVERSE;
+      d.conj_out = h == 1 && s.direction == FFT_INVERSE;
+    }
     d.tiles = batch << (logN - 12);
     d.count_inner = batch << (logN - p.logL);
     const cf* src = h ? work : in;
@@ -732,7 +736,7 @@ bool run_tc_cols_t(const PlanSpec& s, const cf* tables, int64_t batch, const cf*
     g.tw_len = s.table_elems;
     switch (p.logL * 10 + h) {
 #define GB_UC(LG) \
-  case LG * 10: run_umma_t<LG, PREC, 1>(d, src, dst); break; \
+  case LG * 10: run_umma_t<LG, PREC, kFirst>(d, src, dst); break; \
   case LG * 10 + 1: run_umma_t<LG, PREC, 2>(d, src, dst); break;
       GB_UC(7) GB_UC(8) GB_UC(9) GB_UC(10)
 #undef GB_UC
@@ -740,6 +744,16 @@ bool run_tc_cols_t(const PlanSpec& s, const cf* tables, int64_t batch, const cf*
     }
     for (int64_t i = 0; i < E; ++i)
       if (hits[i] != 1) { err("output element not written exactly once", i); break; }
+    if (h == 0 && !kFused) {  // the twiddle transpose, from its definition
+      const PassSpec& t = s.passes[2];
+      std::vector<cf> c(work, work + E);
+      for (int64_t i = 0; i < E; ++i) {
+        const int64_t b = i >> logN, r = (i >> p.logL) & (t.tr_rows - 1), k = i & (t.tr_cols - 1);
+        cf w = root(r * k, int64_t(1) << logN);
+        if (t.tr_sign > 0) w = mk(w.x, -w.y);
+        work[(b << logN) + k * t.tr_rows + r] = cmul(c[i], w);
+      }
+    }
   }
   return true;
 }
