@@ -224,7 +224,8 @@ GBFFT_API fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches);
  * the compile-time kernel of the shape), "compile_time", "generic",
  * "tensor_core" or "copy" -- with its persistent-grid size and L2-prefetch
  * flag, and "lines": 1 when the short-line kernel (contiguous transforms of
- * 2^3 .. 2^10 points, default options) runs the pass instead; "joined": 1 when both passes of a two-pass or 2D plan run as one launch
+ * 2^3 .. 2^10 points; fast convolution of lines and columns of 2^3 .. 2^11;
+ * default options) runs the pass instead; "joined": 1 when both passes of a two-pass or 2D plan run as one launch
  * of a joined kernel, 0 when each runs the kernel named for it) written to buf (NUL-terminated, truncated to len).  Returns
  * FFT_ERR_INVALID_ARG if buf is too small for the whole text.
  */

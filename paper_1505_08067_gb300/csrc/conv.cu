@@ -1,5 +1,5 @@
 // Fast-convolution passes (matched filtering, e.g. SAR range and azimuth
-// compression): generic kernels for every (R, map) and the compile-time
+// compression) other than those of conv_lines.cu: generic kernels for every (R, map) and the compile-time
 // shapes of GB_SHAPES_CONV.  See conv_tile in kernels_impl.cuh.
 #include "kernels_impl.cuh"
 

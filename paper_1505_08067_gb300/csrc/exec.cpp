@@ -7,9 +7,11 @@
 
 namespace gbfft {
 
-// Blocks of a short-line launch: tiles of 4096 elements.
-static int lines_grid(const PassDesc& d, int logL) {
-  return (int)std::min<int64_t>(((d.count_inner << logL) + 4095) >> 12, 0x7fffffff);
+// Blocks of a line launch: tiles of 2^tile_log elements.
+static int lines_grid(const PassDesc& d, int tile_log) {
+  const int64_t outer = d.tiles_inner > 0 ? d.tiles / d.tiles_inner : 0;
+  const int64_t n = (outer * d.count_inner) << d.logL, tile = int64_t(1) << tile_log;
+  return (int)std::min<int64_t>((n + tile - 1) >> tile_log, 0x7fffffff);
 }
 
 cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables, int* status,
@@ -37,7 +39,10 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
         l.specialised = true;
       } else {
         l.fn = resolve_kernel(l.R, l.lmap, l.smap, l.d, s.generic_only, &l.specialised);
-        if (p.line_off >= 0 && resolve_lines(p.logL, &l)) l.grid = lines_grid(l.d, p.logL);
+        if (p.line_off >= 0 && (!p.conv                ? resolve_lines(p.logL, &l)
+                                : p.lmap == MAP_ROWS ? resolve_conv_lines(p.logL, &l)
+                                                     : resolve_conv_cols(p.logL, &l)))
+          l.grid = lines_grid(l.d, l.lines);
       }
       cudaError_t e = prepare_launch(l);
       if (e != cudaSuccess) return e;
@@ -70,7 +75,7 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
       const bool reg4096 = p.variant == 0 && !p.conv && !p.tc_prec && p.logL == 12 &&
                            p.lmap == MAP_ROWS && p.smap == MAP_ROWS;
       const bool want_staged =
-          (p.variant == 0 && !reg4096) || p.variant == 2 || p.variant == 4;
+          ((p.variant == 0 && !reg4096) || p.variant == 2 || p.variant == 4) && !l.lines;
       l.has_staged = want_staged && resolve_staged(l.d, l.lmap, l.smap, s.generic_only, &l.staged);
       l.staged.tmap = p.variant != 4;
       if (l.has_staged) {
@@ -239,7 +244,7 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
         if (e != cudaSuccess) return e;
         d.l2_prefetch = launches[i].d.l2_prefetch;
         l.d.l2_prefetch = d.l2_prefetch;
-        l.grid = l.lines ? lines_grid(d, p.logL)
+        l.grid = l.lines ? lines_grid(d, l.lines)
                          : (int)std::min<int64_t>(d.tiles, l.persistent_grid ? l.persistent_grid
                                                                               : 0x7fffffff);
       }

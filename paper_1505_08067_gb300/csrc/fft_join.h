@@ -107,6 +107,13 @@ struct JoinShape {
   static constexpr int kLast = kNst - 1;
 };
 
+// The same length with the stages in reverse order.
+template <class SH> struct JoinReverse;
+template <int TL, int LOGL, int RA, int RB, int RC>
+struct JoinReverse<JoinShape<TL, LOGL, RA, RB, RC>> {
+  using S = JoinShape<TL, LOGL, RC ? RC : RB, RC ? RB : RA, RC ? RA : 0>;
+};
+
 // What a tile's pass is: the first of a four-step transform (columns in, blocks
 // of the workspace out), columns in and out, or contiguous rows in and out.
 enum { JOIN_FIRST = 0, JOIN_COLS = 1, JOIN_ROWS = 2 };
@@ -194,6 +201,34 @@ GB_UNROLL
   GB_HD static int64_t frame_col(int64_t col, int lc) {
     return ((col >> lc) << (SH::kLogL + lc)) + (col & ((int64_t(1) << lc) - 1));
   }
+  // Fast convolution, between its two rounds: after the forward stages this
+  // thread holds the spectrum at positions jb + i Ns of its last-stage
+  // butterflies, which are the inputs of its first-stage butterflies in the
+  // reversed schedule (Ns = L / radix).  Multiplies them by scale * H and swaps
+  // real and imaginary parts for the inverse.  Rows: line u's filter at
+  // h + (u mod lines) L (first: the tile's first line); columns: column u's in
+  // column u mod lines of a frame of rows of `lines` elements; lines = 1: one
+  // filter for all.
+  GB_HD static void filter(cf (&v)[R], const cf* h, int64_t lines, int64_t first, float scale,
+                           int tid) {
+    constexpr int S = SH::kLast, RR = SH::radix(S), NB = R / RR, Ns = SH::ns(S);
+    if (first >= lines) first %= lines;
+GB_UNROLL
+    for (int q = 0; q < NB; ++q) {
+      int c, jb;
+      coords<S>(q * T + tid, c, jb);
+      int64_t u = lines > 1 ? first + c : 0;
+      if (u >= lines) u %= lines;  // seldom: first is below lines
+      const int64_t e = KIND == JOIN_COLS && lines > 1 ? lines : 1;
+      const cf* p = h + (KIND == JOIN_COLS ? u : u * L) + jb * e;
+GB_UNROLL
+      for (int i = 0; i < RR; ++i) {
+        const cf z = cmul(v[q * RR + i], Mem::ldtw(p + i * Ns * e));
+        v[q * RR + i] = mk(z.y * scale, z.x * scale);
+      }
+    }
+  }
+
   // Stage 0 of a frame's column pass: columns col0 .. col0 + G - 1 of all the
   // frames in buf, of which there are `cols`; zeros beyond.
   GB_HD static void first_frame(cf (&v)[R], const cf* buf, int64_t col0, int64_t cols, int lc,

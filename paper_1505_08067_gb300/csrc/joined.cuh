@@ -180,6 +180,23 @@ __device__ __forceinline__ void join_stages(cf (&v)[kJoinR], cf* sm, const cf* t
   B::template turn<SH::kLast, TW4>(v, tw, col0, logN, tid);
 }
 
+// Both rounds of a fast convolution: forward stages, filter, the stages in
+// reverse order on swapped data (the unnormalised inverse).
+template <class SH, int KIND>
+__device__ __forceinline__ void join_conv(cf (&v)[kJoinR], cf* sm, const cf* tw, const cf* h,
+                                          int64_t lines, int64_t first, float scale, int tid) {
+  join_stages<SH, KIND, false>(v, sm, tw, 0, 0, tid);
+  JoinBody<SH, KIND, JoinMem>::filter(v, h, lines, first, scale, tid);
+  join_sync<SH::kThreads>();  // every thread has read the last exchange
+  join_stages<typename JoinReverse<SH>::S, KIND, false>(v, sm, tw, 0, 0, tid);
+}
+template <class SH, int KIND>
+constexpr int join_conv_slots() {
+  constexpr int a = JoinBody<SH, KIND, JoinMem>::kSlots;
+  constexpr int b = JoinBody<typename JoinReverse<SH>::S, KIND, JoinMem>::kSlots;
+  return a > b ? a : b;
+}
+
 // Four-step transforms of 2^LOGN points.
 template <int LOGN, int TL, bool INV>
 __global__ void __launch_bounds__((1 << TL) / kJoinR + 32, 1 << join_blocks_log(TL))

@@ -73,7 +73,7 @@ struct PassLaunch {
   size_t smem;      // dynamic shared memory in bytes
   const void* fn = nullptr;  // resolved kernel (specialised or generic)
   bool specialised = false;
-  bool lines = false;        // the short-line kernel (resolve_lines): a tile of 4096 elements per block
+  int lines = 0;             // a line kernel (resolve_lines): log2 of its tile, one per block
   bool has_staged = false;   // a staged kernel exists for this shape (see below)
   int persistent_grid = 0;   // nonzero: grid capped at resident blocks (L2-prefetch variant)
   int ctas_per_sm = 0;       // persistent kernels: resident blocks per SM the grid assumes
@@ -149,6 +149,10 @@ cudaError_t launch_transpose(const void* in, void* out, int64_t batch, int64_t r
 // The short-line kernel of a contiguous pass of 2^logL points (lines.cu): sets
 // fn, block and smem; false if there is none.
 bool resolve_lines(int logL, PassLaunch* l);
+// The same for fast convolution (conv_lines.cu): contiguous lines, and the
+// columns of frames.
+bool resolve_conv_lines(int logL, PassLaunch* l);
+bool resolve_conv_cols(int logL, PassLaunch* l);
 
 // Per-kernel attributes a launch needs (opt-in shared memory); call once after
 // resolving, before the first launch_pass.

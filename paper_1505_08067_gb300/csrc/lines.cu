@@ -40,7 +40,7 @@ static bool lines_fn(PassLaunch* l) {
   l->fn = (const void*)short_lines<LOGL>;
   l->smem = JoinBody<typename JoinLen<12, LOGL>::S, JOIN_ROWS, JoinMem>::kSlots * sizeof(cf);
   l->block = 128;
-  l->lines = true;
+  l->lines = 12;
   return true;
 }
 

@@ -571,8 +571,8 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
     }
   }
   for (auto& p : s.passes)
-    if (defaults && p.kind == PASS_FFT && p.batch_is_tiles && !p.tc_prec && !p.conv &&
-        p.logL >= 3 && p.logL <= 10) {
+    if (defaults && p.kind == PASS_FFT && (p.batch_is_tiles || p.conv) && !p.tc_prec &&
+        p.logL >= 3 && p.logL <= (p.conv ? 11 : 10)) {
       p.line_off = off;
       s.tables.push_back(TwSegment{off, int64_t(1) << p.logL, int64_t(1) << p.logL, 1, 1, 1});
       off += int64_t(1) << p.logL;

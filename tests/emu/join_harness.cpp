@@ -22,7 +22,8 @@ using namespace gbfft;
 namespace {
 
 struct Ctx {
-  const cf *in, *tw1, *tw2;
+  const cf *in, *tw1, *tw2, *h;
+  int64_t h_len;
   cf *out, *work;
   int64_t in_len, out_len, work_len;
   std::vector<uint8_t> out_hits;
@@ -88,6 +89,7 @@ struct CheckMem {
   }
   static cf ldtw(const cf* p) {
     const bool one = p >= g.tw1 && p < g.tw1 + g.tw1_len, two = p >= g.tw2 && p < g.tw2 + g.tw2_len;
+    if (p >= g.h && p < g.h + g.h_len) return *p;
     if (!one && !two) { err("twiddle load out of bounds", 0); return mk(1, 0); }
     return *p;
   }
@@ -248,6 +250,56 @@ int64_t run_frames(int64_t batch, int lr, int lc, const cf* in, cf* out) {
   return g.errors;
 }
 
+// ---------------------------------------------------- fast convolution --
+// Lines or columns of frames, tile by tile: the stages, the filter, the stages
+// in reverse order.
+template <int TL, int LOGL, int KIND>
+void conv(const cf* in, cf* out, int64_t total, int lc, const cf* h, int64_t lines, float scale) {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  using RS = typename JoinReverse<SH>::S;
+  using B = JoinBody<SH, KIND, CheckMem>;
+  using BR = JoinBody<RS, KIND, CheckMem>;
+  std::vector<cf> sm(std::max(B::kSlots, BR::kSlots));
+  g.sm = sm.data();
+  g.smem_len = (int)sm.size();
+  g.phase_of.assign(sm.size(), -1);
+  const int64_t n = total >> LOGL;
+  for (int64_t t = 0; t * B::G < n; ++t) {
+    std::vector<cf> keep((size_t)SH::kThreads * kJoinR);
+    auto k = [&](int i) -> cf (&)[kJoinR] { return *reinterpret_cast<cf(*)[kJoinR]>(&keep[(size_t)i * kJoinR]); };
+    auto copy = [](cf (&d)[kJoinR], const cf (&s)[kJoinR]) { for (int j = 0; j < kJoinR; ++j) d[j] = s[j]; };
+    tile<SH, KIND>(
+        sm.data(), sm.data(), g.tw1, 0, 0,
+        [&](cf (&v)[kJoinR], int i) {
+          if constexpr (KIND == JOIN_ROWS) B::template first_rows<false>(v, in + (t << TL), n - t * B::G, i);
+          else B::first_frame(v, g.work, t * B::G, n, lc, i);
+        },
+        [&](cf (&v)[kJoinR], int i) { B::filter(v, h, lines, t * B::G, scale, i); copy(k(i), v); });
+    tile<RS, KIND>(
+        sm.data(), sm.data(), g.tw1, 0, 0, [&](cf (&v)[kJoinR], int i) { copy(v, k(i)); },
+        [&](cf (&v)[kJoinR], int i) {
+          if constexpr (KIND == JOIN_ROWS) BR::template store_rows<true>(v, g.work + (t << TL), n - t * B::G, i);
+          else BR::template store_frame<true>(v, out, t * B::G, n, lc, i);
+        });
+  }
+}
+
+template <int KIND>
+bool conv_len(int logl, const cf* in, cf* out, int64_t total, int lc, const cf* h, int64_t lines, float scale) {
+  switch (logl) {
+#define GB_CV(TL, L) case L: conv<TL, L, KIND>(in, out, total, lc, h, lines, scale); return true;
+    GB_CV(12, 3) GB_CV(12, 4) GB_CV(12, 5) GB_CV(12, 6) GB_CV(12, 7) GB_CV(12, 8)
+    default: break;
+  }
+  if constexpr (KIND == JOIN_ROWS) {
+    switch (logl) { GB_CV(12, 9) GB_CV(12, 10) GB_CV(12, 11) default: break; }
+  } else {
+    switch (logl) { GB_CV(13, 9) GB_CV(13, 10) GB_CV(13, 11) default: break; }
+  }
+#undef GB_CV
+  return false;
+}
+
 }  // namespace
 
 extern "C" int64_t join_run(int logn, int tile_log, int64_t nb, int inverse, int64_t lag, int ring, const float* in,
@@ -278,4 +330,44 @@ extern "C" int64_t join_run_frames(int64_t batch, int lr, int lc, int inverse, c
                         : (inverse ? run_frames<13, true>(batch, lr, lc, x, y) : run_frames<13, false>(batch, lr, lc, x, y));
   snprintf(msg, len, "%s", g.first.c_str());
   return e;
+}
+
+// cols = 0: batch lines of 2^logl; else the columns of 2^logl rows of frames of
+// `cols` columns.  Filters as fft_filter_t lays them out.
+extern "C" int64_t conv_run(int64_t batch, int logl, int cols, int64_t lines, float scale,
+                            const float* h, const float* in, float* out, char* msg, size_t len) {
+  const cf* x = reinterpret_cast<const cf*>(in);
+  cf* y = reinterpret_cast<cf*>(out);
+  const int64_t total = (batch << logl) * (cols ? cols : 1);
+  int lc = 0;
+  while (1 << lc < cols) ++lc;
+  g = Ctx{};
+  std::vector<cf> t1 = roots(1 << logl);
+  g.in = x;
+  g.out = y;
+  g.in_len = g.out_len = g.work_len = total;
+  g.tw1 = t1.data();
+  g.tw1_len = 1 << logl;
+  g.tw2 = nullptr;
+  g.h = reinterpret_cast<const cf*>(h);
+  g.h_len = lines << logl;
+  g.out_hits.assign(total, 0);
+  bool ok;
+  if (cols) {  // columns read and write the output buffer: the input is put there first
+    std::vector<cf> mid(x, x + total);
+    g.work = mid.data();
+    g.work_owner.assign(total, 0);
+    ok = conv_len<JOIN_COLS>(logl, x, y, total, lc, g.h, lines, scale);
+    for (int64_t i = 0; i < total; ++i)
+      if (g.out_hits[i] != 1) { err("output element not written exactly once", i); break; }
+  } else {
+    g.work = y;
+    g.work_owner.assign(total, -1);
+    ok = conv_len<JOIN_ROWS>(logl, x, y, total, 0, g.h, lines, scale);
+    for (int64_t i = 0; i < total; ++i)
+      if (g.work_owner[i] != 0) { err("output element not written", i); break; }
+  }
+  if (!ok) err("no such length", logl);
+  snprintf(msg, len, "%s", g.first.c_str());
+  return g.errors;
 }

@@ -64,3 +64,27 @@ def test_joined_frames(oracle, joined, lr, lc, batch, direction):
     assert n == 0, msg.value.decode()
     ref = oracle.fft2d(x, direction).reshape(batch, -1)
     assert np.max(oracle.rel_l2(y.reshape(batch, -1), ref)) <= 1e-6 * (lr + lc)
+
+
+@pytest.mark.parametrize("logl,cols,batch", [(3, 0, 600), (4, 0, 257), (5, 0, 3), (6, 0, 65), (7, 0, 33),
+                                             (8, 0, 17), (9, 0, 9), (10, 0, 5), (11, 0, 3), (3, 64, 9), (5, 16, 9), (6, 128, 1), (7, 4, 9),
+                                             (8, 32, 1), (9, 8, 3), (10, 16, 1), (11, 8, 1)])
+@pytest.mark.parametrize("per_line", [False, True])
+def test_conv_tiles(oracle, joined, logl, cols, batch, per_line):
+    """Fast convolution of lines (cols = 0) and of frame columns, a ragged last tile."""
+    n = 2 ** logl
+    f = joined.conv_run
+    f.restype = ctypes.c_int64
+    f.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_int64, ctypes.c_float] + \
+        [ctypes.c_void_p] * 3 + [ctypes.c_char_p, ctypes.c_size_t]
+    lines = (cols or batch) if per_line else 1
+    x = synth.uniform(90 + logl, batch, n * max(1, cols)).reshape(batch, n, max(1, cols))
+    h = synth.uniform(190 + logl, lines, n)  # a filter per line
+    hl = np.ascontiguousarray(h.T) if cols else h  # columns: laid out like a frame
+    y = np.zeros_like(x)
+    msg = ctypes.create_string_buffer(256)
+    e = f(batch, logl, cols, lines, 1.0 / n, hl.ctypes.data, x.ctypes.data, y.ctypes.data, msg, 256)
+    assert e == 0, msg.value.decode()
+    H = (h.T[None] if cols else h[:, :, None]).astype(np.complex128)
+    ref = np.fft.ifft(np.fft.fft(x.astype(np.complex128), axis=1) * H, axis=1)
+    assert np.linalg.norm(y - ref) <= 2e-6 * logl * np.linalg.norm(ref)
