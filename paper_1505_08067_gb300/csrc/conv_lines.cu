@@ -30,6 +30,7 @@ conv_lines(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc 
   cf* sm = reinterpret_cast<cf*>(smem_lines);
   const int tid = threadIdx.x;
   const int64_t at = (int64_t)blockIdx.x << TL, line = (int64_t)blockIdx.x * B::G;
+  grid_wait();
   cf v[kJoinR];
   B::template first_rows<false>(v, in + at, d.count_inner - line, tid);
   join_conv<SH, JOIN_ROWS>(v, sm, d.tw + d.tw_line, d.h, d.h_lines, d.h_first + line, d.h_scale, tid);
@@ -47,6 +48,7 @@ conv_cols(const cf* in, cf* out, const __grid_constant__ PassDesc d) {
   cf* sm = reinterpret_cast<cf*>(smem_lines);
   const int tid = threadIdx.x, lc = 31 - __clz((int)d.in.e);
   const int64_t col0 = (int64_t)blockIdx.x * B::G, cols = d.tiles / d.tiles_inner * d.count_inner;
+  grid_wait();
   cf v[kJoinR];
   B::first_frame(v, in, col0, cols, lc, tid);
   join_conv<SH, JOIN_COLS>(v, sm, d.tw + d.tw_line, d.h, d.h_lines, col0, d.h_scale, tid);

@@ -214,6 +214,7 @@ joined_pass(const cf* in, cf* out, cf* work, const __grid_constant__ JoinDesc d)
   const int tid = threadIdx.x;
   if (tid == 0) mbar_init(&stored, T / 32);
   __syncthreads();
+  grid_wait();
   if (tid >= T) {
     join_dispatch(
         d, &stored, s_ticket, tid - T,
@@ -295,6 +296,7 @@ joined_frames(const cf* in, cf* out, const __grid_constant__ JoinDesc d) {
   const int tid = threadIdx.x;
   if (tid == 0) mbar_init(&stored, T / 32);
   __syncthreads();
+  grid_wait();
   if (tid >= T) {
     join_dispatch(
         d, &stored, s_ticket, tid - T,

@@ -66,15 +66,8 @@ cudaError_t launch_joined(const JoinedLaunch& j, int64_t batch, const void* in, 
   const int grid = (int)std::min<int64_t>(j.max_grid, join_tickets(d.o));
   const cf* ci = static_cast<const cf*>(in);
   cf* co = static_cast<cf*>(out);
-  if (j.frames) {
-    using Fn = void (*)(const cf*, cf*, JoinDesc);
-    reinterpret_cast<Fn>(const_cast<void*>(j.fn))<<<grid, j.block, j.smem, st>>>(ci, co, d);
-  } else {
-    using Fn = void (*)(const cf*, cf*, cf*, JoinDesc);
-    reinterpret_cast<Fn>(const_cast<void*>(j.fn))<<<grid, j.block, j.smem, st>>>(
-        ci, co, static_cast<cf*>(work), d);
-  }
-  return cudaGetLastError();
+  if (j.frames) return launch_early(j.fn, grid, j.block, j.smem, st, ci, co, d);
+  return launch_early(j.fn, grid, j.block, j.smem, st, ci, co, static_cast<cf*>(work), d);
 }
 
 }  // namespace gbfft

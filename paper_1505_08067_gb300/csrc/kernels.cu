@@ -173,15 +173,14 @@ bool encode_cols_maps(PassDesc& d, bool map_in, bool map_out, const void* in, vo
 
 cudaError_t launch_staged(const StagedLaunch& s, const PassDesc& d, const void* in, void* out,
                           cudaStream_t st) {
-  KernelFn k = reinterpret_cast<KernelFn>(const_cast<void*>(s.fn));
-  if (!k || s.grid < 1) return cudaErrorInvalidValue;
+  if (s.grid < 1) return cudaErrorInvalidValue;
   PassDesc dm = d;
   if (s.tmap && (s.map_in || s.map_out)) {
     const bool mo = s.map_out && cols_store_map(d);
     encode_cols_maps(dm, s.map_in, mo, in, out);
   }
-  k<<<s.grid, s.block, s.smem, st>>>(static_cast<const cf*>(in), static_cast<cf*>(out), dm);
-  return cudaGetLastError();
+  return launch_early(s.fn, s.grid, s.block, s.smem, st, static_cast<const cf*>(in),
+                      static_cast<cf*>(out), dm);
 }
 
 void encode_tc_cols_map(PassDesc& d, const void* in, int64_t rows, int le, int esz, int cols,
@@ -197,10 +196,8 @@ cudaError_t prepare_launch(PassLaunch& p) {
 }
 
 cudaError_t launch_pass(const PassLaunch& p, const void* in, void* out, cudaStream_t st) {
-  KernelFn k = reinterpret_cast<KernelFn>(const_cast<void*>(p.fn));
-  if (!k) return cudaErrorInvalidValue;
-  k<<<p.grid, p.block, p.smem, st>>>(static_cast<const cf*>(in), static_cast<cf*>(out), p.d);
-  return cudaGetLastError();
+  return launch_early(p.fn, p.grid, p.block, p.smem, st, static_cast<const cf*>(in),
+                      static_cast<cf*>(out), p.d);
 }
 
 cudaError_t occupancy(const PassLaunch& p, int* ctas_per_sm) {

@@ -13,6 +13,14 @@ namespace gbfft {
 
 using KernelFn = void (*)(const cf*, cf*, PassDesc);
 
+// Waits until the kernels before this one in its stream are complete and their
+// writes visible (a no-op unless this launch was allowed to start early).  Every
+// thread of a kernel that launch_early launches calls it before its first access
+// to global memory, twiddle tables included (fft_execute_noalloc regenerates
+// them in the stream), so that a block's end implies that everything before the
+// kernel has ended, whatever starts early after it.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 struct DevMem {
   // Input is read exactly once: stream it with an evict-first hint.
   GB_HD static cf ldg(const cf* p, int64_t off) {
@@ -185,6 +193,7 @@ __device__ __forceinline__ void conv_tile(const cf* __restrict__ in, cf* out, co
 template <int R, int MAP, class TR>
 __global__ void __launch_bounds__(1024)
 stockham_conv(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc d) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cf* sm = reinterpret_cast<cf*>(smem_raw);
   for (int64_t tile = blockIdx.x; tile < d.tiles; tile += gridDim.x) {
@@ -218,6 +227,7 @@ stockham_grouped(const __grid_constant__ PassDesc d0, const __grid_constant__ Gr
 template <int R, int LMAP, int SMAP, class TR>
 __global__ void __launch_bounds__(1024)
 stockham_pass(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc d) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cf* sm = reinterpret_cast<cf*>(smem_raw);
   using B = PassBody<R, LMAP, SMAP, DevMem, TR>;
@@ -518,6 +528,7 @@ stockham_staged(const cf* __restrict__ in, cf* out, const __grid_constant__ Pass
   const bool one_arrival = SH::kG == 1 || SH::kRowsIn || d.tmap_in_ok;
   if (tid == 0) mbar_init(bar, one_arrival ? 1 : SH::kT);
   __syncthreads();
+  grid_wait();
   if (tile < d.tiles) stage_tile<SH>(st, in, d, tile, bar, tid);  // uniform over the block
   // twiddle roots: loaded once here (kHold, kHoldFused) or per tile
   constexpr bool kHold = SH::kHoldRoots && !CONV;

@@ -106,6 +106,7 @@ __device__ __forceinline__ void tc_stage_in(const cf* in, const PassDesc& d, int
 template <int LOGL, int PREC>
 __global__ void __launch_bounds__(256, 2)
 stockham_tc(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc d) {
+  grid_wait();
   constexpr int P = PREC == TC_BF16X3 ? TC_BF16 : PREC;
   using B = TcBody<LOGL, P, DevMem>;
   extern __shared__ __align__(16) unsigned char smem_tc[];

@@ -26,6 +26,7 @@ short_lines(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc
   extern __shared__ __align__(16) unsigned char smem_lines[];
   cf* sm = reinterpret_cast<cf*>(smem_lines);
   const int tid = threadIdx.x;
+  grid_wait();
   const int64_t at = (int64_t)blockIdx.x << 12, valid = d.count_inner - (int64_t)blockIdx.x * B::G;
   cf v[kJoinR];
   if (d.conj_in) B::template first_rows<true>(v, in + at, valid, tid);

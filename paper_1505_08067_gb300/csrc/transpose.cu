@@ -57,6 +57,7 @@ transpose_kernel(const void* __restrict__ in, void* __restrict__ out, int64_t ba
                  int64_t cols, int logN, int sign) {
   constexpr int WY = H || TW ? 4 : 8, PER = 32 / WY;
   __shared__ cf tile[32][33];
+  grid_wait();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x WY
   const int64_t trow = rows / 32, tcol = cols / 32, per = trow * tcol;
   for (int64_t t = blockIdx.x; t < batch * per; t += gridDim.x) {
@@ -107,8 +108,9 @@ cudaError_t launch_transpose(const void* in, void* out, int64_t batch, int64_t r
   const int per_sm = h16 || logN > 0 ? 16 : 8;
   const int grid =
       (int)std::min<int64_t>(tiles, (int64_t)(sm_count > 0 ? sm_count : 152) * per_sm);
-#define GB_TR(HH, TT) \
-  transpose_kernel<HH, TT><<<grid, HH || TT ? 128 : 256, 0, st>>>(in, out, batch, rows, cols, logN, sign)
+#define GB_TR(HH, TT)                                                                      \
+  return launch_early((const void*)transpose_kernel<HH, TT>, grid, HH || TT ? 128 : 256, 0, st, \
+                      in, out, batch, rows, cols, logN, sign)
   if (h16) {
     if (logN > 0) GB_TR(true, true);
     else GB_TR(true, false);
@@ -117,7 +119,6 @@ cudaError_t launch_transpose(const void* in, void* out, int64_t batch, int64_t r
     else GB_TR(false, false);
   }
 #undef GB_TR
-  return cudaGetLastError();
 }
 
 }  // namespace gbfft

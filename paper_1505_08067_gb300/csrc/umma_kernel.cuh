@@ -331,6 +331,7 @@ stockham_umma(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDe
   __syncthreads();
   tc05_fence_after();
   const uint32_t tmem = *tslot;
+  grid_wait();
   // the first tile's copy; `pending`: a copy is in flight that no wait has seen
   bool pending = staged && blockIdx.x < d.tiles;
   if (pending && tid == 0) stage_copy(blockIdx.x);
