@@ -168,11 +168,11 @@ cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, i
 }
 
 cudaError_t enqueue_tables(const PlanSpec& s, cf* tables, cudaStream_t st) {
-  for (const TwSegment& t : s.tables) {
-    cudaError_t e = launch_twiddle_gen(tables + t.off, t.count, t.den, t.mode, t.r, t.mult, st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  TwiddleList list{};
+  static_assert(decltype(s.tables)::capacity() <= 40, "every table fits the list");
+  for (const TwSegment& t : s.tables)
+    list.t[list.n++] = TwiddleTable{t.off, t.count, t.den, t.mult, t.mode, t.r};
+  return launch_twiddle_list(tables, list, st);
 }
 
 static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, const void* in,

@@ -38,15 +38,33 @@ __global__ void copy_kernel(const cf* __restrict__ in, cf* out, int64_t count, i
 //   mode 1 (power table):  exponent = j * mult
 // value = exp(-2 pi i * (exponent mod den) / den).  The exponent is reduced as
 // an integer, so sincospi receives an exact argument in [0, 2).
+__device__ __forceinline__ void twiddle_entry(float2* out, int64_t j, int64_t den, int mode, int r,
+                                              int64_t mult) {
+  int64_t e = (mode == 0) ? (j / r) * (j % r) : j * mult;
+  e %= den;
+  double s, c;
+  sincospi(2.0 * (double)e / (double)den, &s, &c);
+  out[j] = make_float2((float)c, (float)(-s));
+}
+
 __global__ void twiddle_gen(float2* out, int64_t count, int64_t den, int mode, int r,
                             int64_t mult) {
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    int64_t e = (mode == 0) ? (j / r) * (j % r) : j * mult;
-    e %= den;
-    double s, c;
-    sincospi(2.0 * (double)e / (double)den, &s, &c);
-    out[j] = make_float2((float)c, (float)(-s));
+       j += (int64_t)gridDim.x * blockDim.x)
+    twiddle_entry(out, j, den, mode, r, mult);
+}
+
+// Every table of a plan in one launch: blocks take 1024-entry pieces of the
+// tables in turn.
+__global__ void twiddle_gen_all(float2* out, const __grid_constant__ TwiddleList list) {
+  int64_t piece = blockIdx.x;
+  for (int i = 0; i < list.n; ++i) {
+    const TwiddleTable& t = list.t[i];
+    const int64_t pieces = (t.count + 1023) >> 10;
+    for (; piece < pieces; piece += gridDim.x)
+      for (int64_t j = (piece << 10) + threadIdx.x; j < t.count && j < (piece + 1) << 10; j += blockDim.x)
+        twiddle_entry(out + t.off, j, t.den, t.mode, t.r, t.mult);
+    piece -= pieces;
   }
 }
 
@@ -283,6 +301,14 @@ cudaError_t launch_copy(const void* in, void* out, int64_t count, int64_t in_str
   if (blocks > 65535) blocks = 65535;
   copy_kernel<<<(int)blocks, 256, 0, st>>>(static_cast<const cf*>(in), static_cast<cf*>(out),
                                            count, in_stride, out_stride);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_twiddle_list(void* out, const TwiddleList& list, cudaStream_t st) {
+  int64_t pieces = 0;
+  for (int i = 0; i < list.n; ++i) pieces += (list.t[i].count + 1023) >> 10;
+  if (pieces == 0) return cudaSuccess;
+  twiddle_gen_all<<<(int)std::min<int64_t>(pieces, 4096), 256, 0, st>>>(static_cast<float2*>(out), list);
   return cudaGetLastError();
 }
 

@@ -195,6 +195,16 @@ cudaError_t launch_grouped(int R, const PassDesc& d0, const GroupTable& gt, int 
                            size_t smem, cudaStream_t st);
 cudaError_t launch_copy(const void* in, void* out, int64_t count, int64_t in_stride,
                         int64_t out_stride, cudaStream_t st);
+// Twiddle tables (planner.h: TwSegment) at out + off, all in one launch.
+struct TwiddleTable {
+  int64_t off, count, den, mult;
+  int mode, r;
+};
+struct TwiddleList {
+  int n;
+  TwiddleTable t[40];
+};
+cudaError_t launch_twiddle_list(void* out, const TwiddleList& list, cudaStream_t st);
 cudaError_t launch_twiddle_gen(void* out, int64_t count, int64_t den, int mode, int r,
                                int64_t mult, cudaStream_t st);
 

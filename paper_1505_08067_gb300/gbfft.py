@@ -409,11 +409,37 @@ def fft_bandwidth_bound_gflops(n: int, gbs: float, bytes_per_sample: float = 8.0
 
 def _stream_handle(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+_tensor = None
+
+
+def _tensor_type():
+    global _tensor
+    if _tensor is None:
+        import torch
+        _tensor = torch.Tensor
+    return _tensor
+
+
+_raw_stream = None
+
+
+def _current_stream() -> int:
+    """torch's current stream as a cudaStream_t, without a Stream object where
+    torch has the raw call."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        get, dev = (getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        torch.cuda.init()
+        _raw_stream = (lambda: get(dev())) if get and dev else (
+            lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
 
 
 class Plan:
@@ -427,6 +453,16 @@ class Plan:
         self.precision = precision
         self.handle: Optional[int] = fft_plan_create(self.shape, self.batch, direction, precision,
                                                      **options)
+        self._prepare()
+
+    def _prepare(self):
+        """What every execute needs and no execute changes: its C entry point
+        and the type and size its tensors must have."""
+        import torch
+        self._execute = load().fft_execute
+        self._dtype = (torch.complex32 if self.precision == FFT_PREC_TC_FP16_C32
+                       else torch.complex64)
+        self._elements = self.elements
 
     @property
     def elements(self) -> int:
@@ -437,20 +473,28 @@ class Plan:
 
     def _check_tensor(self, t, name):
         import torch
-        want = torch.complex32 if self.precision == FFT_PREC_TC_FP16_C32 else torch.complex64
-        if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != want:
-            raise TypeError(f"{name} must be a CUDA {str(want).split('.')[-1]} tensor")
-        if not t.is_contiguous() or t.numel() != self.elements:
-            raise ValueError(f"{name} must be contiguous with {self.elements} elements")
+        if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != self._dtype:
+            raise TypeError(f"{name} must be a CUDA {str(self._dtype).split('.')[-1]} tensor")
+        if not t.is_contiguous() or t.numel() != self._elements:
+            raise ValueError(f"{name} must be contiguous with {self._elements} elements")
 
     def execute(self, x, out=None, stream=None):
         """Enqueue the transform of tensor ``x`` into ``out`` (allocated if None)."""
-        import torch
-        self._check_tensor(x, "input")
+        # host time of a small call is most of its time: the checks of
+        # _check_tensor without its calls, the C entry point bound once
+        if not (x.__class__ is _tensor_type() and x.is_cuda and x.dtype is self._dtype
+                and x.is_contiguous() and x.numel() == self._elements):
+            self._check_tensor(x, "input")
         if out is None:
+            import torch
             out = torch.empty_like(x)
-        self._check_tensor(out, "output")
-        fft_execute(self.handle, x.data_ptr(), out.data_ptr(), _stream_handle(stream))
+        if not (out.__class__ is _tensor_type() and out.is_cuda and out.dtype is self._dtype
+                and out.is_contiguous() and out.numel() == self._elements):
+            self._check_tensor(out, "output")
+        status = self._execute(self.handle, x.data_ptr(), out.data_ptr(),
+                               _current_stream() if stream is None else _stream_handle(stream))
+        if status:
+            _check(status)
         return out
 
     def execute_graph(self, x, out=None, stream=None):
@@ -520,6 +564,7 @@ class ConvPlan(Plan):
             self.filters.append(h)
             spec.append((h.data_ptr(), lines, scale))
         self.handle = fft_conv_plan_create(self.shape, self.batch, spec, **options)
+        self._prepare()
 
 
 # ----------------------------------------------------------------- serving --
