@@ -371,7 +371,7 @@ static int tc_cols_launches(const PlanSpec& s) {
 fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches) {
   if (!plan_ok(plan)) return fail(FFT_ERR_BAD_PLAN, "null or destroyed plan");
   if (!launches) return fail(FFT_ERR_INVALID_ARG, "launches is null");
-  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined ? 1 : plan->spec.tc_cols ? tc_cols_launches(plan->spec) : (int)plan->spec.passes.size();
+  *launches = plan->spec.batch == 0 ? 0 : plan->spec.joined && !plan->spec.join_apart ? 1 : plan->spec.tc_cols ? tc_cols_launches(plan->spec) : (int)plan->spec.passes.size();
   return FFT_OK;
 }
 

@@ -39,9 +39,10 @@ cudaError_t bind_launches(const PlanSpec& s, const Caps& caps, const cf* tables,
         l.specialised = true;
       } else {
         l.fn = resolve_kernel(l.R, l.lmap, l.smap, l.d, s.generic_only, &l.specialised);
-        if (p.line_off >= 0 && (!p.conv                ? resolve_lines(p.logL, &l)
-                                : p.lmap == MAP_ROWS ? resolve_conv_lines(p.logL, &l)
-                                                     : resolve_conv_cols(p.logL, &l)))
+        const bool rows = p.lmap == MAP_ROWS;
+        if (p.line_off >= 0 &&
+            (p.conv ? (rows ? resolve_conv_lines(p.logL, &l) : resolve_conv_cols(p.logL, &l))
+                    : (rows ? resolve_lines(p.logL, &l) : resolve_cols(p.logL, &l))))
           l.grid = lines_grid(l.d, l.lines);
       }
       cudaError_t e = prepare_launch(l);
@@ -155,7 +156,7 @@ cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, i
   const bool inv = s.direction == FFT_INVERSE;
   const cudaError_t e = s.dims == 2 ? prepare_joined_frames(l1, l0, s.join_tile_log, inv,
                                                             caps.sm_count, j)
-                                    : prepare_joined(l0 + l1, s.join_tile_log, inv,
+                                    : prepare_joined(l0 + l1, s.join_apart, inv,
                                                      caps.sm_count, j);
   if (e != cudaSuccess) return e;
   j->d.tw1 = tables + s.join_tw1;
@@ -208,7 +209,7 @@ static cudaError_t enqueue_range(const PlanSpec& s, const PassLaunch* launches, 
     // the output of one transform is written while the input of a later one is
     // still read: in place or apart, not partly overlapping
     const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out, bytes = (uintptr_t)(nb * E) * 8;
-    if (a == b || a + bytes <= b || b + bytes <= a)
+    if (joined->second || a == b || a + bytes <= b || b + bytes <= a)
       return launch_joined(*joined, nb, in, out, work, st);
   }
   // the second workspace buffer of six-step plans

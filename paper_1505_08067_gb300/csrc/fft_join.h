@@ -309,10 +309,10 @@ GB_UNROLL
   }
 
   // The second factor of the four-step twiddle, w_N^{col Ns i} of the last
-  // stage, for every column of the tile: st[i * G + c] (computed by one warp).
+  // stage, for every column of the tile: st[i * G + c], by `lanes` threads.
   static constexpr int kSteps = G * SH::radix(SH::kLast);
-  GB_HD static void steps(cf* st, int col0, int logN, int lane) {
-    for (int x = lane; x < kSteps; x += 32) {
+  GB_HD static void steps(cf* st, int col0, int logN, int lane, int lanes = 32) {
+    for (int x = lane; x < kSteps; x += lanes) {
       const int i = x / G, c = x - i * G;
       Mem::sts(st, x, Mem::rotor((int64_t)(col0 + c) * (i * SH::ns(SH::kLast)), logN));
     }
@@ -407,8 +407,8 @@ template <int TL> using Join128 = JoinShape<TL, 7, 4, 3>;
 template <int TL> using Join256 = JoinShape<TL, 8, 4, 4>;
 template <int TL> using Join512 = JoinShape<TL, 9, 5, 4>;
 template <int TL> using Join1024 = JoinShape<TL, 10, 5, 5>;
-// Every length a row (2^4 .. 2^13) or column (2^4 .. 2^11) pass of frames has,
-// and short lines (2^3 .. 2^10, lines.cu).
+// Lengths of row and column passes (2^4 .. 2^10 rows, 2^4 .. 2^11 columns in joined
+// frames; 2^3 .. 2^11 in lines.cu and conv_lines.cu).
 template <int TL, int LOGL> struct JoinLen;
 template <int TL> struct JoinLen<TL, 3> { using S = JoinShape<TL, 3, 1, 2>; };
 template <int TL> struct JoinLen<TL, 4> { using S = JoinShape<TL, 4, 2, 2>; };
@@ -419,8 +419,6 @@ template <int TL> struct JoinLen<TL, 8> { using S = Join256<TL>; };
 template <int TL> struct JoinLen<TL, 9> { using S = Join512<TL>; };
 template <int TL> struct JoinLen<TL, 10> { using S = Join1024<TL>; };
 template <int TL> struct JoinLen<TL, 11> { using S = JoinShape<TL, 11, 4, 4, 3>; };
-template <int TL> struct JoinLen<TL, 12> { using S = JoinShape<TL, 12, 4, 4, 4>; };
-template <int TL> struct JoinLen<TL, 13> { using S = JoinShape<TL, 13, 5, 4, 4>; };
 // TL: log2 of the tile (join_tile_log).
 template <int LOGN, int TL> struct JoinPair;
 template <int TL> struct JoinPair<15, TL> : JoinPairOf<Join128<TL>, Join256<TL>> {};
@@ -430,35 +428,34 @@ template <int TL> struct JoinPair<18, TL> : JoinPairOf<Join512<TL>, Join512<TL>>
 template <int TL> struct JoinPair<19, TL> : JoinPairOf<Join512<TL>, Join1024<TL>> {};
 template <int TL> struct JoinPair<20, TL> : JoinPairOf<Join1024<TL>, Join1024<TL>> {};
 constexpr int kJoinMinLog = 15, kJoinMaxLog = 20;
-// Tiles of a transform of 2^logn points in a batch of `elems` elements.  With
-// work for several tiles per block, the tile is the smallest whose row segments
-// are 128 bytes wide (64 in one of the two passes of 2^17 .. 2^19); with less,
-// smaller tiles spread it over more SMs (2^21 elements, 8192 against 4096 per
-// tile: 2^17 19.8 and 18.5 us, 2^18 20.5 and 20.1, 2^19 19.8 and 20.7).
-GB_HD constexpr int join_tile_log(int logn, int64_t elems) {
-  return elems < int64_t(1) << 22 ? (logn <= 18 ? 12 : 13) : logn <= 16 ? 12 : logn <= 19 ? 13 : 14;
+// Tiles of a transform of 2^logn points.  Joined, with work for several tiles per
+// block: the smallest whose row segments are 128 bytes wide (64 in one of the two
+// passes of 2^17 .. 2^19).  Apart, on fewer elements: smaller, over more SMs
+// (2^22 elements: 2^17 20.0 us against 24.1 for twice the tile, 2^18 21.7 and
+// 24.6, 2^20 26.1 and 30.4).
+GB_HD constexpr int join_tile_log(int logn, bool apart) {
+  return apart ? (logn <= 18 ? 12 : 13) : logn <= 16 ? 12 : logn <= 19 ? 13 : 14;
 }
 // log2 of the blocks per SM (512 threads of 32 elements in all).
 GB_HD constexpr int join_blocks_log(int tile_log) { return 14 - tile_log; }
-// Do such transforms run joined?  Measured against two launches: always faster
-// (2^17 x 1 13.8 -> 10.3 us, 2^18 x 2 16.5 -> 12.6; 2^15 alike) but for a little
-// over one wave of first-pass tiles, where the second pass then starts late
-// (2^20 elements: 2^16 14.4 -> 16.5 us, 2^18 16.5 -> 17.5, 2^20 18.4 -> 19.8).
-GB_HD constexpr bool join_transform(int logn, int64_t elems) {
-  return logn >= kJoinMinLog && logn <= kJoinMaxLog &&
-         (elems >= int64_t(1) << 21 || (logn > 15 && elems < int64_t(1) << 20));
-}
+// Such transforms run with the passes of this file: joined, or (join_apart) in
+// a launch each.  While the whole batch fits L2, so does the intermediate in any
+// order, and two launches that start early have no dispatching warp, no waits
+// and more registers.  Measured, the two-launch kernels before (launched early
+// too), apart, and joined: 2^15 x 1 5.7, 4.2, 8.3 us; 2^18 x 1 10.6, 5.4, 8.9;
+// 2^20 x 1 11.4, 8.2, 17.0; 2^18 x 16 34.0, 21.7, 28.2; 2^17 x 64 52.9, 37.4, 45.0;
+// 2^17 x 97 84.2, 63.0, 61.9; 2^17 x 128 110, 88, 78; 2^20 x 12 81, 75, 72.
+GB_HD constexpr bool join_transform(int logn) { return logn >= kJoinMinLog && logn <= kJoinMaxLog; }
+GB_HD constexpr bool join_apart(int64_t elems) { return elems < int64_t(3) << 22; }
 
-// Frames: rows of 2^lc, columns of 2^lr, `elems` elements in all.  The same
-// band is excluded where the passes had fast kernels (256 rows and fewer of 256
-// elements and more, and rows of 2048 and more: 16 x 1024 x 64 15.9 -> 16.7 us,
-// 512 x 2048 18.6 -> 19.4); 1.1 to 2.6 times faster elsewhere (64 x 64 x 64
-// 20.7 -> 10.4 us).
+// Frames: rows of 2^lc, columns of 2^lr, `elems` elements in all.  Below 2^23.6
+// elements the intermediate fits L2 in any order, and a launch per pass (lines.cu)
+// is up to twice as fast (1024 x 1024: 17.0 -> 9 us; 2^23 elements 5% to 20%); rows
+// of 2048 and more are faster in launches of their own at every size.
 GB_HD constexpr bool join_frame(int lr, int lc, int64_t elems) {
-  return lr >= 4 && lr <= 11 && lc >= 4 && lc <= 13 &&
-         ((lr > 8 ? lc < 11 : lc < 8) || elems < int64_t(1) << 20 || elems >= int64_t(1) << 21);
+  return lr >= 4 && lr <= 11 && lc >= 4 && lc <= 10 && elems >= int64_t(3) << 22;
 }
-GB_HD constexpr int join_frame_tile_log(int lr, int lc) { return lr <= 8 && lc <= 12 ? 12 : 13; }
+GB_HD constexpr int join_frame_tile_log(int lr) { return lr <= 8 ? 12 : 13; }
 
 // ------------------------------------------------------------- the order --
 // Tiles are handed out in one order to whichever block asks next (a counter),

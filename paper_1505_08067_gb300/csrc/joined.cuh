@@ -23,13 +23,12 @@
 // blocks, 352 us) and smaller blocks where segments stay wide (2^15, 2^16:
 // four 128-thread blocks, 242 / 245 us).
 //
+// Smaller batches run the same passes in a launch each (apart_first,
+// apart_second; join_apart says where the line lies).
 // Measured, 2^26 elements, before (two launches) and now: 2^15 349 -> 242 us,
 // 2^16 363 -> 245, 2^17 396 -> 275, 2^18 446 -> 289, 2^19 421 -> 302,
-// 2^20 368 -> 336; 2^21 elements 18.8-24.9 -> 18.7-22.3 us.  Below 2^21 elements
-// the tiles no longer fill the GPU and two launches of smaller tiles are
-// faster (2^20 elements: 14.3-18.3 against 16.6-20.7 us).  2^21 and 2^22, whose
-// 2048-point passes need three stages and 64-byte segments, measured slower
-// joined (384 against 371 us, 592 against 387 us).
+// 2^20 368 -> 330.  2^21 and 2^22, whose 2048-point passes need three stages and
+// 64-byte segments, measured slower joined (384 against 371 us, 592 against 387).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -250,6 +249,41 @@ joined_pass(const cf* in, cf* out, cf* work, const __grid_constant__ JoinDesc d)
   });
 }
 
+// The same passes in a launch each, a tile per block: transform b's intermediate
+// at work + b N.
+template <int LOGN, int TL, bool INV>
+__global__ void __launch_bounds__((1 << TL) / kJoinR, 1 << join_blocks_log(TL))
+apart_first(const cf* in, cf* work, const __grid_constant__ JoinDesc d) {
+  using PR = JoinPair<LOGN, TL>;
+  using B = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>;
+  extern __shared__ __align__(16) unsigned char smem_join[];
+  cf* sm = reinterpret_cast<cf*>(smem_join);
+  cf* steps = sm + B::kSlots;
+  const int tid = threadIdx.x, col0 = (int)(blockIdx.x & (PR::kTiles - 1)) * PR::kG1;
+  const int64_t at = (int64_t)(blockIdx.x / PR::kTiles) * PR::kN;
+  B::steps(steps, col0, LOGN, tid, PR::kThreads);
+  grid_wait();
+  cf v[kJoinR];
+  B::template first<INV, false>(v, in + at + col0, PR::kN2, tid);
+  join_stages<typename PR::P1, JOIN_FIRST, true>(v, sm, d.tw1, col0, LOGN, tid);
+  B::template store_block<PR::kG2>(v, work + at + col0 * PR::kG2, steps, PR::kN2, tid);
+}
+template <int LOGN, int TL, bool INV>
+__global__ void __launch_bounds__((1 << TL) / kJoinR, 1 << join_blocks_log(TL))
+apart_second(const cf* work, cf* out, const __grid_constant__ JoinDesc d) {
+  using PR = JoinPair<LOGN, TL>;
+  using B = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>;
+  extern __shared__ __align__(16) unsigned char smem_join[];
+  cf* sm = reinterpret_cast<cf*>(smem_join);
+  const int tid = threadIdx.x, tile = (int)(blockIdx.x & (PR::kTiles - 1));
+  const int64_t at = (int64_t)(blockIdx.x / PR::kTiles) * PR::kN;
+  grid_wait();
+  cf v[kJoinR];
+  B::template first<false, true>(v, work + at + tile * PR::kTile, PR::kG2, tid);
+  join_stages<typename PR::P2, JOIN_COLS, false>(v, sm, d.tw2, 0, 0, tid);
+  B::template store_cols<INV>(v, out + at + tile * PR::kG2, PR::kN1, tid);
+}
+
 // One tile of rows (from in to out) or of columns (in place) of frames.
 template <int TL, int LOGL, bool INV>
 __device__ __forceinline__ void join_rows(const cf* in, cf* out, const JoinDesc& d, int64_t tile,
@@ -281,10 +315,10 @@ __device__ __forceinline__ void join_cols(cf* buf, const JoinDesc& d, int64_t ti
 // 4096 rows and more (16 bytes) keep the staged column kernel and its tensor-map
 // loads.  Tiles of 4096 elements up to 256 rows (measured as for transforms
 // above), else 8192.
-// Measured, 2^25 elements, before (a launch per pass) and now: 16 x 16 390 ->
-// 139 us, 64 x 64 242 -> 123, 256 x 1024 201 -> 144, 512 x 512 247 -> 148,
-// 1024 x 1024 271 -> 161, 1024 x 8192 293 -> 223, 2048 x 1024 272 -> 209,
-// 2048 x 8192 297 -> 270; 2^21 elements: 20.6-39.9 -> 16.7-24.7 us.
+// Measured, 2^25 elements, before (a launch per pass), now a launch per pass
+// (lines.cu), and joined: 16 x 16 390, 158, 136 us, 64 x 64 242, 153, 120,
+// 256 x 1024 201, 159, 143, 512 x 1024 245, 166, 149, 1024 x 1024 271, 182, 158,
+// 2048 x 1024 272, 215, 206.
 template <int TL, bool INV>
 __global__ void __launch_bounds__((1 << TL) / kJoinR + 32, 1 << join_blocks_log(TL))
 joined_frames(const cf* in, cf* out, const __grid_constant__ JoinDesc d) {
@@ -323,11 +357,7 @@ joined_frames(const cf* in, cf* out, const __grid_constant__ JoinDesc d) {
         case 8: join_rows<TL, 8, INV>(in, out, d, tile, sm, tid); break;
         case 9: join_rows<TL, 9, INV>(in, out, d, tile, sm, tid); break;
         case 10: join_rows<TL, 10, INV>(in, out, d, tile, sm, tid); break;
-        case 11: join_rows<TL, 11, INV>(in, out, d, tile, sm, tid); break;
-        case 12: join_rows<TL, 12, INV>(in, out, d, tile, sm, tid); break;
-        default:
-          if constexpr (TL >= 13) join_rows<TL, 13, INV>(in, out, d, tile, sm, tid);
-          break;
+        default: break;
       }
     } else {
       switch (d.lr) {
@@ -351,17 +381,27 @@ joined_frames(const cf* in, cf* out, const __grid_constant__ JoinDesc d) {
 template <int LOGN, int TL>
 inline bool joined_fn(bool inv, JoinedLaunch& j) {
   using PR = JoinPair<LOGN, TL>;
-  using B1 = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>;
-  using B2 = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>;
+  constexpr int s1 = JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>::kSlots;
+  constexpr int s2 = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>::kSlots;
   j.fn = inv ? (const void*)joined_pass<LOGN, TL, true> : (const void*)joined_pass<LOGN, TL, false>;
-  j.smem = ((B1::kSlots > B2::kSlots ? B1::kSlots : B2::kSlots) + 2 * PR::kSteps) * sizeof(cf);
+  j.smem = ((s1 > s2 ? s1 : s2) + 2 * PR::kSteps) * sizeof(cf);
   j.block = PR::kThreads + 32;
   j.d.o.tpt_log = LOGN - TL;
-  j.tile_log = TL;
   j.n1 = PR::kN1;
   j.n2 = PR::kN2;
   j.g1 = PR::kG1;
   j.box_rows = PR::kN1 < 256 ? PR::kN1 : 256;
+  return true;
+}
+template <int LOGN, int TL>
+inline bool apart_fn(bool inv, JoinedLaunch& j) {
+  using PR = JoinPair<LOGN, TL>;
+  j.fn = inv ? (const void*)apart_first<LOGN, TL, true> : (const void*)apart_first<LOGN, TL, false>;
+  j.second = inv ? (const void*)apart_second<LOGN, TL, true> : (const void*)apart_second<LOGN, TL, false>;
+  j.smem = (JoinBody<typename PR::P1, JOIN_FIRST, JoinMem>::kSlots + PR::kSteps) * sizeof(cf);
+  j.second_smem = JoinBody<typename PR::P2, JOIN_COLS, JoinMem>::kSlots * sizeof(cf);
+  j.block = PR::kThreads;
+  j.d.o.tpt_log = LOGN - TL;
   return true;
 }
 
@@ -378,7 +418,7 @@ constexpr int join_frame_slots() {
 template <int TL>
 inline void joined_frames_fn(bool inv, JoinedLaunch& j) {
   j.fn = inv ? (const void*)joined_frames<TL, true> : (const void*)joined_frames<TL, false>;
-  j.smem = join_frame_slots<TL, 4, TL < 13 ? 12 : 13>() * sizeof(cf);
+  j.smem = join_frame_slots<TL, 4, 11>() * sizeof(cf);
   j.block = (1 << TL) / kJoinR + 32;
 }
 

@@ -1,20 +1,19 @@
-// Joined two-pass kernels of 2^18 .. 2^20 points (joined.cuh), and the launch.
+// Two-pass kernels, joined and apart, of 2^18 .. 2^20 points (joined.cuh), and the
+// launches.
 #include <algorithm>
 
 #include "joined.cuh"
 
 namespace gbfft {
 
-bool joined_kernel_a(int logn, int tile_log, bool inv, JoinedLaunch& j);
+bool joined_kernel_a(int logn, bool apart, bool inv, JoinedLaunch& j);
 void joined_frames_kernel(int tile_log, bool inv, JoinedLaunch& j);
 
-static bool joined_kernel_b(int logn, int tile_log, bool inv, JoinedLaunch& j) {
-  switch (logn * 100 + tile_log) {
-    case 1812: return joined_fn<18, 12>(inv, j);
-    case 1813: return joined_fn<18, 13>(inv, j);
-    case 1913: return joined_fn<19, 13>(inv, j);
-    case 2013: return joined_fn<20, 13>(inv, j);
-    case 2014: return joined_fn<20, 14>(inv, j);
+static bool joined_kernel_b(int logn, bool apart, bool inv, JoinedLaunch& j) {
+  switch (logn) {
+    case 18: return apart ? apart_fn<18, join_tile_log(18, true)>(inv, j) : joined_fn<18, join_tile_log(18, false)>(inv, j);
+    case 19: return apart ? apart_fn<19, join_tile_log(19, true)>(inv, j) : joined_fn<19, join_tile_log(19, false)>(inv, j);
+    case 20: return apart ? apart_fn<20, join_tile_log(20, true)>(inv, j) : joined_fn<20, join_tile_log(20, false)>(inv, j);
     default: return false;
   }
 }
@@ -31,15 +30,19 @@ static cudaError_t prepare(int sm_count, JoinedLaunch* j) {
   return cudaSuccess;
 }
 
-cudaError_t prepare_joined(int logn, int tile_log, bool inv, int sm_count, JoinedLaunch* j) {
-  if (!joined_kernel_a(logn, tile_log, inv, *j) && !joined_kernel_b(logn, tile_log, inv, *j))
+cudaError_t prepare_joined(int logn, bool apart, bool inv, int sm_count, JoinedLaunch* j) {
+  if (!joined_kernel_a(logn, apart, inv, *j) && !joined_kernel_b(logn, apart, inv, *j))
     return cudaErrorInvalidValue;
-  return prepare(sm_count, j);
+  j->tile_log = join_tile_log(logn, apart);
+  if (!apart) return prepare(sm_count, j);
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const cudaError_t e = cudaFuncSetAttribute(j->fn, attr, (int)j->smem);
+  return e == cudaSuccess ? cudaFuncSetAttribute(j->second, attr, (int)j->second_smem) : e;
 }
 
 cudaError_t prepare_joined_frames(int lr, int lc, int tl, bool inv, int sm_count,
                                   JoinedLaunch* j) {
-  if (!join_frame(lr, lc, 0) || tl != join_frame_tile_log(lr, lc)) return cudaErrorInvalidValue;
+  if (!join_frame(lr, lc, int64_t(1) << 40) || tl != join_frame_tile_log(lr)) return cudaErrorInvalidValue;
   joined_frames_kernel(tl, inv, *j);
   j->frames = true;
   j->tile_log = tl;
@@ -54,6 +57,15 @@ cudaError_t launch_joined(const JoinedLaunch& j, int64_t batch, const void* in, 
   if (!j.fn || batch < 1) return cudaErrorInvalidValue;
   JoinDesc d = j.d;
   d.o.nb = batch;
+  if (j.second) {
+    const int64_t tiles = batch << d.o.tpt_log;
+    if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    const cudaError_t e = launch_early(j.fn, (int)tiles, j.block, j.smem, st,
+                                       static_cast<const cf*>(in), static_cast<cf*>(work), d);
+    if (e != cudaSuccess) return e;
+    return launch_early(j.second, (int)tiles, j.block, j.second_smem, st,
+                        static_cast<const cf*>(work), static_cast<cf*>(out), d);
+  }
   if (j.frames) {
     d.total = batch << (d.lr + d.lc);
     const int unit = j.tile_log + d.o.tpt_log;

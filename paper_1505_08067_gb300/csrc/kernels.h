@@ -28,6 +28,8 @@ struct JoinDesc {
 struct JoinedLaunch {
   const void* fn = nullptr;  // null: the plan's passes run as launches of their own
   bool frames = false;
+  const void* second = nullptr;  // passes apart (join_apart): fn is the first, this the second
+  size_t second_smem = 0;
   int max_grid = 0;          // resident blocks
   int block = 0;
   size_t smem = 0;
@@ -35,9 +37,9 @@ struct JoinedLaunch {
   int n1 = 0, n2 = 0, g1 = 0, box_rows = 0;
   JoinDesc d{};
 };
-// Kernel for transforms of 2^logn, or frames of 2^lr x 2^lc, in tiles of
-// 2^tile_log, its opt-in shared memory, resident blocks and tiles per unit.
-cudaError_t prepare_joined(int logn, int tile_log, bool inverse, int sm_count, JoinedLaunch* j);
+// Kernel (apart: kernels) for transforms of 2^logn, or frames of 2^lr x 2^lc in
+// tiles of 2^tile_log, its opt-in shared memory, resident blocks and tiles per unit.
+cudaError_t prepare_joined(int logn, bool apart, bool inverse, int sm_count, JoinedLaunch* j);
 cudaError_t prepare_joined_frames(int lr, int lc, int tile_log, bool inverse, int sm_count,
                                   JoinedLaunch* j);
 // `batch` transforms or frames; `work`: the ring of a four-step plan.
@@ -175,6 +177,8 @@ cudaError_t launch_transpose(const void* in, void* out, int64_t batch, int64_t r
 // The short-line kernel of a contiguous pass of 2^logL points (lines.cu): sets
 // fn, block and smem; false if there is none.
 bool resolve_lines(int logL, PassLaunch* l);
+// The same for the column pass of frames of 2^logL rows (lines.cu).
+bool resolve_cols(int logL, PassLaunch* l);
 // The same for fast convolution (conv_lines.cu): contiguous lines, and the
 // columns of frames.
 bool resolve_conv_lines(int logL, PassLaunch* l);

@@ -1,6 +1,7 @@
 // Batches of short contiguous transforms (2^3 .. 2^10 points): a tile of 4096
 // elements per 128-thread block as a row pass of fft_join.h, 32 elements and one
-// exchange per thread.
+// exchange per thread; and the column passes of frames of 2^3 .. 2^11 rows in the
+// same way.
 //
 // Lengths below 256 ran the run-time-parameter kernel, bound by its address
 // arithmetic and, at 16 points (one transform per thread), by loads that touch
@@ -14,6 +15,9 @@
 // less below 2^19 elements (6.2 -> 4.2 us), where 128-thread blocks of one
 // exchange finish sooner.  Not 4 points (272 -> 283 us: two lanes per
 // transform), nor 2048 and 4096 (166 -> 171, 164 -> 186: a third stage).
+// Columns : 2^20
+// elements, both passes of 512 x 2048 17.6 us joined, 15.1 with the kernels before,
+// 8.7 now; 256 x 256 x 16 14.8, 11.5, 7.2; 2^25 elements of 64 x 64 242 -> 153.
 #include "joined.cuh"
 
 namespace gbfft {
@@ -43,6 +47,48 @@ static bool lines_fn(PassLaunch* l) {
   l->block = 128;
   l->lines = 12;
   return true;
+}
+
+// Columns of 2^LOGL rows of d.in.e elements, in place or not.
+template <int TL, int LOGL>
+__global__ void __launch_bounds__((1 << TL) / kJoinR, 1 << join_blocks_log(TL))
+short_cols(const cf* in, cf* out, const __grid_constant__ PassDesc d) {
+  using SH = typename JoinLen<TL, LOGL>::S;
+  using B = JoinBody<SH, JOIN_COLS, JoinMem>;
+  extern __shared__ __align__(16) unsigned char smem_lines[];
+  cf* sm = reinterpret_cast<cf*>(smem_lines);
+  const int tid = threadIdx.x, lc = 31 - __clz((int)d.in.e);
+  const int64_t col0 = (int64_t)blockIdx.x * B::G, cols = d.tiles / d.tiles_inner * d.count_inner;
+  grid_wait();
+  cf v[kJoinR];
+  B::first_frame(v, in, col0, cols, lc, tid);
+  join_stages<SH, JOIN_COLS, false>(v, sm, d.tw + d.tw_line, 0, 0, tid);
+  if (d.conj_out) B::template store_frame<true>(v, out, col0, cols, lc, tid);
+  else B::template store_frame<false>(v, out, col0, cols, lc, tid);
+}
+
+template <int TL, int LOGL>
+static bool cols_fn(PassLaunch* l) {
+  l->fn = (const void*)short_cols<TL, LOGL>;
+  l->smem = JoinBody<typename JoinLen<TL, LOGL>::S, JOIN_COLS, JoinMem>::kSlots * sizeof(cf);
+  l->block = (1 << TL) / kJoinR;
+  l->lines = TL;
+  return true;
+}
+
+bool resolve_cols(int logL, PassLaunch* l) {
+  switch (logL) {
+    case 3: return cols_fn<12, 3>(l);
+    case 4: return cols_fn<12, 4>(l);
+    case 5: return cols_fn<12, 5>(l);
+    case 6: return cols_fn<12, 6>(l);
+    case 7: return cols_fn<12, 7>(l);
+    case 8: return cols_fn<12, 8>(l);
+    case 9: return cols_fn<13, 9>(l);
+    case 10: return cols_fn<13, 10>(l);
+    case 11: return cols_fn<13, 11>(l);
+    default: return false;
+  }
 }
 
 bool resolve_lines(int logL, PassLaunch* l) {

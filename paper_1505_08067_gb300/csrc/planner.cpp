@@ -487,8 +487,10 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       const int64_t chunk = two_pass_chunk(N);
       s.chunk_batch = batch > chunk ? chunk : 0;
       s.work_elems = std::min(batch, chunk) * N;
-      if (defaults && batch > 0 && join_transform(logN, s.work_elems))
-        plan_joined(s, logN, join_tile_log(logN, s.work_elems), std::min(batch, chunk), caps);
+      if (defaults && batch > 0 && join_transform(logN)) {
+        s.join_apart = join_apart(s.work_elems);
+        plan_joined(s, logN, join_tile_log(logN, s.join_apart), std::min(batch, chunk), caps);
+      }
     }
   } else {
     const int64_t rows = n[0], cols = n[1];
@@ -529,7 +531,7 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       s.passes.push_back(p);
     }
     if (defaults && batch > 0 && join_frame(lr, lc, batch << (lr + lc)))
-      plan_joined(s, lr + lc, join_frame_tile_log(lr, lc), batch, caps);
+      plan_joined(s, lr + lc, join_frame_tile_log(lr), batch, caps);
   }
 
   // launch shapes and twiddle tables
@@ -570,13 +572,15 @@ void make_plan(PlanSpec& s, const int64_t* n, int dims, int64_t batch, int direc
       off = (off + 1) & ~int64_t(1);
     }
   }
-  for (auto& p : s.passes)
-    if (defaults && p.kind == PASS_FFT && (p.batch_is_tiles || p.conv) && !p.tc_prec &&
-        p.logL >= 3 && p.logL <= (p.conv ? 11 : 10)) {
-      p.line_off = off;
-      s.tables.push_back(TwSegment{off, int64_t(1) << p.logL, int64_t(1) << p.logL, 1, 1, 1});
-      off += int64_t(1) << p.logL;
-    }
+  // passes of the one-exchange line and column kernels (lines.cu, conv_lines.cu)
+  for (auto& p : s.passes) {
+    if (!defaults || p.kind != PASS_FFT || p.tc_prec) continue;
+    const bool cols = dims == 2 && p.lmap == MAP_COLS && (p.conv || p.count_inner > 1);
+    if ((!p.batch_is_tiles && !cols) || p.logL < 3 || p.logL > (p.conv || cols ? 11 : 10)) continue;
+    p.line_off = off;
+    s.tables.push_back(TwSegment{off, int64_t(1) << p.logL, int64_t(1) << p.logL, 1, 1, 1});
+    off += int64_t(1) << p.logL;
+  }
   if (s.joined) {
     const int64_t L1 = int64_t(1) << s.passes[0].logL, L2 = int64_t(1) << s.passes[1].logL;
     s.join_tw1 = off;
@@ -643,7 +647,7 @@ std::string describe(const PlanSpec& s) {
     << ",\"precision\":" << s.precision << ",\"max_block_log2\":" << s.max_block_log2
     << ",\"generic\":" << (s.generic_only ? 1 : 0) << ",\"conv\":" << (s.conv ? 1 : 0)
     << ",\"workspace_bytes\":" << s.work_elems * 8 << ",\"table_elems\":" << s.table_elems
-    << ",\"chunk_batch\":" << s.chunk_batch << ",\"joined\":" << (s.joined ? 1 : 0)
+    << ",\"chunk_batch\":" << s.chunk_batch << ",\"joined\":" << (s.joined && !s.join_apart ? 1 : 0) << ",\"apart\":" << (s.join_apart ? 1 : 0)
     << ",\"tc_columns\":" << (s.tc_cols ? 1 : 0)
     << ",\"passes\":[";
   for (size_t i = 0; i < s.passes.size(); ++i) {

@@ -122,6 +122,7 @@ struct PlanSpec {
   // plans whose two passes run as one launch (fft_join.h): the order of its
   // tiles and the offsets of its twiddle tables w_L^j for the passes' lengths
   bool joined = false;
+  bool join_apart = false;  // the same passes in a launch each (joined is set too)
   int64_t join_lag = 1;
   int join_ring = 1, join_tile_log = 0;
   int64_t join_tw1 = 0, join_tw2 = 0;

@@ -236,10 +236,10 @@ int64_t run_frames(int64_t batch, int lr, int lc, const cf* in, cf* out) {
     switch (k.pass ? 100 + lr : lc) {
 #define GB_R(L) case L: rows<TL, L, INV>(in, mid.data(), total, at, sm.data()); break;
 #define GB_C(L) case 100 + L: cols<TL, L, INV>(mid.data(), out, total, at, lc, sm.data()); break;
-      GB_R(4) GB_R(5) GB_R(6) GB_R(7) GB_R(8) GB_R(9) GB_R(10) GB_R(11) GB_R(12)
+      GB_R(4) GB_R(5) GB_R(6) GB_R(7) GB_R(8) GB_R(9) GB_R(10)
       GB_C(4) GB_C(5) GB_C(6) GB_C(7) GB_C(8)
       default:
-        if constexpr (TL == 13) switch (k.pass ? 100 + lr : lc) { GB_R(13) GB_C(9) GB_C(10) GB_C(11) default: break; }
+        if constexpr (TL == 13) switch (k.pass ? 100 + lr : lc) { GB_C(9) GB_C(10) GB_C(11) default: break; }
 #undef GB_R
 #undef GB_C
     }
@@ -324,8 +324,8 @@ extern "C" int64_t join_run_frames(int64_t batch, int lr, int lc, int inverse, c
                                    float* out, char* msg, size_t len) {
   const cf* x = reinterpret_cast<const cf*>(in);
   cf* y = reinterpret_cast<cf*>(out);
-  if (!join_frame(lr, lc, 0)) return -1;
-  const int64_t e = join_frame_tile_log(lr, lc) == 12
+  if (!join_frame(lr, lc, int64_t(1) << 40)) return -1;
+  const int64_t e = join_frame_tile_log(lr) == 12
                         ? (inverse ? run_frames<12, true>(batch, lr, lc, x, y) : run_frames<12, false>(batch, lr, lc, x, y))
                         : (inverse ? run_frames<13, true>(batch, lr, lc, x, y) : run_frames<13, false>(batch, lr, lc, x, y));
   snprintf(msg, len, "%s", g.first.c_str());

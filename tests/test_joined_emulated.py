@@ -53,8 +53,8 @@ def test_joined(oracle, joined, logn, tile, batch, lag, ring, direction):
 # every column length and row length, frames smaller than a tile with a ragged
 # last one, both tile sizes
 @pytest.mark.parametrize("lr,lc,batch", [(4, 4, 37), (5, 6, 7), (6, 5, 3), (7, 7, 2), (8, 8, 2),
-                                         (4, 12, 2), (9, 4, 3), (10, 5, 2), (11, 6, 1), (8, 9, 1),
-                                         (5, 10, 2), (4, 11, 1), (5, 13, 1), (9, 9, 1), (10, 4, 5)])
+                                         (9, 4, 3), (10, 5, 2), (11, 6, 1), (8, 9, 1), (5, 10, 2),
+                                         (9, 9, 1), (10, 4, 5)])
 @pytest.mark.parametrize("direction", [-1, 1])
 def test_joined_frames(oracle, joined, lr, lc, batch, direction):
     x = synth.uniform(80 + lr, batch, 2 ** (lr + lc)).reshape(batch, 2 ** lr, 2 ** lc)

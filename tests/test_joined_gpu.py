@@ -1,7 +1,7 @@
-"""The joined two-pass kernel (both passes of 2^15 .. 2^20 in one launch) at the
-edges of its range: the smallest batches that take it, ragged batches whose ring
-of workspace slots wraps, in place, buffers that are only 8-byte aligned,
-repeated and overlapping-buffer calls, against the FP64 oracle."""
+"""The passes of 2^15 .. 2^20, joined in one launch or in a launch each, and those
+of frames, at the edges of their ranges: the smallest batches, ragged batches
+whose ring of workspace slots wraps, in place, buffers that are only 8-byte
+aligned, repeated and overlapping-buffer calls, against the FP64 oracle."""
 import numpy as np
 import pytest
 
@@ -16,18 +16,23 @@ def _check(oracle, y, x_np, idx, direction, logn):
     assert np.max(oracle.rel_l2(y[torch.from_numpy(idx).cuda()].cpu().numpy(), ref)) <= 1e-6 * logn
 
 
-@pytest.mark.parametrize("logn,batch", [(15, 64), (15, 391), (16, 7), (16, 193), (17, 1),
-                                        (17, 16), (17, 75), (18, 1), (18, 3), (18, 39), (19, 1),
-                                        (19, 4), (19, 17), (20, 2), (20, 3), (20, 9)])
+# joined: the smallest batches that are, and larger ones; apart: one transform to
+# the largest batches
+@pytest.mark.parametrize("logn,batch", [(15, 391), (16, 193), (17, 97), (17, 131), (18, 49), (19, 25),
+                                        (20, 12), (20, 13), (15, 1), (15, 3), (15, 64), (16, 7),
+                                        (17, 1), (17, 75), (18, 1), (18, 47), (19, 1), (19, 3),
+                                        (20, 1), (20, 11)])
 @pytest.mark.parametrize("direction", [-1, 1])
 def test_joined(gb, oracle, logn, batch, direction):
+    joined = batch << logn >= 3 << 22
     n = 2 ** logn
     x_np = synth.uniform(700 + logn, batch, n)
     idx = np.unique([0, batch // 2, batch - 1])
     buf = torch.empty(batch * n + 1, dtype=torch.complex64, device="cuda")
     s = torch.cuda.current_stream().cuda_stream
     with gb.Plan(n, batch, direction) as p:
-        assert p.describe()["joined"] == 1 and p.launch_count == 1
+        d = p.describe()
+        assert (d["joined"], d["apart"], p.launch_count) == ((1, 0, 1) if joined else (0, 1, 2))
         first = None
         for shift in (0, 1):  # 16-byte and 8-byte aligned input
             x = buf[shift:shift + batch * n].view(batch, n)
@@ -42,29 +47,30 @@ def test_joined(gb, oracle, logn, batch, direction):
         assert torch.equal(first, x)
 
 
-@pytest.mark.parametrize("logn,batch", [(15, 1), (15, 63), (16, 16), (18, 4), (20, 1), (21, 2)])
+@pytest.mark.parametrize("logn,batch", [(14, 1000), (21, 8)])
 def test_not_joined(gb, logn, batch):
     with gb.Plan(2 ** logn, batch) as p:
-        assert p.describe()["joined"] == 0 and p.launch_count == 2
+        assert p.describe()["joined"] == 0 and p.describe()["apart"] == 0
 
 
-def test_partly_overlapping_buffers(gb, oracle):
+@pytest.mark.parametrize("batch", [40, 193])
+def test_partly_overlapping_buffers(gb, oracle, batch):
     """Output one transform after the input: the passes run apart, so that all
     of the input is read before any output is written."""
-    logn, batch = 16, 40
+    logn = 16
     n = 2 ** logn
     x_np = synth.uniform(771, batch, n)
     buf = torch.empty((batch + 1) * n, dtype=torch.complex64, device="cuda")
     buf[:batch * n].copy_(torch.from_numpy(x_np).view(-1))
     with gb.Plan(n, batch) as p:
-        assert p.describe()["joined"] == 1
+        assert p.describe()["joined"] == (1 if batch == 193 else 0)
         p.execute(buf[:batch * n], buf[n:])
         torch.cuda.synchronize()
     _check(oracle, buf[n:].view(batch, n), x_np, np.array([0, 1, batch - 1]), -1, logn)
 
 
 def test_two_plans_on_two_streams(gb, oracle):
-    logn, batch = 17, 40
+    logn, batch = 17, 100
     n = 2 ** logn
     xs = [torch.from_numpy(synth.uniform(780 + i, batch, n)).cuda() for i in range(2)]
     streams = [torch.cuda.Stream() for _ in xs]
@@ -80,11 +86,14 @@ def test_two_plans_on_two_streams(gb, oracle):
         assert all(torch.equal(a, b) for a, b in zip(want, got))
 
 
-@pytest.mark.parametrize("shape,batch", [((16, 16), 1), ((16, 16), 8193), ((64, 64), 3),
-                                         ((1024, 16), 1), ((32, 64), 1031), ((64, 128), 257),
+# joined frames, then frames whose passes are launches of the short-line kernels
+@pytest.mark.parametrize("shape,batch", [((16, 16), 49153), ((32, 64), 6145), ((64, 128), 1537),
+                                         ((512, 16), 1537), ((128, 32), 3073), ((1024, 512), 25),
+                                         ((2048, 16), 385), ((256, 256), 193), ((512, 1024), 24),
+                                         ((8, 4), 3), ((16, 16), 1), ((16, 16), 8193), ((64, 64), 3),
+                                         ((32, 64), 1031), ((64, 128), 257), ((1024, 16), 1),
                                          ((512, 16), 257), ((256, 8192), 1), ((16, 4096), 33),
-                                         ((32, 2048), 35), ((128, 32), 513), ((1024, 512), 5),
-                                         ((2048, 16), 65), ((2048, 2048), 1), ((256, 256), 33)])
+                                         ((1024, 512), 5), ((2048, 16), 65), ((2048, 2048), 1)])
 @pytest.mark.parametrize("direction", [-1, 1])
 def test_joined_frames(gb, oracle, shape, batch, direction):
     """Frames smaller than a tile with a ragged last one, frames of one tile and
@@ -95,7 +104,8 @@ def test_joined_frames(gb, oracle, shape, batch, direction):
     buf = torch.empty(batch * n + 1, dtype=torch.complex64, device="cuda")
     s = torch.cuda.current_stream().cuda_stream
     with gb.Plan(shape, batch, direction) as p:
-        assert p.describe()["joined"] == 1 and p.launch_count == 1
+        d = p.describe()
+        assert d["joined"] == (1 if batch * n >= 3 << 22 else 0) and d["kernels"][1]["lines"] == 1
         first = None
         for shift in (0, 1):
             x = buf[shift:shift + batch * n].view((batch,) + shape)
@@ -112,8 +122,8 @@ def test_joined_frames(gb, oracle, shape, batch, direction):
     assert np.max(oracle.rel_l2(got, ref)) <= 1e-6 * np.log2(n)
 
 
-@pytest.mark.parametrize("shape,batch", [((8, 4096), 80), ((256, 256), 16), ((4096, 512), 1),
-                                         ((64, 16384), 3), ((4096, 8192), 1)])
+@pytest.mark.parametrize("shape,batch", [((512, 16), 1535), ((8, 4096), 800), ((4096, 512), 10),
+                                         ((64, 2048), 100), ((64, 16384), 30)])
 def test_frames_not_joined(gb, shape, batch):
     with gb.Plan(shape, batch) as p:
         assert p.describe()["joined"] == 0 and p.launch_count == 2
