@@ -223,10 +223,13 @@ GBFFT_API fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches);
  * TMA / cp.async staged kernel, used when the source is 16-byte aligned, else
  * the compile-time kernel of the shape), "compile_time", "generic",
  * "tensor_core" or "copy" -- with its persistent-grid size and L2-prefetch
- * flag, and "lines": 1 when the short-line kernel (contiguous transforms of
- * 2^3 .. 2^10 points; fast convolution of lines and columns of 2^3 .. 2^11;
- * default options) runs the pass instead; "joined": 1 when both passes of a two-pass or 2D plan run as one launch
- * of a joined kernel, "apart": 1 when they are that kernel's passes in a launch each, 0 when each runs the kernel named for it) written to buf (NUL-terminated, truncated to len).  Returns
+ * flag, and "lines": 1 when the one-exchange kernel (default options: contiguous
+ * transforms of 2^3 .. 2^10 points, frame columns and fast convolution of 2^3 ..
+ * 2^11) runs the pass instead; "joined": 1 when both passes of a two-pass or 2D
+ * plan run as one launch of a joined kernel (2D: on the first stream that executes
+ * the plan; on others, and in graphs, each pass is a launch), "apart": 1 when they
+ * are that kernel's passes in a launch each, 0 when each runs the kernel named for
+ * it) written to buf (NUL-terminated, truncated to len).  Returns
  * FFT_ERR_INVALID_ARG if buf is too small for the whole text.
  */
 GBFFT_API fft_status_t fft_plan_describe(fft_plan_t plan, char* buf, size_t len);

@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -52,6 +53,7 @@ struct fft_plan_s {
   void* work = nullptr;    // cf[spec.work_elems]
   PassLaunch launches[kMaxPasses];  // whole-batch launches, device pointers filled
   JoinedLaunch joined;              // both passes of a two-pass plan as one launch
+  std::atomic<uint64_t> join_stream{0};  // id + 1 of the stream of a joined frame plan
   // lazily created resources of fft_execute_host
   cudaStream_t s_h2d = nullptr, s_k = nullptr, s_d2h = nullptr;
   cudaEvent_t ev_start = nullptr, ev_h2d = nullptr, ev_k = nullptr, ev_end = nullptr;
@@ -73,6 +75,24 @@ struct fft_plan_s {
 namespace {
 
 bool plan_ok(fft_plan_t p) { return p && p->magic == kMagic; }
+
+// The joined launch of an execution on st, or null for a launch per pass.  Its
+// tile counters are the plan's, so two of them must not overlap.  Four-step plans
+// have a workspace and may not overlap anyway; executions of frames may, on
+// several streams or as replays of several graphs.  So a frame plan is joined on
+// the first stream that runs it (ids, unlike handles, are not used again), and
+// nowhere else, nor in a capture, whose graph may be launched on any stream.
+const JoinedLaunch* joined_for(fft_plan_t p, cudaStream_t st) {
+  if (!p->joined.frames) return &p->joined;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+      cudaStreamGetId(st, &id) != cudaSuccess)
+    return nullptr;
+  uint64_t owner = 0;
+  if (p->join_stream.compare_exchange_strong(owner, id + 1)) owner = id + 1;
+  return owner == id + 1 ? &p->joined : nullptr;
+}
 
 fft_status_t query_caps(Caps& caps, int& device) {
   cudaError_t e = cudaGetDevice(&device);
@@ -203,7 +223,8 @@ fft_status_t fft_execute(fft_plan_t plan, const void* in, void* out, void* strea
     return fail(FFT_ERR_BAD_PLAN, "plan was created on device %d, current device is %d",
                 plan->device, dev);
   e = enqueue_passes(plan->spec, plan->launches, in, out, plan->work, 0, plan->spec.batch,
-                     static_cast<cudaStream_t>(stream), -1, &plan->joined);
+                     static_cast<cudaStream_t>(stream), -1,
+                     joined_for(plan, static_cast<cudaStream_t>(stream)));
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return FFT_OK;
 }
@@ -261,7 +282,7 @@ fft_status_t fft_execute_host(fft_plan_t plan, const void* host_in, void* host_o
     // the chunks run one after the other on s_k, so each reuses the workspace
     // from its start
     e = enqueue_passes(s, plan->launches, di + off, dout + off, wk, b0, nb, plan->s_k, -1,
-                       &plan->joined);
+                       joined_for(plan, plan->s_k));
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     cudaEventRecord(plan->ev_k, plan->s_k);
     cudaStreamWaitEvent(plan->s_d2h, plan->ev_k, 0);
@@ -303,7 +324,8 @@ fft_status_t fft_execute_graph(fft_plan_t plan, const void* in, void* out, void*
     e = cudaStreamBeginCapture(plan->s_capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "begin capture");
     cudaError_t le = enqueue_passes(plan->spec, plan->launches, in, out, plan->work, 0,
-                                    plan->spec.batch, plan->s_capture, -1, &plan->joined);
+                                    plan->spec.batch, plan->s_capture, -1,
+                                    joined_for(plan, plan->s_capture));
     e = cudaStreamEndCapture(plan->s_capture, &graph);
     if (le != cudaSuccess || e != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);

@@ -15,9 +15,9 @@
 // less below 2^19 elements (6.2 -> 4.2 us), where 128-thread blocks of one
 // exchange finish sooner.  Not 4 points (272 -> 283 us: two lanes per
 // transform), nor 2048 and 4096 (166 -> 171, 164 -> 186: a third stage).
-// Columns : 2^20
-// elements, both passes of 512 x 2048 17.6 us joined, 15.1 with the kernels before,
-// 8.7 now; 256 x 256 x 16 14.8, 11.5, 7.2; 2^25 elements of 64 x 64 242 -> 153.
+// Columns, both passes of frames, before (joined below 2^21 elements) and now:
+// 2^20 elements of 512 x 2048 15.1 -> 8.7 us, of 256 x 256 11.5 -> 7.2; 2^25 of
+// 64 x 64 242 -> 153.
 #include "joined.cuh"
 
 namespace gbfft {

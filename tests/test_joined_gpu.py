@@ -86,6 +86,34 @@ def test_two_plans_on_two_streams(gb, oracle):
         assert all(torch.equal(a, b) for a, b in zip(want, got))
 
 
+def test_one_frame_plan_on_two_streams(gb):
+    """Frame plans have no workspace: executions on several streams may overlap."""
+    shape, batch = (512, 256), 100
+    xs = [torch.from_numpy(synth.uniform(790 + i, batch, shape[0] * shape[1])).cuda()
+          .view((batch,) + shape) for i in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    with gb.Plan(shape, batch) as p:
+        assert p.describe()["joined"] == 1
+        want = [p.execute(x, stream=streams[0]) for x in xs]
+        torch.cuda.synchronize()
+        got = [torch.empty_like(x) for x in xs]
+        for _ in range(8):
+            for x, y, s in zip(xs, got, streams):
+                p.execute(x, y, stream=s)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
+        gb.fft_plan_sync_status(p.handle, streams[0].cuda_stream)
+        # a graph of one execution beside the other on a stream
+        got = [torch.empty_like(x) for x in xs]
+        for _ in range(4):
+            p.execute_graph(xs[1], got[1], stream=streams[1])
+            p.execute(xs[0], got[0], stream=streams[0])
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
+        gb.fft_plan_sync_status(p.handle, streams[0].cuda_stream)
+
+
 # joined frames, then frames whose passes are launches of the short-line kernels
 @pytest.mark.parametrize("shape,batch", [((16, 16), 49153), ((32, 64), 6145), ((64, 128), 1537),
                                          ((512, 16), 1537), ((128, 32), 3073), ((1024, 512), 25),
