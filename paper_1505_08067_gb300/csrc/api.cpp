@@ -165,14 +165,14 @@ fft_status_t build_plan(fft_plan_t* out, const int64_t* n, int dims, int64_t bat
     }
   }
   // tables on the legacy stream, waited for alone (work of the caller on
-  // non-blocking streams is not waited for)
+  // non-blocking streams is not waited for), after the kernels are looked up
   e = enqueue_tables(spec, static_cast<cf*>(p->tables), 0);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   if (e == cudaSuccess)
     e = bind_launches(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status, p->launches);
   if (e == cudaSuccess && spec.joined)
     e = bind_joined(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status,
                     reinterpret_cast<unsigned*>(p->status + 4), &p->joined);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   if (e != cudaSuccess) {
     fft_plan_destroy(p);
     return cuda_fail(e, "twiddle generation");

@@ -54,16 +54,17 @@ __global__ void twiddle_gen(float2* out, int64_t count, int64_t den, int mode, i
     twiddle_entry(out, j, den, mode, r, mult);
 }
 
-// Every table of a plan in one launch: blocks take 1024-entry pieces of the
-// tables in turn.
+// Every table of a plan in one launch: blocks take 256-entry pieces of the
+// tables in turn, an entry per thread (the FP64 sincospi is one long chain).
 __global__ void twiddle_gen_all(float2* out, const __grid_constant__ TwiddleList list) {
   int64_t piece = blockIdx.x;
   for (int i = 0; i < list.n; ++i) {
     const TwiddleTable& t = list.t[i];
-    const int64_t pieces = (t.count + 1023) >> 10;
-    for (; piece < pieces; piece += gridDim.x)
-      for (int64_t j = (piece << 10) + threadIdx.x; j < t.count && j < (piece + 1) << 10; j += blockDim.x)
-        twiddle_entry(out + t.off, j, t.den, t.mode, t.r, t.mult);
+    const int64_t pieces = (t.count + 255) >> 8;
+    for (; piece < pieces; piece += gridDim.x) {
+      const int64_t j = (piece << 8) + threadIdx.x;
+      if (j < t.count) twiddle_entry(out + t.off, j, t.den, t.mode, t.r, t.mult);
+    }
     piece -= pieces;
   }
 }
@@ -306,7 +307,7 @@ cudaError_t launch_copy(const void* in, void* out, int64_t count, int64_t in_str
 
 cudaError_t launch_twiddle_list(void* out, const TwiddleList& list, cudaStream_t st) {
   int64_t pieces = 0;
-  for (int i = 0; i < list.n; ++i) pieces += (list.t[i].count + 1023) >> 10;
+  for (int i = 0; i < list.n; ++i) pieces += (list.t[i].count + 255) >> 8;
   if (pieces == 0) return cudaSuccess;
   twiddle_gen_all<<<(int)std::min<int64_t>(pieces, 4096), 256, 0, st>>>(static_cast<float2*>(out), list);
   return cudaGetLastError();
