@@ -160,21 +160,28 @@ double time_candidate(const fft_plan_options_t& o, const int64_t* n, int dims, i
   make_plan(s, n, dims, batch, direction, FFT_PREC_FP32, &o, caps);
   if (s.status != FFT_OK) return kInf;
   DevBuf tables, work;
-  if (tables.alloc((size_t)s.table_elems * 8 + 16) != cudaSuccess) return kInf;
+  const size_t words = 16 + (s.joined ? 4 * (size_t)(2 + 2 * s.join_ring) : 0);
+  if (tables.alloc((size_t)s.table_elems * 8 + words) != cudaSuccess) return kInf;
   if (s.work_elems && work.alloc((size_t)s.work_elems * 8) != cudaSuccess) return kInf;
   int* status = reinterpret_cast<int*>(static_cast<char*>(tables.p) + (size_t)s.table_elems * 8);
-  cudaMemsetAsync(status, 0, 16, st);
+  cudaMemsetAsync(status, 0, words, st);
   PassLaunch launches[kMaxPasses];
+  JoinedLaunch joined;  // the form that a plan with these options runs
   if (enqueue_tables(s, static_cast<cf*>(tables.p), st) != cudaSuccess) return kInf;
   if (bind_launches(s, caps, static_cast<const cf*>(tables.p), status, launches) != cudaSuccess)
     return kInf;
+  if (s.joined && bind_joined(s, caps, static_cast<const cf*>(tables.p), status,
+                              reinterpret_cast<unsigned*>(status + 4), &joined) != cudaSuccess)
+    return kInf;
   for (int it = 0; it < 2; ++it)
-    if (enqueue_passes(s, launches, in, out, work.p, 0, batch, st) != cudaSuccess) return kInf;
+    if (enqueue_passes(s, launches, in, out, work.p, 0, batch, st, -1, &joined) != cudaSuccess)
+      return kInf;
   Ev ev;
   const int reps = 5;
   cudaEventRecord(ev.a, st);
   for (int it = 0; it < reps; ++it)
-    if (enqueue_passes(s, launches, in, out, work.p, 0, batch, st) != cudaSuccess) return kInf;
+    if (enqueue_passes(s, launches, in, out, work.p, 0, batch, st, -1, &joined) != cudaSuccess)
+      return kInf;
   cudaEventRecord(ev.b, st);
   if (cudaEventSynchronize(ev.b) != cudaSuccess) {
     cudaGetLastError();
