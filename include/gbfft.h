@@ -214,7 +214,9 @@ GBFFT_API fft_status_t fft_plan_destroy(fft_plan_t plan);
 /* Bytes of device workspace owned by the plan (0 for single-pass plans). */
 GBFFT_API fft_status_t fft_plan_workspace_bytes(fft_plan_t plan, size_t* bytes);
 
-/* Kernel launches one fft_execute enqueues (per sub-batch, see fft_plan_create). */
+/* Kernel launches one fft_execute enqueues (per sub-batch, see fft_plan_create; 1
+ * for a plan that describes itself as joined, which takes 2 where it runs a launch
+ * per pass: partly overlapping buffers, and 2D plans as fft_plan_describe says). */
 GBFFT_API fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches);
 
 /*
