@@ -197,6 +197,9 @@ cudaError_t launch_stage_bench(int R, const PassDesc& d, int Ns, int reps, int g
 // per thread; d0 is the pass descriptor of one job (tables, shape, strides).
 cudaError_t launch_grouped(int R, const PassDesc& d0, const GroupTable& gt, int grid, int block,
                            size_t smem, cudaStream_t st);
+// The same for a pass of the short-line kernels (l.lines; GroupEntry::tiles count
+// tiles of 2^l.lines elements).
+cudaError_t launch_grouped_lines(const PassLaunch& l, const GroupTable& gt, cudaStream_t st);
 cudaError_t launch_copy(const void* in, void* out, int64_t count, int64_t in_stride,
                         int64_t out_stride, cudaStream_t st);
 // Twiddle tables (planner.h: TwSegment) at out + off, all in one launch.

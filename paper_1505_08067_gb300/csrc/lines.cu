@@ -40,6 +40,31 @@ short_lines(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc
   else B::template store_rows<false>(v, out + at, valid, tid);
 }
 
+// The same for a coalesced launch (GroupTable): block t runs tile t of the jobs'
+// tiles one after another, with the arithmetic of short_lines, so that a server
+// job's bits do not depend on whether it was coalesced.
+template <int LOGL>
+__global__ void __launch_bounds__(128, 4)
+grouped_lines(const __grid_constant__ PassDesc d, const __grid_constant__ GroupTable gt) {
+  using SH = typename JoinLen<12, LOGL>::S;
+  using B = JoinBody<SH, JOIN_ROWS, JoinMem>;
+  extern __shared__ __align__(16) unsigned char smem_lines[];
+  cf* sm = reinterpret_cast<cf*>(smem_lines);
+  const int tid = threadIdx.x;
+  int j = 0;
+  while (j + 1 < gt.n && gt.e[j + 1].tile_begin <= blockIdx.x) ++j;
+  const int64_t tile = blockIdx.x - gt.e[j].tile_begin, at = tile << 12;
+  const int64_t valid = gt.e[j].count - tile * B::G;
+  const cf* in = gt.e[j].in + at;
+  cf* out = gt.e[j].out + at;
+  cf v[kJoinR];
+  if (d.conj_in) B::template first_rows<true>(v, in, valid, tid);
+  else B::template first_rows<false>(v, in, valid, tid);
+  join_stages<SH, JOIN_ROWS, false>(v, sm, d.tw + d.tw_line, 0, 0, tid);
+  if (d.conj_out) B::template store_rows<true>(v, out, valid, tid);
+  else B::template store_rows<false>(v, out, valid, tid);
+}
+
 template <int LOGL>
 static bool lines_fn(PassLaunch* l) {
   l->fn = (const void*)short_lines<LOGL>;
@@ -103,6 +128,32 @@ bool resolve_lines(int logL, PassLaunch* l) {
     case 10: return lines_fn<10>(l);
     default: return false;
   }
+}
+
+cudaError_t launch_grouped_lines(const PassLaunch& l, const GroupTable& gt, cudaStream_t st) {
+  if (!l.lines || gt.n < 1 || gt.n > kMaxGroup) return cudaErrorInvalidValue;
+  const int64_t tiles = gt.e[gt.n - 1].tile_begin + gt.e[gt.n - 1].tiles;
+  if (tiles < 1 || tiles > 0x7fffffff) return cudaErrorInvalidValue;
+  const void* f = nullptr;
+  switch (l.d.logL) {
+    case 3: f = (const void*)grouped_lines<3>; break;
+    case 4: f = (const void*)grouped_lines<4>; break;
+    case 5: f = (const void*)grouped_lines<5>; break;
+    case 6: f = (const void*)grouped_lines<6>; break;
+    case 7: f = (const void*)grouped_lines<7>; break;
+    case 8: f = (const void*)grouped_lines<8>; break;
+    case 9: f = (const void*)grouped_lines<9>; break;
+    case 10: f = (const void*)grouped_lines<10>; break;
+    default: return cudaErrorInvalidValue;
+  }
+  if (l.smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+    if (e != cudaSuccess) return e;
+  }
+  using GFn = void (*)(PassDesc, GroupTable);
+  reinterpret_cast<GFn>(const_cast<void*>(f))<<<(int)tiles, l.block, l.smem, st>>>(l.d, gt);
+  return cudaGetLastError();
 }
 
 }  // namespace gbfft

@@ -73,6 +73,7 @@ struct PlanEntry {
   void* tables = nullptr;   // twiddles + status word
   int* status = nullptr;
   PassLaunch launches[kMaxPasses];
+  JoinedLaunch apart;       // two-pass plans of fft_execute's one-exchange kernels
   bool groupable = false;   // contiguous single-pass FP32: coalesced launches
   int64_t elems = 0;        // complex elements per batch entry
   int64_t work_per_entry = 0;  // workspace elements per batch entry (two-pass plans)
@@ -165,6 +166,15 @@ PlanEntry* plan_for(fft_server_t s, const JobKey& k, fft_status_t* st) {
   if (e == cudaSuccess)
     e = bind_launches(pe->spec, s->caps, static_cast<const cf*>(pe->tables), pe->status,
                       pe->launches);
+  // the passes that fft_execute runs, for the same bits, in the form that needs
+  // no counters (groups of one plan overlap).  Measured against the staged
+  // passes, both above L2: 2^15 x 2^13 1348 -> 1201 us, 2^18 x 2^10 1731 -> 1394,
+  // 2^20 x 2^8 1448 -> 1449.
+  if (e == cudaSuccess && k.dims == 1 && pe->spec.joined) {
+    pe->spec.join_apart = true;
+    e = bind_joined(pe->spec, s->caps, static_cast<const cf*>(pe->tables), pe->status, nullptr,
+                    &pe->apart);
+  }
   if (e != cudaSuccess) {
     cudaFree(pe->tables);
     delete pe;
@@ -258,7 +268,8 @@ bool launch_group(fft_server_t s, Running& r) {
   if (pe->groupable && g.jobs.size() > 1) {
     // one coalesced launch per kMaxGroup jobs
     const PassSpec& p0 = pe->spec.passes[0];
-    PassDesc d0 = pe->launches[0].d;
+    const PassLaunch& l0 = pe->launches[0];
+    const int64_t lines = l0.lines ? (int64_t(1) << l0.lines) >> p0.logL : p0.G;  // per tile
     for (size_t b = 0; b < g.jobs.size() && e == cudaSuccess; b += kMaxGroup) {
       GroupTable gt{};
       int64_t tiles = 0;
@@ -268,12 +279,13 @@ bool launch_group(fft_server_t s, Running& r) {
         ge.in = static_cast<const cf*>(rec.job.in);
         ge.out = static_cast<cf*>(rec.job.out);
         ge.count = rec.job.batch;
-        ge.tiles = (rec.job.batch + p0.G - 1) / p0.G;
+        ge.tiles = (rec.job.batch + lines - 1) / lines;
         ge.tile_begin = tiles;
         tiles += ge.tiles;
       }
       const int grid = (int)std::min<int64_t>(tiles, (int64_t)s->caps.sm_count * 16);
-      e = launch_grouped(p0.R, d0, gt, grid, p0.block, p0.smem, st);
+      e = l0.lines ? launch_grouped_lines(l0, gt, st)
+                   : launch_grouped(p0.R, l0.d, gt, grid, p0.block, p0.smem, st);
       ++s->launches;
     }
     s->coalesced += g.jobs.size();
@@ -293,7 +305,8 @@ bool launch_group(fft_server_t s, Running& r) {
       }
       // a six-step plan's second buffer follows this job's first one
       e = enqueue_passes(pe->spec, pe->launches, rec.job.in, rec.job.out, ws, 0, rec.job.batch, st,
-                         pe->spec.work2_off > 0 ? ws_entries * pe->elems : -1);
+                         pe->spec.work2_off > 0 ? ws_entries * pe->elems : -1,
+                         pe->apart.fn ? &pe->apart : nullptr);
       if (ws) cudaFreeAsync(ws, st);  // after the passes, in stream order
       ++s->launches;
       if (e != cudaSuccess) break;

@@ -1,0 +1,69 @@
+"""One transform, one result: every entry point runs an FP32 shape with the same
+arithmetic, so a job's output has the bits of fft_execute with default options,
+whatever else is waiting."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _bits(t):
+    return t.view(torch.int64)
+
+
+def _case(gb, logn, batches, direction):
+    """Inputs, what fft_execute gives for them, and outputs inside guard elements."""
+    n = 2 ** logn
+    torch.manual_seed(logn)
+    xs = [torch.randn(b * n, dtype=torch.complex64, device="cuda") for b in batches]
+    want = []
+    for x, b in zip(xs, batches):
+        with gb.Plan(n, b, direction) as p:
+            want.append(p.execute(x))
+    outs = [torch.full((b * n + 1,), 7.0 + 7.0j, dtype=torch.complex64, device="cuda") for b in batches]
+    torch.cuda.synchronize()
+    return n, xs, want, outs
+
+
+def _check(xs, want, outs):
+    torch.cuda.synchronize()
+    for x, w, y in zip(xs, want, outs):
+        assert torch.equal(_bits(y[:-1]), _bits(w)) and y[-1].item() == 7.0 + 7.0j
+
+
+@pytest.mark.parametrize("logn", list(range(1, 21)) + [21])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_server(gb, logn, direction):
+    """A job alone, and jobs of several sizes in one held burst (lengths up to 2^14:
+    one coalesced launch, here in more than one table of jobs), with ragged tiles."""
+    t = max(1, 4096 >> logn)
+    batches = [1, t, t + 1, 3 * t - 1 or 1, 2] * (14 if logn <= 14 else 1)
+    n, xs, want, outs = _case(gb, logn, batches, direction)
+    srv = gb.fft_server_create(memory_budget_bytes=4 << 30)
+    try:
+        submit = lambda x, y, b: gb.fft_server_submit(srv, n, b, direction, 0, x.data_ptr(), y.data_ptr())
+        for x, y, b in list(zip(xs, outs, batches))[:5]:
+            assert gb.fft_server_wait(srv, submit(x, y, b), 60.0)["status"] == 0
+        assert gb.fft_server_stats(srv)["coalesced_jobs"] == 0
+        _check(xs[:5], want[:5], outs[:5])
+        gb.fft_server_pause(srv, True)
+        tickets = [submit(x, y, b) for x, y, b in zip(xs, outs, batches)]
+        gb.fft_server_pause(srv, False)
+        assert all(gb.fft_server_wait(srv, k, 60.0)["status"] == 0 for k in tickets)
+        assert gb.fft_server_stats(srv)["coalesced_jobs"] == (len(batches) if logn <= 14 else 0)
+    finally:
+        gb.fft_server_destroy(srv)
+    _check(xs, want, outs)
+
+
+@pytest.mark.parametrize("logn", [15, 17, 18, 20])
+def test_server_large(gb, logn):
+    """Jobs large enough for fft_execute to join the passes."""
+    n, xs, want, outs = _case(gb, logn, [(3 << 22 >> logn) + 1], -1)
+    srv = gb.fft_server_create(memory_budget_bytes=4 << 30)
+    try:
+        k = gb.fft_server_submit(srv, n, xs[0].numel() // n, -1, 0, xs[0].data_ptr(), outs[0].data_ptr())
+        assert gb.fft_server_wait(srv, k, 60.0)["status"] == 0
+    finally:
+        gb.fft_server_destroy(srv)
+    _check(xs, want, outs)
