@@ -50,6 +50,7 @@ struct DeviceState {
   int direction = 0;
   PlanSpec spec;
   PassLaunch launches[kMaxPasses];
+  JoinedLaunch apart;         // two-pass shapes of the one-exchange kernels, a launch each
   bool tables_valid = false;  // the array holds the tables of `spec` (segment list below)
   SmallVec<TwSegment, 40> table_layout;
 };
@@ -123,9 +124,9 @@ extern "C" fft_status_t fft_execute_noalloc(int64_t n, int64_t batch, int direct
       caps.smem_optin = v;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxThreadsPerBlock, dev) == cudaSuccess)
       caps.max_block = v;
-    fft_plan_options_t opt{};
-    opt.epilogue = 4;  // four-step twiddles computed in-kernel: no N-entry table in static memory
-    make_plan(ds.spec, &n, 1, batch, direction, FFT_PREC_FP32, &opt, caps);
+    // the plan and kernels of fft_execute, whose bits this call gives (its
+    // four-step twiddles are computed in-kernel: no N-entry table in static memory)
+    make_plan(ds.spec, &n, 1, batch, direction, FFT_PREC_FP32, nullptr, caps);
     if (ds.spec.status != FFT_OK) return set_error(ds.spec.status, ds.spec.error);
     if (ds.spec.work_elems > kWorkElems)
       return set_error(FFT_ERR_UNSUPPORTED_SIZE,
@@ -136,6 +137,11 @@ extern "C" fft_status_t fft_execute_noalloc(int64_t n, int64_t batch, int direct
       return set_error(FFT_ERR_UNSUPPORTED_SIZE,
                        "fft_execute_noalloc: twiddle tables exceed the static area");
     cudaError_t e = bind_launches(ds.spec, caps, tables, status, ds.launches);
+    ds.apart = JoinedLaunch();
+    if (e == cudaSuccess && ds.spec.joined) {  // never joined in one launch: no counters here
+      ds.spec.join_apart = true;
+      e = bind_joined(ds.spec, caps, tables, status, nullptr, &ds.apart);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return set_error(FFT_ERR_CUDA, cudaGetErrorString(e));
@@ -158,7 +164,9 @@ extern "C" fft_status_t fft_execute_noalloc(int64_t n, int64_t batch, int direct
       ds.tables_valid = true;
     }
   }
-  if (e == cudaSuccess) e = enqueue_passes(ds.spec, ds.launches, in, out, work, 0, batch, cs);
+  if (e == cudaSuccess)
+    e = enqueue_passes(ds.spec, ds.launches, in, out, work, 0, batch, cs, -1,
+                       ds.apart.fn ? &ds.apart : nullptr);
   if (e != cudaSuccess) {
     cudaGetLastError();
     ds.tables_valid = false;

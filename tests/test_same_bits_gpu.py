@@ -67,3 +67,19 @@ def test_server_large(gb, logn):
     finally:
         gb.fft_server_destroy(srv)
     _check(xs, want, outs)
+
+
+@pytest.mark.parametrize("logn", range(0, 24))
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_noalloc(gb, logn, direction):
+    """Every length, the largest batch of the two-pass ones included, in and out of place."""
+    t = max(1, 4096 >> logn)
+    batches = [1, 3 * t + 1] if logn <= 14 else sorted({1, min(3, 2 ** 23 >> logn), 2 ** 23 >> logn})
+    n, xs, want, outs = _case(gb, logn, batches, direction)
+    s = torch.cuda.current_stream().cuda_stream
+    for x, y, b in zip(xs, outs, batches):
+        gb.fft_execute_noalloc(n, b, direction, x.data_ptr(), y.data_ptr(), s)
+    _check(xs, want, outs)
+    gb.fft_execute_noalloc(n, batches[-1], direction, xs[-1].data_ptr(), xs[-1].data_ptr(), s)
+    torch.cuda.synchronize()
+    assert torch.equal(_bits(xs[-1]), _bits(want[-1]))
