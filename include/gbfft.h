@@ -26,6 +26,10 @@
  *     exp(+2 pi i nk/N) and is NOT normalised: inverse(forward(x)) = N x.
  *   - Pointers named `in`/`out` are device pointers owned by the caller,
  *     aligned to the element size (8 bytes; 4 for complex32).  `in` is never written.  in == out (in place) is allowed.
+ *   - One FP32 shape has one result: fft_execute of a plan with default options,
+ *     fft_execute_graph, fft_execute_host, fft_execute_noalloc, the server
+ *     (whatever else is waiting) and the work queue give the same bits for
+ *     16-byte-aligned buffers.
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream).
  *   - Errors are returned as fft_status_t and never abort; fft_last_error()
  *     gives a human-readable message for the calling thread.  No entry point

@@ -179,6 +179,20 @@ __device__ __forceinline__ void join_stages(cf (&v)[kJoinR], cf* sm, const cf* t
   B::template turn<SH::kLast, TW4>(v, tw, col0, logN, tid);
 }
 
+// A tile of 4096 elements of contiguous lines of 2^LOGL points, `valid` of them.
+template <int LOGL>
+__device__ __forceinline__ void line_tile(const cf* in, cf* out, const PassDesc& d, int64_t valid,
+                                          cf* sm, int tid) {
+  using SH = typename JoinLen<12, LOGL>::S;
+  using B = JoinBody<SH, JOIN_ROWS, JoinMem>;
+  cf v[kJoinR];
+  if (d.conj_in) B::template first_rows<true>(v, in, valid, tid);
+  else B::template first_rows<false>(v, in, valid, tid);
+  join_stages<SH, JOIN_ROWS, false>(v, sm, d.tw + d.tw_line, 0, 0, tid);
+  if (d.conj_out) B::template store_rows<true>(v, out, valid, tid);
+  else B::template store_rows<false>(v, out, valid, tid);
+}
+
 // Both rounds of a fast convolution: forward stages, filter, the stages in
 // reverse order on swapped data (the unnormalised inverse).
 template <class SH, int KIND>

@@ -25,19 +25,11 @@ namespace gbfft {
 template <int LOGL>
 __global__ void __launch_bounds__(128, 4)
 short_lines(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc d) {
-  using SH = typename JoinLen<12, LOGL>::S;
-  using B = JoinBody<SH, JOIN_ROWS, JoinMem>;
   extern __shared__ __align__(16) unsigned char smem_lines[];
-  cf* sm = reinterpret_cast<cf*>(smem_lines);
-  const int tid = threadIdx.x;
+  const int64_t tile = blockIdx.x, at = tile << 12;
   grid_wait();
-  const int64_t at = (int64_t)blockIdx.x << 12, valid = d.count_inner - (int64_t)blockIdx.x * B::G;
-  cf v[kJoinR];
-  if (d.conj_in) B::template first_rows<true>(v, in + at, valid, tid);
-  else B::template first_rows<false>(v, in + at, valid, tid);
-  join_stages<SH, JOIN_ROWS, false>(v, sm, d.tw + d.tw_line, 0, 0, tid);
-  if (d.conj_out) B::template store_rows<true>(v, out + at, valid, tid);
-  else B::template store_rows<false>(v, out + at, valid, tid);
+  line_tile<LOGL>(in + at, out + at, d, d.count_inner - tile * (4096 >> LOGL),
+                  reinterpret_cast<cf*>(smem_lines), threadIdx.x);
 }
 
 // The same for a coalesced launch (GroupTable): block t runs tile t of the jobs'
@@ -46,23 +38,12 @@ short_lines(const cf* __restrict__ in, cf* out, const __grid_constant__ PassDesc
 template <int LOGL>
 __global__ void __launch_bounds__(128, 4)
 grouped_lines(const __grid_constant__ PassDesc d, const __grid_constant__ GroupTable gt) {
-  using SH = typename JoinLen<12, LOGL>::S;
-  using B = JoinBody<SH, JOIN_ROWS, JoinMem>;
   extern __shared__ __align__(16) unsigned char smem_lines[];
-  cf* sm = reinterpret_cast<cf*>(smem_lines);
-  const int tid = threadIdx.x;
   int j = 0;
   while (j + 1 < gt.n && gt.e[j + 1].tile_begin <= blockIdx.x) ++j;
   const int64_t tile = blockIdx.x - gt.e[j].tile_begin, at = tile << 12;
-  const int64_t valid = gt.e[j].count - tile * B::G;
-  const cf* in = gt.e[j].in + at;
-  cf* out = gt.e[j].out + at;
-  cf v[kJoinR];
-  if (d.conj_in) B::template first_rows<true>(v, in, valid, tid);
-  else B::template first_rows<false>(v, in, valid, tid);
-  join_stages<SH, JOIN_ROWS, false>(v, sm, d.tw + d.tw_line, 0, 0, tid);
-  if (d.conj_out) B::template store_rows<true>(v, out, valid, tid);
-  else B::template store_rows<false>(v, out, valid, tid);
+  line_tile<LOGL>(gt.e[j].in + at, gt.e[j].out + at, d, gt.e[j].count - tile * (4096 >> LOGL),
+                  reinterpret_cast<cf*>(smem_lines), threadIdx.x);
 }
 
 template <int LOGL>

@@ -32,6 +32,7 @@
 #include "../../include/gbfft.h"
 #include "exec.h"
 #include "kernels.h"
+#include "joined.cuh"
 #include "kernels_impl.cuh"
 #include "planner.h"
 #include "queue_ring.h"
@@ -112,12 +113,33 @@ __device__ __forceinline__ void st_release_gpu(void* p, uint64_t v) {
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Blocks of at most 256 threads: the queue's single-pass plans (R = 16 up to
-// 4096 points with 256 threads per tile; shorter lengths 64 threads).  TR:
-// the compile-time shape of the length where one exists (kernel_shapes.h),
-// else every parameter from the descriptor.
+// The tiles of a job, so that it has the bits of fft_execute.  The register
+// kernel's: blocks of at most 256 threads (R = 16 up to 4096 points with 256
+// threads per tile; shorter lengths 64 threads); TR: the compile-time shape of the
+// length where one exists (kernel_shapes.h), else every parameter from the
+// descriptor.
 template <int R, class TR>
-__global__ void __launch_bounds__(256)
+struct RegisterTile {
+  static constexpr int kThreads = 256, kBlocks = 0;  // 0: no least number (58 registers; 1: 106)
+  static __device__ __forceinline__ void run(const cf* in, cf* out, const PassDesc& d,
+                                             int64_t tile, cf* sm, int tid) {
+    pass_tile<R, MAP_ROWS, MAP_ROWS, TR>(in, out, d, tile, sm, tid);
+  }
+};
+// 2^3 .. 2^10 points: the short-line kernels' (lines.cu).
+template <int LOGL>
+struct LineTile {
+  static constexpr int kThreads = 128, kBlocks = 4;
+  static __device__ __forceinline__ void run(const cf* in, cf* out, const PassDesc& d,
+                                             int64_t tile, cf* sm, int tid) {
+    __syncthreads();  // every thread has read the last tile's shared memory
+    line_tile<LOGL>(in + (tile << 12), out + (tile << 12), d,
+                    d.count_inner - tile * (4096 >> LOGL), sm, tid);
+  }
+};
+
+template <class Tile>
+__global__ void __launch_bounds__(Tile::kThreads, Tile::kBlocks)
 queue_worker(const __grid_constant__ PassDesc d0, const __grid_constant__ QueueArgs q) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cf* sm = reinterpret_cast<cf*>(smem_raw);
@@ -173,7 +195,7 @@ queue_worker(const __grid_constant__ PassDesc d0, const __grid_constant__ QueueA
     const cf* in = reinterpret_cast<const cf*>(s_in);
     cf* out = reinterpret_cast<cf*>(s_out);
     for (int64_t tile = blockIdx.x; tile < d.tiles; tile += gridDim.x)
-      pass_tile<R, MAP_ROWS, MAP_ROWS, TR>(in, out, d, tile, sm, tid);
+      Tile::run(in, out, d, tile, sm, tid);
     __syncthreads();  // this block's stores are issued; s_* is rewritten next
     if (tid == 0) {
       __threadfence();
@@ -189,14 +211,29 @@ queue_worker(const __grid_constant__ PassDesc d0, const __grid_constant__ QueueA
 const void* worker_fn(int R, const PassDesc& d) {
 #define GB_TRY(LOGL, SCHED, NST, RR, G, LM, SM, CONTIG, EPI)                                     \
   if (shape_matches(d, R, MAP_ROWS, MAP_ROWS, LOGL, SCHED, NST, RR, G, LM, SM, CONTIG, EPI))     \
-    return (const void*)queue_worker<RR, CtTraits<LOGL, SCHED, NST, RR, G, CONTIG, EPI>>;
+    return (const void*)queue_worker<RegisterTile<RR, CtTraits<LOGL, SCHED, NST, RR, G, CONTIG, EPI>>>;
   GB_SHAPES_CONTIG(GB_TRY)
 #undef GB_TRY
   switch (R) {
-    case 2: return (const void*)queue_worker<2, RtTraits>;
-    case 4: return (const void*)queue_worker<4, RtTraits>;
-    case 8: return (const void*)queue_worker<8, RtTraits>;
-    case 16: return (const void*)queue_worker<16, RtTraits>;
+    case 2: return (const void*)queue_worker<RegisterTile<2, RtTraits>>;
+    case 4: return (const void*)queue_worker<RegisterTile<4, RtTraits>>;
+    case 8: return (const void*)queue_worker<RegisterTile<8, RtTraits>>;
+    case 16: return (const void*)queue_worker<RegisterTile<16, RtTraits>>;
+    default: return nullptr;
+  }
+}
+
+// The worker of a pass that fft_execute runs with the short-line kernels.
+const void* line_worker_fn(int logL) {
+  switch (logL) {
+    case 3: return (const void*)queue_worker<LineTile<3>>;
+    case 4: return (const void*)queue_worker<LineTile<4>>;
+    case 5: return (const void*)queue_worker<LineTile<5>>;
+    case 6: return (const void*)queue_worker<LineTile<6>>;
+    case 7: return (const void*)queue_worker<LineTile<7>>;
+    case 8: return (const void*)queue_worker<LineTile<8>>;
+    case 9: return (const void*)queue_worker<LineTile<9>>;
+    case 10: return (const void*)queue_worker<LineTile<10>>;
     default: return nullptr;
   }
 }
@@ -332,9 +369,7 @@ fft_status_t fft_queue_create(fft_queue_t* queue, int64_t n, int64_t max_batch, 
   q->device = dev;
   q->slots = slots;
   q->max_batch = max_batch;
-  fft_plan_options_t opt{};
-  opt.variant = 1;  // the register kernel's tiles (one tile per block at a time)
-  make_plan(q->spec, &n, 1, max_batch, direction, FFT_PREC_FP32, &opt, caps);
+  make_plan(q->spec, &n, 1, max_batch, direction, FFT_PREC_FP32, nullptr, caps);
   if (q->spec.status != FFT_OK) {
     fft_status_t st = q->spec.status;
     char msg[256];
@@ -345,13 +380,16 @@ fft_status_t fft_queue_create(fft_queue_t* queue, int64_t n, int64_t max_batch, 
   const PassSpec& p = q->spec.passes[0];
   const bool one_pass = q->spec.passes.size() == 1 && p.kind == PASS_FFT && p.batch_is_tiles;
   if (one_pass) q->d0 = pass_desc(p, 0, max_batch, max_batch);
-  q->fn = one_pass ? worker_fn(p.R, q->d0) : nullptr;
+  PassLaunch lines{};
+  const bool by_lines = one_pass && p.line_off >= 0 && resolve_lines(p.logL, &lines);
+  if (by_lines) q->d0.G = (1 << lines.lines) >> p.logL;
+  q->fn = by_lines ? line_worker_fn(p.logL) : one_pass ? worker_fn(p.R, q->d0) : nullptr;
   if (!q->fn) {
     delete q;
     return set_error(FFT_ERR_NOT_IMPLEMENTED, "no single-pass register plan for this length");
   }
-  q->block = p.block;
-  q->smem = p.smem;
+  q->block = by_lines ? lines.block : p.block;
+  q->smem = by_lines ? lines.smem : p.smem;
   if ((e = cudaStreamCreateWithFlags(&q->stream, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaMalloc(&q->tables, (size_t)q->spec.table_elems * 8 + 16)) != cudaSuccess ||
       (e = cudaMalloc(&q->dev, (size_t)slots * (sizeof(QGo) + sizeof(int)))) != cudaSuccess ||
@@ -388,7 +426,7 @@ fft_status_t fft_queue_create(fft_queue_t* queue, int64_t n, int64_t max_batch, 
   q->d0.tw = static_cast<const cf*>(q->tables);
   q->d0.status = status;
   const int64_t resident = (int64_t)per_sm * caps.sm_count;
-  const int64_t tiles = (max_batch + p.G - 1) / p.G;
+  const int64_t tiles = (max_batch + q->d0.G - 1) / q->d0.G;
   q->grid = (int)std::min<int64_t>(blocks > 0 ? blocks : tiles, resident);
   q->args.ring = reinterpret_cast<QSlot*>(static_cast<char*>(dhost) + sizeof(QHeader));
   q->args.header = static_cast<const QHeader*>(dhost);

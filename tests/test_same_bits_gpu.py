@@ -83,3 +83,24 @@ def test_noalloc(gb, logn, direction):
     gb.fft_execute_noalloc(n, batches[-1], direction, xs[-1].data_ptr(), xs[-1].data_ptr(), s)
     torch.cuda.synchronize()
     assert torch.equal(_bits(xs[-1]), _bits(want[-1]))
+
+
+@pytest.mark.parametrize("logn", range(1, 13))
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_queue(gb, logn, direction):
+    """Jobs below, at and above a tile, more tiles than worker blocks, in place."""
+    t = max(1, 4096 >> logn)
+    batches = [1, t, t + 1, 9 * t - 1]
+    n, xs, want, outs = _case(gb, logn, batches, direction)
+    for blocks in (0, 2):
+        for y in outs:
+            y[:-1].zero_()
+        torch.cuda.synchronize()
+        with gb.Queue(n, max(batches), direction, blocks=blocks) as q:
+            for k in [q.submit_ptr(x.data_ptr(), y.data_ptr(), b) for x, y, b in zip(xs, outs, batches)]:
+                q.wait(k, 10.0)
+        _check(xs, want, outs)
+    with gb.Queue(n, max(batches), direction) as q:
+        q.wait(q.submit_ptr(xs[-1].data_ptr(), xs[-1].data_ptr(), batches[-1]), 10.0)
+    torch.cuda.synchronize()
+    assert torch.equal(_bits(xs[-1]), _bits(want[-1]))
