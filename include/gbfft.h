@@ -29,7 +29,7 @@
  *   - One FP32 shape has one result: fft_execute of a plan with default options,
  *     fft_execute_graph, fft_execute_host, fft_execute_noalloc, the server
  *     (whatever else is waiting) and the work queue give the same bits for
- *     16-byte-aligned buffers.
+ *     16-byte-aligned buffers that are the same or do not overlap.
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream).
  *   - Errors are returned as fft_status_t and never abort; fft_last_error()
  *     gives a human-readable message for the calling thread.  No entry point
@@ -506,7 +506,7 @@ GBFFT_API const char* fft_last_error(void);
 
 /* Diagnostic of the device-side bounded waits.  Every wait in the library's
  * kernels (the staged kernels' and the tensor-core kernel's waits on an
- * mbarrier, the work queue's polls) gives up after a fixed number of polls,
+ * mbarrier, the joined launches' waits for tiles, the work queue's polls) gives up after a fixed number of polls,
  * sets a status word and returns instead of hanging.  This call runs that
  * wait where it must run out: one block whose threads wait on an mbarrier
  * that nothing completes, with the library's wait loop limited to `polls`
@@ -515,6 +515,17 @@ GBFFT_API const char* fft_last_error(void);
  * synchronises the current device and leaves it usable.  FFT_ERR_INVALID_ARG
  * for polls outside that range or a null gave_up; FFT_ERR_CUDA if no device. */
 GBFFT_API fft_status_t fft_wait_selftest(uint32_t polls, int* gave_up);
+
+/* Diagnostic of a joined launch's waits: one execution of `plan` (of its first
+ * sub-batch) on `stream` that finds `handed_out` tiles marked as handed out
+ * already, which no block computes, and whose waits give up after `polls` polls
+ * (1 .. 2^21; 2^21 is the limit the kernels use, about a second).  Tiles that
+ * depend on the missing ones give up: the launch ends, `out` is incomplete,
+ * fft_plan_sync_status returns FFT_ERR_TIMEOUT once, and the plan's next
+ * execution is right again.  FFT_ERR_INVALID_ARG where the plan does not describe
+ * itself as joined or would not be joined on `stream`. */
+GBFFT_API fft_status_t fft_join_selftest(fft_plan_t plan, const void* in, void* out,
+                                         uint32_t handed_out, uint32_t polls, void* stream);
 
 /* ------------------------------------------------ schedule model (host) --
  * Sec. 3.2 "FFT performance model": a radix schedule for N = 2^L is a path in

@@ -515,9 +515,32 @@ fft_status_t fft_plan_sync_status(fft_plan_t plan, void* stream) {
   if (e != cudaSuccess) return cuda_fail(e, "status word");
   if (flag) {
     cudaMemset(plan->status, 0, sizeof flag);
-    return fail(FFT_ERR_TIMEOUT, "a kernel gave up waiting for its TMA copy (bounded wait)");
+    return fail(FFT_ERR_TIMEOUT, "a kernel gave up a bounded wait (its copy into shared memory, or "
+                                 "the tiles of a joined launch); the output is incomplete");
   }
   return FFT_OK;
+}
+
+fft_status_t fft_join_selftest(fft_plan_t plan, const void* in, void* out, uint32_t handed_out,
+                               uint32_t polls, void* stream) {
+  if (!plan_ok(plan)) return fail(FFT_ERR_BAD_PLAN, "null or destroyed plan");
+  if (!in || !out || ((uintptr_t)in & 7) || ((uintptr_t)out & 7) || polls < 1 || polls > kJoinPolls)
+    return fail(FFT_ERR_INVALID_ARG, "fft_join_selftest: aligned buffers and polls 1 .. 2^21");
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if (dev != plan->device) return fail(FFT_ERR_BAD_PLAN, "plan/device mismatch");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const JoinedLaunch* own = joined_for(plan, st);
+  if (!own || !own->fn || own->second)
+    return fail(FFT_ERR_INVALID_ARG, "fft_join_selftest: the plan is not joined on this stream");
+  JoinedLaunch j = *own;
+  j.d.polls = polls;
+  const PlanSpec& s = plan->spec;
+  const int64_t nb = s.chunk_batch > 0 ? std::min(s.batch, s.chunk_batch) : s.batch;
+  e = cudaMemcpyAsync(j.d.ctr, &handed_out, sizeof handed_out, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = launch_joined(j, nb, in, out, plan->work, st);
+  return e == cudaSuccess ? FFT_OK : cuda_fail(e, "joined launch");
 }
 
 const char* fft_last_error(void) { return g_err; }

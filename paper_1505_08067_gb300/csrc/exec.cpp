@@ -165,6 +165,7 @@ cudaError_t bind_joined(const PlanSpec& s, const Caps& caps, const cf* tables, i
   j->d.o.ring = s.join_ring;
   j->d.ctr = counters;
   j->d.status = status;
+  j->d.polls = kJoinPolls;
   return cudaSuccess;
 }
 

@@ -65,8 +65,6 @@ __device__ __forceinline__ void red_release_gpu(unsigned* p) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
 
-constexpr uint32_t kJoinPolls = 1u << 21;  // about a second before a wait gives up
-
 // Finished-tile counters (JoinDesc::ctr): [0] tickets handed out, [1] blocks
 // that have left, then per pass and ring slot the tiles finished.  All zero
 // between launches: the last block to leave clears them.
@@ -112,7 +110,7 @@ __device__ __forceinline__ void join_dispatch(const JoinDesc& d, uint64_t* store
         const JoinDep dep = join_dep(d.o, k);
         const unsigned* c = join_done(d, dep.pass, dep.slot);
         bool ok = dep.count == 0;
-        for (uint32_t it = 0; it < kJoinPolls && !ok; ++it) {
+        for (uint32_t it = 0; it < d.polls && !ok; ++it) {
           ok = ld_acquire_gpu(c) >= dep.count;
           if (!ok && finished && mbar_test(stored, (n - 1) & 1)) {
             red_release_gpu(finished);
@@ -121,7 +119,7 @@ __device__ __forceinline__ void join_dispatch(const JoinDesc& d, uint64_t* store
           if (!ok && it > 16) __nanosleep(64);
         }
         if (!ok) {
-          atomicExch(d.status, 1);
+          atomicOr(d.status, kStatusGaveUp);
           t = total;
         }
       }

@@ -10,12 +10,15 @@ namespace gbfft {
 
 // The joined kernels (joined.cuh): both passes of a four-step transform, or of
 // 2D frames, in one launch.
+constexpr uint32_t kJoinPolls = 1u << 21;  // about a second before a wait gives up
+constexpr int kStatusGaveUp = 1;           // status word: a bounded wait gave up
 struct JoinDesc {
   const cf* tw1;  // w_L^j of the first pass's length, and of the second's
   const cf* tw2;
   JoinOrder o;
   unsigned* ctr;  // 2 + 2 ring counters, zero between launches
   int* status;
+  uint32_t polls;  // kJoinPolls, or fewer in a test of the waits
   // frames: log2 rows and columns, elements of the whole batch
   int lr, lc;
   int64_t total;

@@ -100,6 +100,7 @@ _SIGS = {
     "fft_execute_noalloc": [_i64, _i64, ctypes.c_int, _vp, _vp, _vp],
     "fft_fill_uniform": [_vp, _i64, ctypes.c_uint64, ctypes.c_uint64, _vp],
     "fft_wait_selftest": [ctypes.c_uint32, ctypes.POINTER(ctypes.c_int)],
+    "fft_join_selftest": [_vp, _vp, _vp, ctypes.c_uint32, ctypes.c_uint32, _vp],
     "fft_plan_destroy": [_vp],
     "fft_plan_workspace_bytes": [_vp, ctypes.POINTER(ctypes.c_size_t)],
     "fft_plan_launch_count": [_vp, ctypes.POINTER(ctypes.c_int)],
@@ -289,6 +290,13 @@ def fft_wait_selftest(polls: int) -> int:
     g = ctypes.c_int(0)
     _check(load().fft_wait_selftest(ctypes.c_uint32(int(polls) & 0xFFFFFFFF), ctypes.byref(g)))
     return g.value
+
+
+def fft_join_selftest(plan: int, in_ptr: int, out_ptr: int, handed_out: int, polls: int,
+                      stream: int = 0) -> None:
+    """One joined launch that finds `handed_out` tiles handed out already and whose
+    waits are limited to `polls` polls (see include/gbfft.h)."""
+    _check(load().fft_join_selftest(plan, in_ptr, out_ptr, int(handed_out), int(polls), stream))
 
 
 def fft_plan_destroy(plan: int) -> None:

@@ -31,3 +31,41 @@ def test_wait_gives_up_and_device_stays_usable(gb, oracle):
             gb.fft_plan_sync_status(p.handle, torch.cuda.current_stream().cuda_stream)
         err = oracle.rel_l2(y.cpu().numpy(), oracle.fft(x_np))
         assert np.max(err) <= 1e-6 * np.log2(n), float(np.max(err))
+
+
+JOINED = [((2 ** 15,), 391), ((2 ** 17,), 131), ((2 ** 20,), 13), ((16, 16), 49153), ((1024, 512), 25)]
+
+
+def _joined(gb, shape, batch):
+    torch.manual_seed(batch)
+    x = torch.randn((batch,) + shape, dtype=torch.complex64, device="cuda")
+    p = gb.Plan(shape if len(shape) > 1 else shape[0], batch)
+    assert p.describe()["joined"] == 1
+    return p, x, p.execute(x)
+
+
+@pytest.mark.parametrize("shape,batch", JOINED)
+@pytest.mark.parametrize("lost", [1, 7])
+def test_joined_wait_gives_up(gb, shape, batch, lost):
+    """The first `lost` tiles are never computed: what depends on them gives up, in
+    whichever block it falls to, the launch ends, the host reads it from the
+    status word, and the next execution starts from clean counters."""
+    s = torch.cuda.current_stream().cuda_stream
+    p, x, want = _joined(gb, shape, batch)
+    with p:
+        y = torch.empty_like(x)
+        for polls in (1, 64, 4096):
+            t0 = time.perf_counter()
+            gb.fft_join_selftest(p.handle, x.data_ptr(), y.data_ptr(), lost, polls, s)
+            with pytest.raises(gb.GbfftError) as e:
+                gb.fft_plan_sync_status(p.handle, s)
+            assert e.value.status == gb.FFT_ERR_TIMEOUT and time.perf_counter() - t0 < 5.0
+            y.fill_(float("nan"))
+            p.execute(x, y)
+            gb.fft_plan_sync_status(p.handle, s)
+            assert torch.equal(y, want)
+        for polls in (0, 2 ** 21 + 1):
+            with pytest.raises(gb.GbfftError):
+                gb.fft_join_selftest(p.handle, x.data_ptr(), y.data_ptr(), lost, polls, s)
+    with gb.Plan(1024, 4) as q, pytest.raises(gb.GbfftError):
+        gb.fft_join_selftest(q.handle, x.data_ptr(), y.data_ptr(), lost, 64, s)
