@@ -184,7 +184,9 @@ GBFFT_API fft_status_t fft_plan_create_ex(fft_plan_t* plan, const int64_t* n, in
  * the conventions above).  Asynchronous: returns after enqueueing; no host
  * synchronisation and no allocation.  A plan may be used from several host
  * threads only on distinct streams and only if no two executions overlap on
- * the device when the plan has a workspace (multi-pass 1D).
+ * the device when the plan has a workspace (multi-pass 1D).  Executions that
+ * overlap all the same spoil each other's outputs; where the plan describes itself
+ * as joined, also later ones until fft_plan_sync_status has reported it.
  * Sec. 3.4 (each pass reads and writes global memory once).
  */
 GBFFT_API fft_status_t fft_execute(fft_plan_t plan, const void* in, void* out, void* stream);
@@ -251,7 +253,11 @@ GBFFT_API fft_status_t fft_plan_dry_run(const int64_t* n, int dims, int64_t batc
                               int smem_optin_bytes, char* buf, size_t len);
 
 /* Wait for the stream-ordered work of the plan's last execute and report any
- * asynchronous CUDA error it raised. */
+ * asynchronous CUDA error it raised; FFT_ERR_TIMEOUT if a kernel of the plan gave
+ * up a bounded wait since the last call, FFT_ERR_CUDA if a joined launch found its
+ * tile counters used by another one (executions of a plan with a workspace that
+ * overlapped).  Either is reported once and the plan, with none of its executions
+ * at work, is as new. */
 GBFFT_API fft_status_t fft_plan_sync_status(fft_plan_t plan, void* stream);
 
 /* -------------------------------------------------- fast convolution --
@@ -522,7 +528,9 @@ GBFFT_API fft_status_t fft_wait_selftest(uint32_t polls, int* gave_up);
  * (1 .. 2^21; 2^21 is the limit the kernels use, about a second).  Tiles that
  * depend on the missing ones give up: the launch ends, `out` is incomplete,
  * fft_plan_sync_status returns FFT_ERR_TIMEOUT once, and the plan's next
- * execution is right again.  FFT_ERR_INVALID_ARG where the plan does not describe
+ * execution is right again.  With more than the launch has, no tile is
+ * computed and none is waited for, as after executions that overlapped:
+ * FFT_ERR_CUDA.  FFT_ERR_INVALID_ARG where the plan does not describe
  * itself as joined or would not be joined on `stream`. */
 GBFFT_API fft_status_t fft_join_selftest(fft_plan_t plan, const void* in, void* out,
                                          uint32_t handed_out, uint32_t polls, void* stream);

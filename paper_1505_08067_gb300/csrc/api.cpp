@@ -94,6 +94,11 @@ const JoinedLaunch* joined_for(fft_plan_t p, cudaStream_t st) {
   return owner == id + 1 ? &p->joined : nullptr;
 }
 
+// After the tables: the status word, then the joined launch's counters.
+size_t status_bytes(const PlanSpec& s) {
+  return 16 + (s.joined ? 4 * (size_t)(2 + 2 * s.join_ring) : 0);
+}
+
 fft_status_t query_caps(Caps& caps, int& device) {
   cudaError_t e = cudaGetDevice(&device);
   if (e != cudaSuccess) return cuda_fail(e, "no usable CUDA device");
@@ -139,8 +144,7 @@ fft_status_t build_plan(fft_plan_t* out, const int64_t* n, int dims, int64_t bat
   p->caps = caps;
   p->spec = spec;
   cudaError_t e;
-  // after the tables: the status word, then the joined launch's counters
-  const size_t words = 16 + (spec.joined ? 4 * (size_t)(2 + 2 * spec.join_ring) : 0);
+  const size_t words = status_bytes(spec);
   e = cudaMalloc(&p->tables, (size_t)spec.table_elems * 8 + words);
   if (e != cudaSuccess) {
     delete p;
@@ -514,9 +518,14 @@ fft_status_t fft_plan_sync_status(fft_plan_t plan, void* stream) {
   e = cudaMemcpy(&flag, plan->status, sizeof flag, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "status word");
   if (flag) {
-    cudaMemset(plan->status, 0, sizeof flag);
-    return fail(FFT_ERR_TIMEOUT, "a kernel gave up a bounded wait (its copy into shared memory, or "
-                                 "the tiles of a joined launch); the output is incomplete");
+    // a four-step plan's counters too (a frame plan's may be at work on a stream)
+    const bool ctr = plan->spec.joined && !plan->joined.frames;
+    cudaMemset(plan->status, 0, ctr ? status_bytes(plan->spec) : sizeof flag);
+    if (flag & kStatusGaveUp)
+      return fail(FFT_ERR_TIMEOUT, "a kernel gave up a bounded wait (its copy into shared memory, "
+                                   "or the tiles of a joined launch); the output is incomplete");
+    return fail(FFT_ERR_CUDA, "the tile counters of a joined launch were not its own: executions "
+                              "of the plan overlapped; outputs are incomplete");
   }
   return FFT_OK;
 }

@@ -67,7 +67,13 @@ __device__ __forceinline__ void red_release_gpu(unsigned* p) {
 
 // Finished-tile counters (JoinDesc::ctr): [0] tickets handed out, [1] blocks
 // that have left, then per pass and ring slot the tiles finished.  All zero
-// between launches: the last block to leave clears them.
+// between launches: the last block to leave clears them.  A whole launch hands out
+// one ticket per tile and one more per block, and as many blocks leave as it has.
+// A block that gets a later ticket, or leaves after them, reports kStatusCounters:
+// another execution of the plan drew on the counters meanwhile, which the plan's
+// contract forbids and which would otherwise pass unseen, here and in the launches
+// that find the counters it left.  (Comparing every counter before clearing it
+// costs 1 to 4.7 us a launch; this costs nothing.)
 __device__ __forceinline__ unsigned* join_done(const JoinDesc& d, int pass, int slot) {
   return d.ctr + 2 + pass * d.o.ring + slot;
 }
@@ -100,10 +106,12 @@ __device__ __forceinline__ void join_dispatch(const JoinDesc& d, uint64_t* store
                                               Prepare prepare) {
   const unsigned total = (unsigned)join_tickets(d.o);
   unsigned* finished = nullptr;
+  bool foreign = false;
   for (int n = 0;; ++n) {
     unsigned t = 0;
     if (lane == 0) {
       t = atomicAdd(d.ctr, 1u);
+      foreign = t >= total && t - total >= gridDim.x;
       if (t < total) {
         const JoinTicket k = join_ticket(d.o, t);
         if (k.pass == 0) prefetch(k);
@@ -136,7 +144,9 @@ __device__ __forceinline__ void join_dispatch(const JoinDesc& d, uint64_t* store
   unsigned last = 0;
   if (lane == 0) {
     __threadfence();
-    last = atomicAdd(d.ctr + 1, 1u) == gridDim.x - 1;
+    const unsigned left = atomicAdd(d.ctr + 1, 1u);
+    last = left == gridDim.x - 1;
+    if (foreign || left >= gridDim.x) atomicOr(d.status, kStatusCounters);
   }
   if (__shfl_sync(~0u, last, 0))
     for (int i = lane; i < 2 + 2 * d.o.ring; i += 32) d.ctr[i] = 0;

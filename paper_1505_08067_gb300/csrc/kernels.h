@@ -12,6 +12,7 @@ namespace gbfft {
 // 2D frames, in one launch.
 constexpr uint32_t kJoinPolls = 1u << 21;  // about a second before a wait gives up
 constexpr int kStatusGaveUp = 1;           // status word: a bounded wait gave up
+constexpr int kStatusCounters = 2;         // and: a joined launch's counters were not its own
 struct JoinDesc {
   const cf* tw1;  // w_L^j of the first pass's length, and of the second's
   const cf* tw2;

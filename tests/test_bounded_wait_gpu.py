@@ -69,3 +69,22 @@ def test_joined_wait_gives_up(gb, shape, batch, lost):
                 gb.fft_join_selftest(p.handle, x.data_ptr(), y.data_ptr(), lost, polls, s)
     with gb.Plan(1024, 4) as q, pytest.raises(gb.GbfftError):
         gb.fft_join_selftest(q.handle, x.data_ptr(), y.data_ptr(), lost, 64, s)
+
+
+@pytest.mark.parametrize("shape,batch", JOINED)
+def test_joined_counters_not_its_own(gb, shape, batch):
+    """A launch that finds every tile handed out computes nothing and waits for
+    nothing: it is reported, once, and the plan is as new."""
+    s = torch.cuda.current_stream().cuda_stream
+    p, x, want = _joined(gb, shape, batch)
+    with p:
+        y = torch.empty_like(x)
+        for handed_out in (2 * x.numel(), 2 ** 31):
+            gb.fft_join_selftest(p.handle, x.data_ptr(), y.data_ptr(), handed_out, 64, s)
+            with pytest.raises(gb.GbfftError) as e:
+                gb.fft_plan_sync_status(p.handle, s)
+            assert e.value.status == gb.FFT_ERR_CUDA
+            y.fill_(float("nan"))
+            p.execute(x, y)
+            gb.fft_plan_sync_status(p.handle, s)
+            assert torch.equal(y, want)
