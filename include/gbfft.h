@@ -234,8 +234,9 @@ GBFFT_API fft_status_t fft_plan_launch_count(fft_plan_t plan, int* launches);
  * flag, and "lines": 1 when the one-exchange kernel (default options: contiguous
  * transforms of 2^3 .. 2^10 points, frame columns and fast convolution of 2^3 ..
  * 2^11) runs the pass instead; "joined": 1 when both passes of a two-pass or 2D
- * plan run as one launch of a joined kernel (2D: on the first stream that executes
- * the plan; on others, and in graphs, each pass is a launch), "apart": 1 when they
+ * plan run as one launch of a joined kernel (2D: on the first four streams that execute
+ * the plan, fft_execute_host's own counting as one; on others, and in graphs, each
+ * pass is a launch), "apart": 1 when they
  * are that kernel's passes in a launch each, 0 when each runs the kernel named for
  * it) written to buf (NUL-terminated, truncated to len).  Returns
  * FFT_ERR_INVALID_ARG if buf is too small for the whole text.

@@ -6,7 +6,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -14,6 +13,7 @@
 #include "../../include/gbfft.h"
 #include "autotune.h"
 #include "exec.h"
+#include "join_owner.h"
 #include "kernels.h"
 #include "planner.h"
 #include "trace.h"
@@ -52,8 +52,9 @@ struct fft_plan_s {
   int* status = nullptr;   // set by kernels whose bounded waits give up
   void* work = nullptr;    // cf[spec.work_elems]
   PassLaunch launches[kMaxPasses];  // whole-batch launches, device pointers filled
-  JoinedLaunch joined;              // both passes of a two-pass plan as one launch
-  std::atomic<uint64_t> join_stream{0};  // id + 1 of the stream of a joined frame plan
+  JoinedLaunch joined[kJoinSets];   // both passes of a two-pass or frame plan as one launch,
+                                    // with each set of counters (four-step plans: one)
+  JoinOwners join_owners;           // frame plans: the sets' streams
   // lazily created resources of fft_execute_host
   cudaStream_t s_h2d = nullptr, s_k = nullptr, s_d2h = nullptr;
   cudaEvent_t ev_start = nullptr, ev_h2d = nullptr, ev_k = nullptr, ev_end = nullptr;
@@ -76,28 +77,26 @@ namespace {
 
 bool plan_ok(fft_plan_t p) { return p && p->magic == kMagic; }
 
-// The joined launch of an execution on st, or null for a launch per pass.  Its
-// tile counters are the plan's, so two of them must not overlap.  Four-step plans
-// have a workspace and may not overlap anyway; executions of frames may, on
-// several streams or as replays of several graphs.  So a frame plan is joined on
-// the first stream that runs it (ids, unlike handles, are not used again), and
-// nowhere else, nor in a capture, whose graph may be launched on any stream.
+// The joined launch of an execution on st, or null for a launch per pass.  Two
+// launches with one set of tile counters must not overlap.  Four-step plans have a
+// workspace and may not overlap anyway; executions of frames may, so they are
+// joined on streams that have a set (JoinOwners) and nowhere else, nor in a
+// capture, whose graph may be launched on any stream.
 const JoinedLaunch* joined_for(fft_plan_t p, cudaStream_t st) {
-  if (!p->joined.frames) return &p->joined;
+  if (!p->joined[0].frames) return &p->joined[0];
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   unsigned long long id = 0;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
       cudaStreamGetId(st, &id) != cudaSuccess)
     return nullptr;
-  uint64_t owner = 0;
-  if (p->join_stream.compare_exchange_strong(owner, id + 1)) owner = id + 1;
-  return owner == id + 1 ? &p->joined : nullptr;
+  const int set = p->join_owners.claim(id);
+  return set < 0 ? nullptr : &p->joined[set];
 }
 
-// After the tables: the status word, then the joined launch's counters.
-size_t status_bytes(const PlanSpec& s) {
-  return 16 + (s.joined ? 4 * (size_t)(2 + 2 * s.join_ring) : 0);
-}
+// After the tables: the status word, then the joined launch's sets of counters.
+int join_sets(const PlanSpec& s) { return !s.joined ? 0 : s.dims == 2 ? kJoinSets : 1; }
+size_t join_words(const PlanSpec& s) { return 2 + 2 * (size_t)s.join_ring; }
+size_t status_bytes(const PlanSpec& s) { return 16 + 4 * join_sets(s) * join_words(s); }
 
 fft_status_t query_caps(Caps& caps, int& device) {
   cudaError_t e = cudaGetDevice(&device);
@@ -173,9 +172,14 @@ fft_status_t build_plan(fft_plan_t* out, const int64_t* n, int dims, int64_t bat
   e = enqueue_tables(spec, static_cast<cf*>(p->tables), 0);
   if (e == cudaSuccess)
     e = bind_launches(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status, p->launches);
+  unsigned* counters = reinterpret_cast<unsigned*>(p->status + 4);
   if (e == cudaSuccess && spec.joined)
-    e = bind_joined(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status,
-                    reinterpret_cast<unsigned*>(p->status + 4), &p->joined);
+    e = bind_joined(p->spec, p->caps, static_cast<const cf*>(p->tables), p->status, counters,
+                    &p->joined[0]);
+  for (int i = 1; i < join_sets(spec); ++i) {
+    p->joined[i] = p->joined[0];
+    p->joined[i].d.ctr = counters + i * join_words(spec);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   if (e != cudaSuccess) {
     fft_plan_destroy(p);
@@ -519,7 +523,7 @@ fft_status_t fft_plan_sync_status(fft_plan_t plan, void* stream) {
   if (e != cudaSuccess) return cuda_fail(e, "status word");
   if (flag) {
     // a four-step plan's counters too (a frame plan's may be at work on a stream)
-    const bool ctr = plan->spec.joined && !plan->joined.frames;
+    const bool ctr = plan->spec.joined && !plan->joined[0].frames;
     cudaMemset(plan->status, 0, ctr ? status_bytes(plan->spec) : sizeof flag);
     if (flag & kStatusGaveUp)
       return fail(FFT_ERR_TIMEOUT, "a kernel gave up a bounded wait (its copy into shared memory, "
