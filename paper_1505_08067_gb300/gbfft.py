@@ -465,12 +465,19 @@ class Plan:
 
     def _prepare(self):
         """What every execute needs and no execute changes: its C entry point
-        and the type and size its tensors must have."""
-        import torch
+        and the size its tensors must have (their type: _dtype)."""
         self._execute = load().fft_execute
+        self._elements = self.elements
+
+    def __getattr__(self, name):
+        # the type of the tensors, looked up by the first call that takes any:
+        # planning and execution from pointers need no torch
+        if name != "_dtype":
+            raise AttributeError(f"{type(self).__name__!r} object has no attribute {name!r}")
+        import torch
         self._dtype = (torch.complex32 if self.precision == FFT_PREC_TC_FP16_C32
                        else torch.complex64)
-        self._elements = self.elements
+        return self._dtype
 
     @property
     def elements(self) -> int:
