@@ -1072,7 +1072,8 @@ def ours(args, rank: int, world: int) -> None:
             "config": headline_config(args, world),
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1),
                          "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": round(frac, 4),
-                         "traffic": traffic, "kernel": "stockham_pass",
+                         "traffic": traffic,
+                         "kernel": "short_lines, stockham_pass, stockham_staged (by length)",
                          "alg_bytes_per_launch": alg_bytes,
                          "peak_source": peaks["source"] + " (MEASURED_PEAKS.json hbm_gbs)"},
             "pct_hbm_roofline": round(100 * frac, 2),
@@ -1085,7 +1086,59 @@ def ours(args, rank: int, world: int) -> None:
         }
         if configs is not None:
             line["configs"] = configs
-        print(json.dumps(line))
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(brief_line(line)))
+
+
+# What the printed line keeps of a configuration's record: key, where it stands.
+BRIEF = (("error", ("error",)), ("ms", ("ms_per_step",)), ("ms", ("ms_per_frame",)),
+         ("gflops", ("gflops",)), ("frac", ("roofline", "frac")),
+         ("e2e_gflops", ("e2e", "value")), ("p50_ms", ("latency_ms", "p50")),
+         ("p99_ms", ("latency_ms", "p99")), ("gbs", ("achieved_alg_gbs",)),
+         ("all_served", ("all_offered_served",)),
+         ("device_us", ("from_c", "calls", "fft_execute", "device_us")),
+         ("round_trip_us", ("from_c", "calls", "fft_execute", "round_trip_us")),
+         ("queue_round_trip_us", ("from_c", "fft_queue", "round_trip_us")))
+
+
+def brief_line(line: dict) -> dict:
+    """The line that is printed: every key of the headline, two numbers per size and a
+    few per configuration, below 3000 characters (a reader that keeps only the end of
+    the output still finds it whole; with every item it was 30000).  The whole record
+    goes to --detail."""
+    def num(v):
+        return round(v, 4 if abs(v) < 100 else 1) if isinstance(v, float) else v
+
+    out = {k: v for k, v in line.items() if k not in ("autotune_model", "per_size", "configs", "e2e")}
+    if line.get("e2e"):
+        out["e2e"] = {k: v for k, v in line["e2e"].items() if k != "host_numa"}
+    else:
+        out["e2e"] = line.get("e2e")
+    out["ms_and_frac_per_size"] = {k: [v["ms"], v["frac"]] for k, v in line.get("per_size", {}).items()}
+    if "configs" in line:
+        out["configs"] = {}
+        for name, rec in line["configs"].items():
+            short = {}
+            if isinstance(rec, str):
+                short = rec
+            else:
+                for key, path in BRIEF:
+                    v = rec
+                    for p in path:
+                        v = v.get(p) if isinstance(v, dict) else None
+                    if v is not None:
+                        short[key] = v[:80] if isinstance(v, str) else num(v)
+                speed = [i["speedup_vs_cufft"] for i in (rec.get("per_item") or {}).values()
+                         if isinstance(i, dict) and "speedup_vs_cufft" in i]
+                if speed:
+                    short["speedup_vs_cufft_geomean"] = round(
+                        math.exp(sum(map(math.log, speed)) / len(speed)), 3)
+                if (rec.get("clocks") or {}).get("reasons"):
+                    short["clock_reasons"] = rec["clocks"]["reasons"]
+            out["configs"][name] = short
+    return out
 
 
 SECTION_KEYS = {"small": "cfg1_small_call", "multipass": "cfg3_multipass", "sar": "cfg3_sar_frame",
@@ -1169,6 +1222,9 @@ def main() -> None:
                     help="sweep workload: comma-separated per-configuration sections timed after "
                          "the headline and reported under 'configs' (small, multipass, sar, tc, "
                          "serve, sar_compress), or 'none'")
+    ap.add_argument("--detail", default="",
+                    help="sweep workload: also write the whole record (every item of every "
+                         "configuration, the autotuner's model) to this JSON file")
     ap.add_argument("--serve-tc-max-log", type=int, default=22,
                     help="serving: largest log2 N of the tensor-core jobs (14: single-pass only)")
     ap.add_argument("--serve-jobs", type=int, default=4000,
