@@ -155,3 +155,30 @@ def test_joined_frames(gb, oracle, shape, batch, direction):
 def test_frames_not_joined(gb, shape, batch):
     with gb.Plan(shape, batch) as p:
         assert p.describe()["joined"] == 0 and p.launch_count == 2
+
+
+@pytest.mark.parametrize("logn", [15, 18, 20])
+def test_joined_sub_batches(gb, oracle, logn):
+    """A batch above 2^28 elements: the last sub-batch is a few transforms through
+    the ring and the counters that the whole one before left, and the same from a graph."""
+    n, chunk = 2 ** logn, 2 ** (28 - logn)
+    batch = chunk + 3
+    g = torch.Generator(device="cuda")
+    g.manual_seed(logn)
+    x = torch.view_as_complex(torch.rand((batch, n, 2), generator=g, device="cuda").mul_(2).sub_(1))
+    s = torch.cuda.current_stream().cuda_stream
+    idx = np.array([0, chunk - 1, chunk, batch - 1])
+    with gb.Plan(n, batch) as p:
+        d = p.describe()
+        assert (d["joined"], d["chunk_batch"]) == (1, chunk)
+        y = p.execute(x)
+        gb.fft_plan_sync_status(p.handle, s)
+        rows = x[torch.from_numpy(idx).cuda()]
+        _check(oracle, y, np.broadcast_to(rows[0].cpu().numpy(), (1, n)), np.array([0]), -1, logn)
+        with gb.Plan(n, len(idx)) as q:  # apart
+            assert torch.equal(q.execute(rows), y[torch.from_numpy(idx).cuda()])
+        z = torch.empty_like(x)
+        p.execute_graph(x, z)
+        p.execute(x, x)
+        gb.fft_plan_sync_status(p.handle, s)
+        assert torch.equal(z, y) and torch.equal(x, y)

@@ -70,3 +70,27 @@ def test_columns(gb, oracle, logn, batch, precision):
         gb.fft_execute(p.handle, x.data_ptr(), x.data_ptr(), s)
         gb.fft_plan_sync_status(p.handle, s)
         assert torch.equal(x.view(bits), y.view(bits))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("logn,batch", [(15, 83), (16, 5), (17, 3), (18, 11), (19, 1), (20, 5)])
+@pytest.mark.parametrize("precision", [1, 2, 3, 4])
+def test_six_steps(gb, oracle, logn, batch, precision):
+    """The six-step form of the same lengths (the generic option) against the oracle;
+    FP16 and BF16 with complex64 data keep its bits on column tiles."""
+    torch = pytest.importorskip("torch")
+    n, direction = 2 ** logn, 1 if batch % 2 else -1
+    x_np = synth.uniform(340 + logn, batch, n)
+    x = torch.from_numpy(x_np).cuda()
+    if precision == 4:
+        h = torch.view_as_real(x).half().contiguous()
+        x, x_np = torch.view_as_complex(h), torch.view_as_complex(h.float()).cpu().numpy()
+    with gb.Plan(n, batch, direction, precision, generic=1) as p, gb.Plan(n, batch, direction, precision) as q:
+        assert p.describe()["tc_columns"] == 0 and q.describe()["tc_columns"] == 1
+        y, z = p.execute(x), q.execute(x)
+        torch.cuda.synchronize()
+    if precision <= 2:
+        assert torch.equal(y.view(torch.int64), z.view(torch.int64))
+    ref = oracle.fft_select(x_np, np.array([0, batch - 1]), direction)
+    v = torch.view_as_real(y).float().cpu().numpy()[[0, batch - 1]]
+    assert np.max(oracle.rel_l2(v[..., 0] + 1j * v[..., 1], ref)) <= TOL[precision](n)
