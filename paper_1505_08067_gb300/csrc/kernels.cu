@@ -279,10 +279,9 @@ cudaError_t launch_grouped(int R, const PassDesc& d0, const GroupTable& gt, int 
                            size_t smem, cudaStream_t st) {
   if (gt.n < 1 || gt.n > kMaxGroup) return cudaErrorInvalidValue;
   const void* f = nullptr;
-  switch (R) {
+  switch (R) {  // 2^1, 2^2, and 2^11 .. 2^14 points; the others: launch_grouped_lines
     case 2: f = (const void*)stockham_grouped<2>; break;
     case 4: f = (const void*)stockham_grouped<4>; break;
-    case 8: f = (const void*)stockham_grouped<8>; break;
     case 16: f = (const void*)stockham_grouped<16>; break;
     default: return cudaErrorInvalidValue;
   }

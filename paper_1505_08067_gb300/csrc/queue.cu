@@ -208,8 +208,10 @@ queue_worker(const __grid_constant__ PassDesc d0, const __grid_constant__ QueueA
   }
 }
 
+// The worker of 2, 4, 2048 and 4096 points.
 const void* worker_fn(int R, const PassDesc& d) {
 #define GB_TRY(LOGL, SCHED, NST, RR, G, LM, SM, CONTIG, EPI)                                     \
+  if constexpr (LOGL == 11 || LOGL == 12)                                                        \
   if (shape_matches(d, R, MAP_ROWS, MAP_ROWS, LOGL, SCHED, NST, RR, G, LM, SM, CONTIG, EPI))     \
     return (const void*)queue_worker<RegisterTile<RR, CtTraits<LOGL, SCHED, NST, RR, G, CONTIG, EPI>>>;
   GB_SHAPES_CONTIG(GB_TRY)
@@ -217,7 +219,6 @@ const void* worker_fn(int R, const PassDesc& d) {
   switch (R) {
     case 2: return (const void*)queue_worker<RegisterTile<2, RtTraits>>;
     case 4: return (const void*)queue_worker<RegisterTile<4, RtTraits>>;
-    case 8: return (const void*)queue_worker<RegisterTile<8, RtTraits>>;
     case 16: return (const void*)queue_worker<RegisterTile<16, RtTraits>>;
     default: return nullptr;
   }
