@@ -10,9 +10,10 @@
 // powers of a single root, and costs as many multiplies.
 //
 // Four-step transforms.  N = N1 N2, x[n1 N2 + n2], X[k2 N1 + k1]:
-//   pass 1  a tile holds G1 = 8192 / N1 adjacent columns n2; the output is
+//   pass 1  a tile of 2^TL elements (4096 .. 16384) holds G1 = 2^TL / N1 adjacent
+//           columns n2; the output is
 //           multiplied by w_N^{n2 k1} and written to the workspace in blocks of
-//           G2 = 8192 / N2 values k1: element (n2, k1) at
+//           G2 = 2^TL / N2 values k1: element (n2, k1) at
 //             (k1 / G2) (N2 G2) + n2 G2 + (k1 mod G2);
 //   pass 2  a tile holds G2 adjacent k1 -- one contiguous block of the
 //           workspace -- and writes G2 adjacent outputs per row k2.

@@ -7,9 +7,9 @@
 // (2^18 x 256: 379 against 446 us, 2^20 x 64: 358 against 368 us): two
 // shared-memory exchanges, in the longer passes in half-buffer rounds with
 // eight barriers per tile.  Here a tile crosses shared memory once, and the
-// order of the tiles keeps the intermediate in L2 (ncu, 2^18 x 64: DRAM reads
-// equal to the input, DRAM writes 1.3 times the output, where two launches
-// move twice both).
+// order of the tiles keeps the intermediate in L2 (ncu, 2^18 x 64: 278 MB read and
+// written in DRAM, input and output being 268 MB, where two launches move twice
+// that).
 //
 // What bounds this kernel: the first pass (2^26 elements, 512 points: 161 us
 // alone, the second 135), by latency -- issue 38% busy, FMA pipe 36%, DRAM 47%.
@@ -24,7 +24,8 @@
 // four 128-thread blocks, 242 / 245 us).
 //
 // Smaller batches run the same passes in a launch each (apart_first,
-// apart_second; join_apart says where the line lies).
+// apart_second; join_apart says where the line lies), and so do server jobs and
+// fft_execute_noalloc at every size: that form needs no counters.
 // Measured, 2^26 elements, before (two launches) and now: 2^15 349 -> 242 us,
 // 2^16 363 -> 245, 2^17 396 -> 275, 2^18 446 -> 289, 2^19 421 -> 302,
 // 2^20 368 -> 330.  2^21 and 2^22, whose 2048-point passes need three stages and

@@ -1,7 +1,8 @@
 // Batches of short contiguous transforms (2^3 .. 2^10 points): a tile of 4096
 // elements per 128-thread block as a row pass of fft_join.h, 32 elements and one
 // exchange per thread; and the column passes of frames of 2^3 .. 2^11 rows in the
-// same way.
+// same way.  Server jobs run the same tiles alone (short_lines) or coalesced
+// (grouped_lines), and the work queue's worker does (queue.cu).
 //
 // Lengths below 256 ran the run-time-parameter kernel, bound by its address
 // arithmetic and, at 16 points (one transform per thread), by loads that touch
