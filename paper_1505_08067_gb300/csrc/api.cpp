@@ -524,7 +524,12 @@ fft_status_t fft_plan_sync_status(fft_plan_t plan, void* stream) {
   if (flag) {
     // a four-step plan's counters too (a frame plan's may be at work on a stream)
     const bool ctr = plan->spec.joined && !plan->joined[0].frames;
-    cudaMemset(plan->status, 0, ctr ? status_bytes(plan->spec) : sizeof flag);
+    // waited for: the plan's next execution may be on any stream, and a memset of
+    // device memory returns before it is done
+    e = cudaMemsetAsync(plan->status, 0, ctr ? status_bytes(plan->spec) : sizeof flag,
+                        static_cast<cudaStream_t>(stream));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "status word");
     if (flag & kStatusGaveUp)
       return fail(FFT_ERR_TIMEOUT, "a kernel gave up a bounded wait (its copy into shared memory, "
                                    "or the tiles of a joined launch); the output is incomplete");

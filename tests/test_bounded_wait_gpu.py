@@ -88,3 +88,22 @@ def test_joined_counters_not_its_own(gb, shape, batch):
             p.execute(x, y)
             gb.fft_plan_sync_status(p.handle, s)
             assert torch.equal(y, want)
+
+
+@pytest.mark.parametrize("shape,batch", [((2 ** 15,), 391), ((2 ** 18,), 49)])
+def test_cleared_counters_before_the_next_execution(gb, shape, batch):
+    """fft_plan_sync_status returns with the counters cleared: an execution that follows
+    at once, on a stream that waits for no other, finds them so."""
+    p, x, want = _joined(gb, shape, batch)
+    outs = [torch.full_like(x, float("nan")) for _ in range(8)]
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with p:
+        for i in range(40):
+            y = outs[i % 8]
+            gb.fft_join_selftest(p.handle, x.data_ptr(), y.data_ptr(), 2 ** 31, 64, a.cuda_stream)
+            with pytest.raises(gb.GbfftError):
+                gb.fft_plan_sync_status(p.handle, a.cuda_stream)
+            gb.fft_execute(p.handle, x.data_ptr(), y.data_ptr(), b.cuda_stream)
+            gb.fft_plan_sync_status(p.handle, b.cuda_stream)
+        assert all(torch.equal(y, want) for y in outs)
