@@ -532,7 +532,7 @@ GBFFT_API fft_status_t fft_wait_selftest(uint32_t polls, int* gave_up);
  * execution is right again.  With more than the launch has, no tile is
  * computed and none is waited for, as after executions that overlapped:
  * FFT_ERR_CUDA.  FFT_ERR_INVALID_ARG where the plan does not describe
- * itself as joined or would not be joined on `stream`. */
+ * itself as joined or would not be joined on `stream`, and in a capture. */
 GBFFT_API fft_status_t fft_join_selftest(fft_plan_t plan, const void* in, void* out,
                                          uint32_t handed_out, uint32_t polls, void* stream);
 

@@ -549,6 +549,12 @@ fft_status_t fft_join_selftest(fft_plan_t plan, const void* in, void* out, uint3
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
   if (dev != plan->device) return fail(FFT_ERR_BAD_PLAN, "plan/device mismatch");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // not into a graph: its copy node would read handed_out when that is long gone
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  e = cudaStreamIsCapturing(st, &cap);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
+  if (cap != cudaStreamCaptureStatusNone)
+    return fail(FFT_ERR_INVALID_ARG, "fft_join_selftest: the stream is being captured");
   const JoinedLaunch* own = joined_for(plan, st);
   if (!own || !own->fn || own->second)
     return fail(FFT_ERR_INVALID_ARG, "fft_join_selftest: the plan is not joined on this stream");

@@ -107,3 +107,21 @@ def test_cleared_counters_before_the_next_execution(gb, shape, batch):
             gb.fft_execute(p.handle, x.data_ptr(), y.data_ptr(), b.cuda_stream)
             gb.fft_plan_sync_status(p.handle, b.cuda_stream)
         assert all(torch.equal(y, want) for y in outs)
+
+
+def test_joined_selftest_is_not_captured(gb):
+    """Refused in a capture, which stays valid."""
+    p, x, want = _joined(gb, (2 ** 15,), 391)
+    y = torch.empty_like(x)
+    torch.cuda.synchronize()
+    with p:
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            s = torch.cuda.current_stream().cuda_stream
+            with pytest.raises(gb.GbfftError) as e:
+                gb.fft_join_selftest(p.handle, x.data_ptr(), y.data_ptr(), 1, 64, s)
+            gb.fft_execute(p.handle, x.data_ptr(), y.data_ptr(), s)
+        assert e.value.status == gb.FFT_ERR_INVALID_ARG
+        g.replay()
+        gb.fft_plan_sync_status(p.handle, torch.cuda.current_stream().cuda_stream)
+        assert torch.equal(y, want)
