@@ -104,3 +104,56 @@ def test_queue(gb, logn, direction):
         q.wait(q.submit_ptr(xs[-1].data_ptr(), xs[-1].data_ptr(), batches[-1]), 10.0)
     torch.cuda.synchronize()
     assert torch.equal(_bits(xs[-1]), _bits(want[-1]))
+
+
+@pytest.mark.parametrize("shape,batch", [((8, 8), 700), ((16, 1024), 3), ((64, 64), 33), ((128, 2048), 2),
+                                         ((512, 256), 101), ((1024, 512), 25), ((2048, 16), 5), ((4096, 64), 3),
+                                         ((32, 16384), 2), ((1, 64), 9), ((64, 1), 9)])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_frames(gb, shape, batch, direction):
+    """Frames, joined or not: a graph, host buffers, server jobs of the whole batch and of
+    parts of it, and another stream beyond those that have counters."""
+    torch.manual_seed(batch)
+    x = torch.randn((batch,) + shape, dtype=torch.complex64, device="cuda")
+    host = x.cpu().pin_memory()
+    back, tmp = torch.empty_like(host).pin_memory(), torch.empty_like(x)
+    with gb.Plan(shape, batch, direction) as p:
+        want = p.execute(x)
+        torch.cuda.synchronize()
+        outs = [p.execute_graph(x, torch.empty_like(x))]
+        streams = [torch.cuda.Stream() for _ in range(5)]
+        outs += [p.execute(x, torch.empty_like(x), stream=s) for s in streams]
+        torch.cuda.synchronize()
+        p.execute_host(host, back, tmp, tmp)
+        torch.cuda.synchronize()
+    cut = batch // 2
+    whole, parts = torch.empty_like(x), torch.empty_like(x)
+    torch.cuda.synchronize()
+    srv = gb.fft_server_create(memory_budget_bytes=4 << 30)
+    try:
+        jobs = [(x, whole, batch), (x[:cut], parts[:cut], cut), (x[cut:], parts[cut:], batch - cut)]
+        tickets = [gb.fft_server_submit(srv, shape, b, direction, 0, i.data_ptr(), o.data_ptr())
+                   for i, o, b in jobs]
+        assert all(gb.fft_server_wait(srv, k, 60.0)["status"] == 0 for k in tickets)
+    finally:
+        gb.fft_server_destroy(srv)
+    for y in outs + [back.cuda(), whole, parts]:
+        assert torch.equal(_bits(y), _bits(want))
+
+
+@pytest.mark.parametrize("n,batch", [(2, 2200001), (64, 70001), (1024, 5001), (2048, 2101), (4096, 1051), (16384, 301),
+                                     (2 ** 15, 391), (2 ** 18, 49), (2 ** 20, 13), (2 ** 21, 7)])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_graph_and_host(gb, n, batch, direction):
+    """Graphs, and host buffers in chunks that are a launch each."""
+    torch.manual_seed(batch)
+    x = torch.randn((batch, n), dtype=torch.complex64, device="cuda")
+    host = x.cpu().pin_memory()
+    back, tmp = torch.empty_like(host).pin_memory(), torch.empty_like(x)
+    with gb.Plan(n, batch, direction) as p:
+        want = p.execute(x)
+        torch.cuda.synchronize()
+        y = p.execute_graph(x, torch.empty_like(x))
+        p.execute_host(host, back, tmp, tmp)
+        torch.cuda.synchronize()
+    assert torch.equal(_bits(y), _bits(want)) and torch.equal(back, want.cpu())
